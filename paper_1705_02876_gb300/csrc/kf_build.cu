@@ -129,32 +129,36 @@ struct BuildParams {
 constexpr int kMaxN = 8;
 constexpr uint32_t kNoKey = 0xffffffffu;
 
-// Chi2 increment of a hit (m, packed V) against the predicted candidate, in
-// the layer's local frame (n, t, z) with the radial row of C projected out
-// (the same arithmetic as the update): ctt = C_tt, ctz = C_tz, czz = C_zz.
-// f3 receives the residual in that frame divided by the square roots of S's
-// diagonal (the proposal's first three inputs).
+// Chi2 increment of a hit (m, packed V) against the predicted candidate, as
+// the update computes it: S over (n, t, z) factorised in that order, from the
+// predicted position x, its frame (nx, ny) and ctt, ctz, czz of the local
+// covariance.  f3 receives the residual in that frame divided by the square
+// roots of S's diagonal (the proposal's first three inputs).
 __device__ __forceinline__ bool hit_eval(const float x[3], float nx, float ny, float ctt, float ctz, float czz,
                                          const float m[3], const float v[6], float *out, float f3[3])
 {
-    const float vnn = fmaf(nx * nx, v[0], fmaf(2.0f * nx * ny, v[1], ny * ny * v[2]));
-    const float vnt = fmaf(nx * ny, v[2] - v[0], (nx * nx - ny * ny) * v[1]);
-    const float vtt = fmaf(ny * ny, v[0], fmaf(-2.0f * nx * ny, v[1], nx * nx * v[2]));
+    const float nn = nx * nx, tt = ny * ny, nt = nx * ny;
+    const float vnn = fmaf(nn, v[0], fmaf(2.0f * nt, v[1], tt * v[2]));
+    const float vnt = fmaf(nt, v[2] - v[0], fmaf(nx, nx, -tt) * v[1]);
+    const float vtt = fmaf(tt, v[0], fmaf(-2.0f * nt, v[1], nn * v[2]));
     const float vnz = fmaf(nx, v[3], ny * v[4]), vtz = fmaf(nx, v[4], -ny * v[3]);
-    const float a = vnn, b = vnt, cc = ctt + vtt, d = vnz, e = ctz + vtz, f = czz + v[5];
-    const float i00 = cc * f - e * e, i10 = d * e - b * f, i11 = a * f - d * d;
-    const float i20 = b * e - cc * d, i21 = b * d - a * e, i22 = a * cc - b * b;
-    const float det = fmaf(a, i00, fmaf(b, i10, d * i20));
+    const float stt = ctt + vtt, szz = czz + v[5];
     const float d0 = m[0] - x[0], d1 = m[1] - x[1];
     const float rn = fmaf(nx, d0, ny * d1), rt = fmaf(nx, d1, -ny * d0), rz = m[2] - x[2];
-    f3[0] = rn * rsqrtf(fmaxf(a, 1e-30f));
-    f3[1] = rt * rsqrtf(fmaxf(cc, 1e-30f));
-    f3[2] = rz * rsqrtf(fmaxf(f, 1e-30f));
-    if (!(a > 0.0f && i22 > 0.0f && det > 0.0f)) return false;
-    const float q0 = fmaf(i00, rn, fmaf(i10, rt, i20 * rz));
-    const float q1 = fmaf(i10, rn, fmaf(i11, rt, i21 * rz));
-    const float q2 = fmaf(i20, rn, fmaf(i21, rt, i22 * rz));
-    *out = __fdividef(fmaf(rn, q0, fmaf(rt, q1, rz * q2)), det);
+    f3[0] = rn * rsqrtf(fmaxf(vnn, 1e-30f));
+    f3[1] = rt * rsqrtf(fmaxf(stt, 1e-30f));
+    f3[2] = rz * rsqrtf(fmaxf(szz, 1e-30f));
+    const float ia = __fdividef(1.0f, vnn);
+    const float vt = vnt * ia, vz = vnz * ia;
+    const float dt = fmaf(-vnt, vt, stt);
+    const float it = __fdividef(1.0f, dt);
+    const float e = fmaf(-vnt, vz, ctz + vtz);
+    const float l = e * it;
+    const float dz = fmaf(-l, e, fmaf(-vnz, vz, szz));
+    if (!(vnn > 0.0f && dt > 0.0f && dz > 0.0f && dz < INFINITY)) return false;
+    const float r1 = fmaf(-vt, rn, rt);
+    const float r2 = fmaf(-l, r1, fmaf(-vz, rn, rz));
+    *out = fmaf(rn * rn, ia, fmaf(r1 * r1, it, __fdividef(r2 * r2, dz)));
     return true;
 }
 
@@ -208,17 +212,18 @@ __host__ __device__ constexpr size_t build_smem_base(int L) { return ((size_t)(L
 
 // Proposal mode: where a lane parks, in shared memory, what walking the wide
 // windows needs ([kWcWords][128] words, one column per thread; the candidate
-// state x, C goes to the thread's update slot, idle at that point).  While
+// itself goes to the thread's update slot, idle at that point).  While
 // the warp walks the wide windows the candidate state is out of the
 // registers, so that the scoring's fragments do not spill it.
 constexpr int kWcHb = 0;                        // [kMaxN] collected (or ranked) hits
-constexpr int kWcNx = 8, kWcNy = 9, kWcCtt = 10, kWcCtz = 11, kWcCzz = 12;
-constexpr int kWcSegLo = 13;                    // 2 words
-constexpr int kWcBo = 15;                       // 2 words
-constexpr int kWcPhic = 17, kWcDphi = 18, kWcZ = 19, kWcDz = 20;
-constexpr int kWcIz0 = 21, kWcIz1 = 22, kWcIp0 = 23, kWcNphi = 24;
-constexpr int kWcNhits = 25, kWcQkb = 26;      // the candidate's hit count, its charge x field term
-constexpr int kWcWords = 27;
+constexpr int kWcSegLo = 8;                     // 2 words
+constexpr int kWcBo = 10;                       // 2 words
+constexpr int kWcPhic = 12, kWcDphi = 13, kWcZ = 14, kWcDz = 15;
+constexpr int kWcIz0 = 16, kWcIz1 = 17, kWcIp0 = 18, kWcNphi = 19;
+constexpr int kWcNhits = 20, kWcQkb = 21;      // the candidate's hit count, its charge x field term
+constexpr int kWcWords = 22;
+// where the update slot holds the parked candidate: position and momentum
+// from kSlotX, the local covariance from kSlotC, the two frames from kSlotFrame
 constexpr size_t kBuildSmemMlp = (size_t)(kWcWords * 128 + 4 * 32 * kStageLd) * sizeof(float);
 
 // What scan_wide reads besides the parked columns.
@@ -230,6 +235,18 @@ struct WideArgs {
     const __nv_bfloat16 *W1, *W2;
     const float *w32;
 };
+
+// The diagonal of the Cartesian covariance of local coordinates.
+__device__ __forceinline__ void cartesian_variances(float f0, float f1, float nx, float ny, float ctt, float czz,
+                                                    float cuu, float cvu, float cvv, float cpp, float var[6])
+{
+    var[0] = ny * ny * ctt;
+    var[1] = nx * nx * ctt;
+    var[2] = czz;
+    var[3] = fmaf(f0 * f0, cuu, fmaf(-2.0f * f0 * f1, cvu, f1 * f1 * cvv));
+    var[4] = fmaf(f1 * f1, cuu, fmaf(2.0f * f0 * f1, cvu, f0 * f0 * cvv));
+    var[5] = cpp;
+}
 
 // The windows of one warp wider than topk, walked by the whole warp
 // (warp-collective: every lane calls it, converged; every lane has parked its
@@ -275,10 +292,15 @@ __device__ __forceinline__ void scan_wide(const WideArgs p, bool wide, const flo
     // the owner's candidate inputs, staged once in this lane's row
     {
         float *row = xs + lane * kStageLd;
+        const auto C = [&](int i, int j) { return os[(kSlotC + pk(i, j)) * 128]; };
+        const float f0 = os[kSlotFrame * 128], f1 = os[(kSlotFrame + 1) * 128];
+        const float nx = os[(kSlotFrame + 2) * 128], ny = os[(kSlotFrame + 3) * 128];
+        float var[6];
+        cartesian_variances(f0, f1, nx, ny, C(0, 0), C(1, 1), C(2, 2), C(3, 2), C(3, 3), C(4, 4), var);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) row[3 + i] = log10f(fmaxf(os[(kSlotC + pk(i, i)) * 128], 1e-30f));
+        for (int i = 0; i < 6; ++i) row[3 + i] = log10f(fmaxf(var[i], 1e-30f));
         const float px3 = os[(kSlotX + 3) * 128], px4 = os[(kSlotX + 4) * 128];
-        row[9] = copysignf(rsqrtf(px3 * px3 + px4 * px4), col(kWcQkb));
+        row[9] = copysignf(rsqrtf(fmaf(px3, px3, px4 * px4)), col(kWcQkb));
         row[10] = __fdiv_rn((float)p.l, (float)p.L);  // correctly rounded, whatever the division flags
         row[11] = (float)(p.l - icol(kWcNhits));
     }
@@ -356,7 +378,8 @@ __device__ __forceinline__ void scan_wide(const WideArgs p, bool wide, const flo
 #pragma unroll
             for (int i = 0; i < 6; ++i) v[i] = p.hit_cov[i * p.H + hg];
             const float xp[3] = {os[(kSlotX + 0) * 128], os[(kSlotX + 1) * 128], os[(kSlotX + 2) * 128]};
-            hit_eval(xp, col(kWcNx), col(kWcNy), col(kWcCtt), col(kWcCtz), col(kWcCzz), m, v, &dc, f3);
+            hit_eval(xp, os[(kSlotFrame + 2) * 128], os[(kSlotFrame + 3) * 128], os[kSlotC * 128], os[(kSlotC + 1) * 128],
+                     os[(kSlotC + 2) * 128], m, v, &dc, f3);
         }
         __syncwarp();  // the previous round's rows are read
 #pragma unroll
@@ -435,7 +458,8 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
     const int N = p.N;
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << gbase);
 
-    float x[6], c[21];
+    Local t{};  // the candidate's estimate on the last layer it reached, and its covariance
+    float c[15], pn = 1.0f;
     float chi2 = 0.0f;
     int nhits = 0;
     bool stopped = false;
@@ -446,36 +470,33 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
     const bool ev_ok = ev_in >= 0 && ev_in < p.n_events;  // a seed of an unknown event builds nothing
     const int ev = ev_ok ? ev_in : 0;
     const float qkb = seed_ok ? (float)p.seed_charge[s] * p.g.qk : 0.0f;
-    if (seed_ok && ev_ok) {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) x[i] = p.seed_state[i * p.S + s];
+    for (int i = 0; i < 15; ++i) c[i] = 0.0f;
+    if (!(seed_ok && ev_ok)) nc = 0;
+    if (slot < nc) {  // the seed, taken to the first layer by the group's first lane
+        float x6[6], c6[21];
 #pragma unroll
-        for (int i = 0; i < 21; ++i) c[i] = p.seed_cov[i * p.S + s];
-    } else {
+        for (int i = 0; i < 6; ++i) x6[i] = p.seed_state[i * p.S + s];
 #pragma unroll
-        for (int i = 0; i < 6; ++i) x[i] = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 21; ++i) c[i] = 0.0f;
-        nc = 0;
+        for (int i = 0; i < 21; ++i) c6[i] = p.seed_cov[i * p.S + s];
+        flags = enter_local(x6, c6, qkb, p.g.r[0], p.g.inv_r[0], p.g.z_half, t, c, pn);
+        stopped = flags != 0u;
     }
+    const bool at_seed = stopped;  // no layer reached: the seed's one candidate, all holes, stays the seed
     const int nbins = p.bg.n_phi * p.bg.n_z;
     for (int l = 0; l < L; ++l) {
         const bool valid = slot < nc;
         bool reached = false;
         if (valid && !stopped) {
-            float xn[6], sd;
-            Jac J;
-            if (!propagate(x, qkb, p.g.r[l], xn, sd, &J)) {
-                stopped = true;
-                flags |= KF_FLAG_UNREACHABLE;
-            } else if (fabsf(xn[2]) > p.g.z_half) {
-                stopped = true;
-                flags |= KF_FLAG_LEFT_BARREL;
-            } else {
-                transport(J, c);
-                add_scattering(xn, p.g.inv_r[l], p.g.xx0[l], c);
-#pragma unroll
-                for (int i = 0; i < 6; ++i) x[i] = xn[i];
+            if (l > 0) {
+                LocalJac J;
+                const uint32_t stop = step_local(t, qkb, p.g.r[l], p.g.inv_r[l], p.g.z_half, J, pn);
+                flags |= stop;
+                stopped = stop != 0u;
+                if (!stopped) transport_local(J, c);
+            }
+            if (!stopped) {
+                scatter_local(t, noise_local(t, pn, p.g.xx0[l]), c);
                 reached = true;
             }
         }
@@ -509,25 +530,18 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
         const int64_t seg = (int64_t)ev * (L + 1) + l;
         int64_t seg_lo = seed_ok ? p.ev_off[seg] : 0;
         Window win{};
-        float nx = 0.0f, ny = 0.0f, ctt = 0.0f, ctz = 0.0f, czz = 0.0f;
         if (reached) {
-            const float ir = rsqrtf(x[0] * x[0] + x[1] * x[1]);
-            nx = x[0] * ir;
-            ny = x[1] * ir;
-            ctt = fmaf(ny * ny, c[pk(0, 0)], fmaf(-2.0f * nx * ny, c[pk(1, 0)], nx * nx * c[pk(1, 1)]));
-            ctz = fmaf(nx, c[pk(2, 1)], -ny * c[pk(2, 0)]);
-            czz = c[pk(2, 2)];
-            win.dphi = fminf(p.nsigma * sqrtf(ctt + p.sig_rphi2) * p.g.inv_r[l], p.max_dphi);
-            win.dz = fminf(p.nsigma * sqrtf(czz + p.sig_z2), p.max_dz);
-            win.phic = atan2f(x[1], x[0]);
-            win.z = x[2];
+            win.dphi = fminf(p.nsigma * sqrtf(c[pk(0, 0)] + p.sig_rphi2) * p.g.inv_r[l], p.max_dphi);
+            win.dz = fminf(p.nsigma * sqrtf(c[pk(1, 1)] + p.sig_z2), p.max_dz);
+            win.phic = atan2f(t.y, t.x);
+            win.z = t.z;
             win.bo = p.bin_off + (((int64_t)ev * L + l) * (nbins + 1));
             win.seg_lo = seg_lo;
             // bin ranges widened by a rounding margin: a hit that passes the
             // exact window test always lies in a scanned bin
-            const float zm = 1e-4f * (1.0f + fabsf(x[2])), pm = 1e-5f;
-            win.iz0 = z_bin(x[2] - win.dz - zm, p.bg);
-            win.iz1 = z_bin(x[2] + win.dz + zm, p.bg);
+            const float zm = 1e-4f * (1.0f + fabsf(t.z)), pm = 1e-5f;
+            win.iz0 = z_bin(t.z - win.dz - zm, p.bg);
+            win.iz1 = z_bin(t.z + win.dz + zm, p.bg);
             int ip0, ip1;
             if (win.dphi >= kPi - pm) {
                 ip0 = 0;
@@ -546,11 +560,18 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
 #pragma unroll
             for (int i = 0; i < 6; ++i) v[i] = p.hit_cov[i * p.H + hg];
         };
+        auto eval = [&](const float m[3], const float v[6], float *dc, float f3[3]) {
+            const float xp[3] = {t.x, t.y, t.z};
+            return hit_eval(xp, t.nx, t.ny, c[pk(0, 0)], c[pk(1, 0)], c[pk(1, 1)], m, v, dc, f3);
+        };
         // inputs of the proposal shared by every hit of this candidate
         auto cand_features = [&](float f[kMlpIn]) {
+            float var[6];
+            cartesian_variances(t.f0, t.f1, t.nx, t.ny, c[pk(0, 0)], c[pk(1, 1)], c[pk(2, 2)], c[pk(3, 2)], c[pk(3, 3)],
+                                c[pk(4, 4)], var);
 #pragma unroll
-            for (int i = 0; i < 6; ++i) f[3 + i] = log10f(fmaxf(c[pk(i, i)], 1e-30f));
-            f[9] = copysignf(rsqrtf(x[3] * x[3] + x[4] * x[4]), qkb);
+            for (int i = 0; i < 6; ++i) f[3 + i] = log10f(fmaxf(var[i], 1e-30f));
+            f[9] = copysignf(rsqrtf(fmaf(t.q1, t.q1, t.q2 * t.q2)), qkb);
             f[10] = __fdiv_rn((float)l, (float)L);  // correctly rounded, whatever the division flags
             f[11] = (float)(l - nhits);
         };
@@ -605,17 +626,20 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
                 // lane's state, walk the warp's wide windows, take it back
                 volatile float *vs = slots + threadIdx.x;
                 volatile float *vw = wc + threadIdx.x;
+                vs[kSlotX * 128] = t.x;
+                vs[(kSlotX + 1) * 128] = t.y;
+                vs[(kSlotX + 2) * 128] = t.z;
+                vs[(kSlotX + 3) * 128] = t.q1;
+                vs[(kSlotX + 4) * 128] = t.q2;
+                vs[(kSlotX + 5) * 128] = t.pz;
 #pragma unroll
-                for (int i = 0; i < 6; ++i) vs[(kSlotX + i) * 128] = x[i];
-#pragma unroll
-                for (int i = 0; i < 21; ++i) vs[(kSlotC + i) * 128] = c[i];
+                for (int i = 0; i < 15; ++i) vs[(kSlotC + i) * 128] = c[i];
+                vs[kSlotFrame * 128] = t.f0;
+                vs[(kSlotFrame + 1) * 128] = t.f1;
+                vs[(kSlotFrame + 2) * 128] = t.nx;
+                vs[(kSlotFrame + 3) * 128] = t.ny;
 #pragma unroll
                 for (int k = 0; k < kMaxN; ++k) vw[(kWcHb + k) * 128] = __int_as_float((int)hb[k]);
-                vw[kWcNx * 128] = nx;
-                vw[kWcNy * 128] = ny;
-                vw[kWcCtt * 128] = ctt;
-                vw[kWcCtz * 128] = ctz;
-                vw[kWcCzz * 128] = czz;
                 vw[kWcSegLo * 128] = __int_as_float((int)(uint32_t)(unsigned long long)seg_lo);
                 vw[(kWcSegLo + 1) * 128] = __int_as_float((int)(uint32_t)((unsigned long long)seg_lo >> 32));
                 const unsigned long long bo_bits = reinterpret_cast<unsigned long long>(win.bo);
@@ -635,17 +659,14 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
                 const WideArgs wa{p.bkey,    p.hit_pos, p.hit_cov, p.H,       p.bg.n_phi,
                                   p.topk,    l,         L,         p.mlp_W1, p.mlp_W2, p.mlp_w32};
                 scan_wide(wa, wide, slots, wc, xs);
+                t = Local{vs[kSlotX * 128],           vs[(kSlotX + 1) * 128],     vs[(kSlotX + 2) * 128],
+                          vs[(kSlotX + 3) * 128],     vs[(kSlotX + 4) * 128],     vs[(kSlotX + 5) * 128],
+                          vs[kSlotFrame * 128],       vs[(kSlotFrame + 1) * 128], vs[(kSlotFrame + 2) * 128],
+                          vs[(kSlotFrame + 3) * 128]};
 #pragma unroll
-                for (int i = 0; i < 6; ++i) x[i] = vs[(kSlotX + i) * 128];
-#pragma unroll
-                for (int i = 0; i < 21; ++i) c[i] = vs[(kSlotC + i) * 128];
+                for (int i = 0; i < 15; ++i) c[i] = vs[(kSlotC + i) * 128];
 #pragma unroll
                 for (int k = 0; k < kMaxN; ++k) hb[k] = (uint32_t)__float_as_int(vw[(kWcHb + k) * 128]);
-                nx = vw[kWcNx * 128];
-                ny = vw[kWcNy * 128];
-                ctt = vw[kWcCtt * 128];
-                ctz = vw[kWcCtz * 128];
-                czz = vw[kWcCzz * 128];
                 seg_lo = (int64_t)(((unsigned long long)(uint32_t)__float_as_int(vw[(kWcSegLo + 1) * 128]) << 32) |
                                    (uint32_t)__float_as_int(vw[kWcSegLo * 128]));
             }
@@ -657,7 +678,7 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
                     if (hb[k2] == kNoKey) continue;
                     float m[3], v[6], dc, f3[3];
                     load_hit(hb[k2], m, v);
-                    if (hit_eval(x, nx, ny, ctt, ctz, czz, m, v, &dc, f3) && dc <= p.chi2_cut)
+                    if (eval(m, v, &dc, f3) && dc <= p.chi2_cut)
                         insert(dc, hb[k2], kNoKey);
                 }
             } else if (!(MODE == kModePlain && p.flag_over > 0)) {
@@ -669,7 +690,7 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
                 for (uint32_t hl = cur.next(p, win); hl != kNoKey; hl = cur.next(p, win)) {
                     float m[3], v[6], dc, f3[3];
                     load_hit(hl, m, v);
-                    if (hit_eval(x, nx, ny, ctt, ctz, czz, m, v, &dc, f3) && dc <= p.chi2_cut) insert(dc, hl, kNoKey);
+                    if (eval(m, v, &dc, f3) && dc <= p.chi2_cut) insert(dc, hl, kNoKey);
                 }
             }
         } else if (reached) {
@@ -680,7 +701,7 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
             for (uint32_t hl = cur.next(p, win); hl != kNoKey; hl = cur.next(p, win)) {
                 float m[3], v[6], dc, feat[kMlpIn];
                 load_hit(hl, m, v);
-                const bool ok = hit_eval(x, nx, ny, ctt, ctz, czz, m, v, &dc, feat);
+                const bool ok = eval(m, v, &dc, feat);
                 uint32_t row = kNoKey;
                 const unsigned long long r = atomicAdd(p.log_n, 1ull);
                 if (r < p.log_cap) {
@@ -763,19 +784,20 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
         }
         // each lane takes over child `slot` from its parent lane
         const int src = gbase + (new_parent >= 0 ? new_parent : slot);
-        float px[6], pc[21];
+        Local pt;
+        float pc[15];
+        auto from = [&](float v) { return __shfl_sync(gmask, v, src, 32); };
+        pt = Local{from(t.x),  from(t.y),  from(t.z),  from(t.q1), from(t.q2),
+                   from(t.pz), from(t.f0), from(t.f1), from(t.nx), from(t.ny)};
 #pragma unroll
-        for (int i = 0; i < 6; ++i) px[i] = __shfl_sync(gmask, x[i], src, 32);
-#pragma unroll
-        for (int i = 0; i < 21; ++i) pc[i] = __shfl_sync(gmask, c[i], src, 32);
+        for (int i = 0; i < 15; ++i) pc[i] = from(c[i]);
         const int pstop = __shfl_sync(gmask, (int)stopped, src, 32);
         const uint32_t pflags = __shfl_sync(gmask, flags, src, 32);
         nc = n_new;
         if (slot < nc) {
+            t = pt;
 #pragma unroll
-            for (int i = 0; i < 6; ++i) x[i] = px[i];
-#pragma unroll
-            for (int i = 0; i < 21; ++i) c[i] = pc[i];
+            for (int i = 0; i < 15; ++i) c[i] = pc[i];
             stopped = pstop != 0;
             flags = pflags;
             chi2 = new_chi2;
@@ -787,7 +809,7 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
                 for (int i = 0; i < 3; ++i) m[i] = p.hit_pos[i * p.H + hg];
 #pragma unroll
                 for (int i = 0; i < 6; ++i) v[i] = p.hit_cov[i * p.H + hg];
-                const int st = update(x, c, m, v, p.rt, &d, slots + threadIdx.x, 128);
+                const int st = update_local(t, c, m, v, p.rt, &d, slots + threadIdx.x, 128);
                 if (st == 1) flags |= KF_FLAG_INVERSION_FAILED;
                 if (st >= 2) flags |= KF_FLAG_FP64_PATH;
                 if (st == 3) flags |= KF_FLAG_PSD_REPAIRED;
@@ -806,10 +828,19 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
     const int64_t sj = s * N_ + slot;
     if (slot < N_) {
         const bool have = slot < nc;
+        float x6[6], c6[21];
+        if (have && at_seed) {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) p.out_state[i * p.S * N_ + sj] = have ? x[i] : 0.0f;
+            for (int i = 0; i < 6; ++i) x6[i] = p.seed_state[i * p.S + s];
 #pragma unroll
-        for (int i = 0; i < 21; ++i) p.out_cov[i * p.S * N_ + sj] = have ? c[i] : 0.0f;
+            for (int i = 0; i < 21; ++i) c6[i] = p.seed_cov[i * p.S + s];
+        } else {
+            leave_local(t, c, x6, c6);
+        }
+#pragma unroll
+        for (int i = 0; i < 6; ++i) p.out_state[i * p.S * N_ + sj] = have ? x6[i] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 21; ++i) p.out_cov[i * p.S * N_ + sj] = have ? c6[i] : 0.0f;
         p.out_chi2[sj] = have ? chi2 : 0.0f;
         p.out_nhits[sj] = (int16_t)(have ? nhits : -1);
         p.out_flags[sj] = have ? flags : 0u;

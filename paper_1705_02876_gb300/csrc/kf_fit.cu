@@ -1,5 +1,5 @@
 // Kalman-filter track fit on sm_103a: one thread per track (Section 4.2),
-// state and packed covariance in registers, structure-of-arrays inputs read
+// state and packed local covariance (kf_math.cuh) in registers, structure-of-arrays inputs read
 // coalesced (Section 4.1: element (i, j) of consecutive tracks is contiguous).
 #include <mutex>
 #include <set>
@@ -13,16 +13,6 @@ namespace kf {
 namespace {
 
 constexpr uint32_t kStop = KF_FLAG_UNREACHABLE | KF_FLAG_LEFT_BARREL | KF_FLAG_NAN_INPUT;
-
-// 0 * v is 0 for finite v and NaN otherwise
-template <int N>
-__device__ __forceinline__ bool all_finite(const float *v)
-{
-    float acc = 0.0f;
-#pragma unroll
-    for (int i = 0; i < N; ++i) acc = fmaf(0.0f, v[i], acc);
-    return acc == 0.0f;
-}
 
 __device__ __forceinline__ void cp_async4(float *dst, const float *src)
 {
@@ -47,14 +37,14 @@ __device__ __forceinline__ void fit_track(const FitGeom &g, const Routing &rt, c
                                           float *slot, int stride, float *ring = nullptr)
 {
     const int64_t T = io.T;
-    float x[6], c[21];
+    float sx[6], sc[21];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) x[i] = __ldcs(io.seed_state + i * T + t);
+    for (int i = 0; i < 6; ++i) sx[i] = __ldcs(io.seed_state + i * T + t);
 #pragma unroll
-    for (int i = 0; i < 21; ++i) c[i] = __ldcs(io.seed_cov + i * T + t);
+    for (int i = 0; i < 21; ++i) sc[i] = __ldcs(io.seed_cov + i * T + t);
     const float qkb = (float)io.charge[t] * g.qk;
     const uint32_t mask = __ldcs(io.hit_mask + t);
-    uint32_t flags = (all_finite<6>(x) && all_finite<21>(c)) ? 0u : (uint32_t)KF_FLAG_NAN_INPUT;
+    uint32_t flags = (all_finite<6>(sx) && all_finite<21>(sc)) ? 0u : (uint32_t)KF_FLAG_NAN_INPUT;
     float chi2 = 0.0f;
     int nhits = 0;
     const float *hp = io.hit_pos + t;  // layer l, component i: hp[(3 l + i) T]
@@ -90,6 +80,13 @@ __device__ __forceinline__ void fit_track(const FitGeom &g, const Routing &rt, c
 #pragma unroll
         for (int k = 0; k < DEPTH; ++k) issue();
     }
+    Local p;
+    float c[15], pn;
+    bool at_seed = true;  // no layer reached
+    if (!flags) {
+        flags = enter_local(sx, sc, qkb, g.r[0], g.inv_r[0], g.z_half, p, c, pn);
+        at_seed = flags != 0u;
+    }
     for (int l = 0; l < g.L && !(flags & kStop); ++l) {
         const bool has = (mask >> l) & 1u;
         const bool has_next = l + 1 < g.L && ((mask >> (l + 1)) & 1u);
@@ -110,23 +107,19 @@ __device__ __forceinline__ void fit_track(const FitGeom &g, const Routing &rt, c
             }
             stage_out = stage_out == DEPTH ? 0 : stage_out + 1;
         }
-        float xn[6], s;
-        Jac J;
-        if (!propagate(x, qkb, g.r[l], xn, s, &J)) {
-            flags |= KF_FLAG_UNREACHABLE;
-            break;
+        if (l > 0) {
+            LocalJac J;
+            const uint32_t stop = step_local(p, qkb, g.r[l], g.inv_r[l], g.z_half, J, pn);
+            if (stop) {
+                flags |= stop;
+                break;
+            }
+            transport_local(J, c);
         }
-        if (fabsf(xn[2]) > g.z_half) {
-            flags |= KF_FLAG_LEFT_BARREL;
-            break;
-        }
-        transport(J, c);
-        add_scattering(xn, g.inv_r[l], g.xx0[l], c);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) x[i] = xn[i];
+        scatter_local(p, noise_local(p, pn, g.xx0[l]), c);
         if (has) {
             float d = 0.0f;
-            const int st = update(x, c, m, v, rt, &d, slot, stride);
+            const int st = update_local(p, c, m, v, rt, &d, slot, stride);
             if (st == 1 || !isfinite(d)) {
                 if (!all_finite<3>(m) || !all_finite<6>(v)) {
                     flags |= KF_FLAG_NAN_INPUT;
@@ -152,18 +145,21 @@ __device__ __forceinline__ void fit_track(const FitGeom &g, const Routing &rt, c
         }
     }
     if constexpr (DEPTH > 1) cp_async_wait<0>();  // no copy of this track may land in the next one's ring
-    if (flags & KF_FLAG_NAN_INPUT) {  // a track with bad input returns its seed
+    float x[6], c6[21];
+    if (at_seed || (flags & KF_FLAG_NAN_INPUT)) {  // a track with bad input returns its seed
 #pragma unroll
         for (int i = 0; i < 6; ++i) x[i] = io.seed_state[i * T + t];
 #pragma unroll
-        for (int i = 0; i < 21; ++i) c[i] = io.seed_cov[i * T + t];
+        for (int i = 0; i < 21; ++i) c6[i] = io.seed_cov[i * T + t];
         chi2 = 0.0f;
         nhits = 0;
+    } else {
+        leave_local(p, c, x, c6);
     }
 #pragma unroll
     for (int i = 0; i < 6; ++i) __stcs(io.out_state + i * T + t, x[i]);
 #pragma unroll
-    for (int i = 0; i < 21; ++i) __stcs(io.out_cov + i * T + t, c[i]);
+    for (int i = 0; i < 21; ++i) __stcs(io.out_cov + i * T + t, c6[i]);
     __stcs(io.out_chi2 + t, chi2);
     io.out_ndof[t] = (int16_t)(3 * nhits - 6);
     io.out_flags[t] = flags;

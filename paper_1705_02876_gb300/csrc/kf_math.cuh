@@ -7,11 +7,23 @@
 
 #include <stdint.h>
 
+#include "kf.h"
+
 namespace kf {
 
 constexpr float kField = 0.00299792458f;  // GeV / (cm T)
 
 __host__ __device__ constexpr int pk(int i, int j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; }
+
+// 0 * v is 0 for finite v and NaN otherwise
+template <int N>
+__device__ __forceinline__ bool all_finite(const float *v)
+{
+    float acc = 0.0f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc = fmaf(0.0f, v[i], acc);
+    return acc == 0.0f;
+}
 
 // Divisions on the FP32 path use __fdividef (reciprocal approximation and a
 // multiply, within 2 ulp for divisors of magnitude 2^-126..2^126, which every
@@ -43,19 +55,20 @@ struct Jac {
 // in tau, so only one atan (for z) is evaluated.  A start moving inwards with
 // u + sqrt(Q) <= 0 takes the general two-root path.  Returns false if the
 // cylinder is not reached.
-__device__ __forceinline__ bool propagate(const float x[6], float qkb, float r, float xn[6],
-                                          float &s_out, Jac *J)
+//
+// crossing() solves for the turn of a start (x, y) moving along (tx, ty):
+// the transverse path length s, and with the turning angle phi = om s
+// a = sin(phi) / om, b = (1 - cos(phi)) / om, sn = sin(phi), c = cos(phi).
+struct Turn {
+    float s, a, b, sn, c;
+};
+__device__ __forceinline__ bool crossing(float x, float y, float tx, float ty, float om, float pt2, float r, Turn &t)
 {
-    const float px = x[3], py = x[4], pz = x[5];
-    const float pt2 = px * px + py * py;
-    const float ipt = rsqrtf(pt2);
-    const float tx = px * ipt, ty = py * ipt;
-    const float om = qkb * ipt;
-    const float u = x[0] * tx + x[1] * ty;
-    const float w = x[0] * ty - x[1] * tx;
-    const float D = r * r - (x[0] * x[0] + x[1] * x[1]);
-    const float Bp = 1.0f + om * w - 0.25f * om * om * D;
-    const float Qd = u * u + D * Bp;
+    const float u = fmaf(x, tx, y * ty);
+    const float w = fmaf(x, ty, -y * tx);
+    const float D = fmaf(r, r, -fmaf(x, x, y * y));
+    const float Bp = fmaf(-0.25f * om * om, D, fmaf(om, w, 1.0f));
+    const float Qd = fmaf(u, u, D * Bp);
     if (!(Qd >= 0.0f) || !(pt2 > 0.0f)) return false;
     const float sq = sqrtf(Qd);
     float s, tau, sigma;
@@ -100,41 +113,54 @@ __device__ __forceinline__ bool propagate(const float x[6], float qkb, float r, 
         sigma = om != 0.0f ? 2.0f * tau / om : s;
         if (!(s < INFINITY)) return false;
     }
-    const float g = __fdividef(1.0f, 1.0f + tau * tau);
-    const float a = sigma * g;          // sin(phi) / omega
-    const float b = sigma * tau * g;    // (1 - cos(phi)) / omega
-    const float sn = 2.0f * tau * g;    // sin(phi)
-    const float c = 1.0f - 2.0f * tau * tau * g;  // cos(phi)
-    xn[0] = x[0] + tx * a + ty * b;
-    xn[1] = x[1] + ty * a - tx * b;
-    xn[2] = x[2] + pz * s * ipt;
-    xn[3] = px * c + py * sn;
-    xn[4] = py * c - px * sn;
+    const float g = __fdividef(1.0f, fmaf(tau, tau, 1.0f));
+    t.s = s;
+    t.a = sigma * g;
+    t.b = sigma * tau * g;
+    t.sn = 2.0f * tau * g;
+    t.c = fmaf(-tau, t.sn, 1.0f);
+    return true;
+}
+
+__device__ __forceinline__ bool propagate(const float x[6], float qkb, float r, float xn[6], Jac &J)
+{
+    const float px = x[3], py = x[4], pz = x[5];
+    const float pt2 = fmaf(px, px, py * py);
+    const float ipt = rsqrtf(pt2);
+    const float tx = px * ipt, ty = py * ipt;
+    const float om = qkb * ipt;
+    Turn t;
+    if (!crossing(x[0], x[1], tx, ty, om, pt2, r, t)) return false;
+    const float s = t.s, a = t.a, b = t.b, sn = t.sn, c = t.c;
+    xn[0] = x[0] + fmaf(tx, a, ty * b);
+    xn[1] = x[1] + fmaf(ty, a, -tx * b);
+    xn[2] = fmaf(pz * s, ipt, x[2]);
+    xn[3] = fmaf(px, c, py * sn);
+    xn[4] = fmaf(py, c, -px * sn);
     xn[5] = pz;
-    s_out = s;
-    if (J) {
-        const float phi = om * s;
-        const float txn = xn[3] * ipt, tyn = xn[4] * ipt;
-        // D = dF/dx0 at fixed s (phi depends on pT through omega)
-        const float d03 = (a - s * tx * txn) * ipt, d04 = (b - s * ty * txn) * ipt;
-        const float d13 = (-b - s * tx * tyn) * ipt, d14 = (a - s * ty * tyn) * ipt;
-        const float d33 = c - phi * tx * tyn, d34 = sn - phi * ty * tyn;
-        const float d43 = -sn + phi * tx * txn, d44 = c + phi * ty * txn;
-        const float lz = pz * ipt;  // dz/ds
-        const float d23 = -s * lz * tx * ipt, d24 = -s * lz * ty * ipt;
-        // ds/dx0 from the constraint x'^2 + y'^2 = r^2
-        const float iden = __fdividef(-1.0f, xn[0] * txn + xn[1] * tyn);
-        const float ds0 = xn[0] * iden, ds1 = xn[1] * iden;
-        const float ds3 = (xn[0] * d03 + xn[1] * d13) * iden;
-        const float ds4 = (xn[0] * d04 + xn[1] * d14) * iden;
-        const float f0 = txn, f1 = tyn, f3 = om * xn[4], f4 = -om * xn[3];  // dF/ds on P
-        J->T[0][0] = 1.0f + f0 * ds0; J->T[0][1] = f0 * ds1; J->T[0][2] = d03 + f0 * ds3; J->T[0][3] = d04 + f0 * ds4;
-        J->T[1][0] = f1 * ds0; J->T[1][1] = 1.0f + f1 * ds1; J->T[1][2] = d13 + f1 * ds3; J->T[1][3] = d14 + f1 * ds4;
-        J->T[2][0] = f3 * ds0; J->T[2][1] = f3 * ds1; J->T[2][2] = d33 + f3 * ds3; J->T[2][3] = d34 + f3 * ds4;
-        J->T[3][0] = f4 * ds0; J->T[3][1] = f4 * ds1; J->T[3][2] = d43 + f4 * ds3; J->T[3][3] = d44 + f4 * ds4;
-        J->jz[0] = lz * ds0; J->jz[1] = lz * ds1; J->jz[2] = d23 + lz * ds3; J->jz[3] = d24 + lz * ds4;
-        J->jzpz = s * ipt;
+    const float phi = om * s;
+    const float txn = xn[3] * ipt, tyn = xn[4] * ipt;
+    // D = dF/dx0 at fixed s (phi depends on pT through omega)
+    const float d03 = fmaf(-s * tx, txn, a) * ipt, d04 = fmaf(-s * ty, txn, b) * ipt;
+    const float d13 = fmaf(-s * tx, tyn, -b) * ipt, d14 = fmaf(-s * ty, tyn, a) * ipt;
+    const float d33 = fmaf(-phi * tx, tyn, c), d34 = fmaf(-phi * ty, tyn, sn);
+    const float d43 = fmaf(phi * tx, txn, -sn), d44 = fmaf(phi * ty, txn, c);
+    const float lz = pz * ipt;  // dz/ds
+    const float d23 = -s * lz * tx * ipt, d24 = -s * lz * ty * ipt;
+    // ds/dx0 from the constraint x'^2 + y'^2 = r^2
+    const float iden = __fdividef(-1.0f, fmaf(xn[0], txn, xn[1] * tyn));
+    const float ds[4] = {xn[0] * iden, xn[1] * iden, fmaf(xn[0], d03, xn[1] * d13) * iden,
+                         fmaf(xn[0], d04, xn[1] * d14) * iden};
+    const float f[4] = {txn, tyn, om * xn[4], -om * xn[3]};  // dF/ds on P
+    const float d[4][4] = {{1.0f, 0.0f, d03, d04}, {0.0f, 1.0f, d13, d14}, {0.0f, 0.0f, d33, d34}, {0.0f, 0.0f, d43, d44}};
+    const float dz[4] = {0.0f, 0.0f, d23, d24};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) J.T[i][j] = fmaf(f[i], ds[j], d[i][j]);
+        J.jz[j] = fmaf(lz, ds[j], dz[j]);
     }
+    J.jzpz = s * ipt;
     return true;
 }
 
@@ -204,36 +230,6 @@ __device__ __forceinline__ void transport(const Jac &J, float c[21])
     for (int i = 0; i < 21; ++i) c[i] = nc[i];
 }
 
-// theta0^2 of the Highland formula (beta = 1) for a thin layer of x_over_x0
-// radiation lengths crossed at xn on radius 1/inv_r (path x_over_x0 /
-// |cos(incidence)|); p2 receives |p|^2.
-__device__ __forceinline__ float scattering_theta2(const float xn[6], float inv_r, float x_over_x0, float &p2)
-{
-    const float px = xn[3], py = xn[4], pz = xn[5];
-    p2 = px * px + py * py + pz * pz;
-    const float ip = rsqrtf(p2);
-    const float cosi = fabsf(px * xn[0] + py * xn[1]) * ip * inv_r;
-    const float xx0 = __fdividef(x_over_x0, cosi);
-    const float th = 0.0136f * ip * sqrtf(xx0) * (1.0f + 0.038f * __logf(xx0));
-    return th * th;
-}
-
-// Multiple scattering of a thin layer: Q = theta0^2 (|p|^2 I3 - p p^T) added
-// to the momentum block.
-__device__ __forceinline__ void add_scattering(const float xn[6], float inv_r, float x_over_x0, float c[21])
-{
-    if (!(x_over_x0 > 0.0f)) return;
-    const float px = xn[3], py = xn[4], pz = xn[5];
-    float p2;
-    const float t2 = scattering_theta2(xn, inv_r, x_over_x0, p2);
-    c[pk(3, 3)] = fmaf(t2, p2 - px * px, c[pk(3, 3)]);
-    c[pk(4, 3)] = fmaf(-t2, px * py, c[pk(4, 3)]);
-    c[pk(4, 4)] = fmaf(t2, p2 - py * py, c[pk(4, 4)]);
-    c[pk(5, 3)] = fmaf(-t2, pz * px, c[pk(5, 3)]);
-    c[pk(5, 4)] = fmaf(-t2, pz * py, c[pk(5, 4)]);
-    c[pk(5, 5)] = fmaf(t2, p2 - pz * pz, c[pk(5, 5)]);
-}
-
 // The extended-precision paths are out of line and rare.  A non-inlined
 // function's registers count towards the kernel's allocation, so these work
 // from a per-thread slot of shared memory ([kSlotSize][stride] floats,
@@ -241,19 +237,7 @@ __device__ __forceinline__ void add_scattering(const float xn[6], float inv_r, f
 // writing the covariance one row at a time: the kernel keeps the register
 // budget of the FP32 main path.
 constexpr int kSlotX = 0, kSlotC = 6, kSlotM = 27, kSlotV = 30, kSlotChi2 = 36, kSlotSize = 37;
-
-__device__ __forceinline__ void slot_write(float *slot, int stride, const float x[6], const float c[21], const float m[3],
-                                           const float v[6])
-{
-#pragma unroll
-    for (int i = 0; i < 6; ++i) slot[(kSlotX + i) * stride] = x[i];
-#pragma unroll
-    for (int i = 0; i < 21; ++i) slot[(kSlotC + i) * stride] = c[i];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) slot[(kSlotM + i) * stride] = m[i];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) slot[(kSlotV + i) * stride] = v[i];
-}
+constexpr int kSlotFrame = kSlotC + 15;  // f0, f1, nx, ny
 
 struct SlotRef {
     float *p;
@@ -263,59 +247,13 @@ struct SlotRef {
     __device__ __forceinline__ float &m(int i) const { return p[(kSlotM + i) * stride]; }
     __device__ __forceinline__ float &v(int i) const { return p[(kSlotV + i) * stride]; }
     __device__ __forceinline__ float &chi2() const { return p[kSlotChi2 * stride]; }
+    __device__ __forceinline__ float n(int i) const { return p[(kSlotFrame + 2 + i) * stride]; }
 };
 
-// The slow paths work in the same local frame as the FP32 update (below):
-// n = (x, y)/|(x, y)| at the predicted position, t = z x n.  The slot holds
-// the Cartesian covariance, whose radial row is the FP32 rounding residue of
-// an exact zero; the local block over (t, z, px, py, pz) drops it, exactly as
-// the FP32 path does (in Cartesian form that residue, of order 1e-7 C_tt, can
-// rival a fine hit's V_nn and bias the update).  The slot's 21 covariance
-// floats are rewritten in place as the 15 of the local block (packed, local
-// index u = 0 t, 1 z, 2 px, 3 py, 4 pz) and back: every value is streamed
-// through the slot so that these out-of-line paths keep the register budget
-// of the FP32 main path.  After the update the Cartesian covariance is
-// rebuilt from the local block (x = -n_y t, y = n_x t), so its radial row is
-// exactly zero again.
-template <class R>
-__device__ __forceinline__ void slot_to_local(const SlotRef &sl, R nx, R ny)
-{
-    float *c = sl.p + kSlotC * sl.stride;
-    auto C = [&](int i, int j) -> float & { return c[pk(i, j) * sl.stride]; };
-    const float ltt = (float)(ny * ny * (R)C(0, 0) - 2 * nx * ny * (R)C(1, 0) + nx * nx * (R)C(1, 1));
-    float lkt[4];
-#pragma unroll
-    for (int k = 2; k < 6; ++k) lkt[k - 2] = (float)(nx * (R)C(k, 1) - ny * (R)C(k, 0));
-    // increasing local position: every source lies above its destination and
-    // is read before it is overwritten
-#pragma unroll 1
-    for (int u = 1; u < 5; ++u)
-#pragma unroll 1
-        for (int w = 1; w <= u; ++w) C(u, w) = C(u + 1, w + 1);
-    C(0, 0) = ltt;
-#pragma unroll
-    for (int u = 1; u < 5; ++u) C(u, 0) = lkt[u - 1];
-}
-
-template <class R>
-__device__ __forceinline__ void slot_to_cartesian(const SlotRef &sl, R nx, R ny)
-{
-    float *c = sl.p + kSlotC * sl.stride;
-    auto C = [&](int i, int j) -> float & { return c[pk(i, j) * sl.stride]; };
-    // decreasing Cartesian position: every source lies below its destination
-#pragma unroll 1
-    for (int i = 5; i >= 2; --i) {
-#pragma unroll 1
-        for (int j = i; j >= 2; --j) C(i, j) = C(i - 1, j - 1);
-        const R lt = (R)C(i - 1, 0);
-        C(i, 1) = (float)(nx * lt);
-        C(i, 0) = (float)(-ny * lt);
-    }
-    const R ltt = (R)C(0, 0);
-    C(1, 1) = (float)(nx * nx * ltt);
-    C(1, 0) = (float)(-nx * ny * ltt);
-    C(0, 0) = (float)(ny * ny * ltt);
-}
+// The slow paths work in the same local coordinates as the FP32 update
+// (below): n = (x, y)/|(x, y)| at the predicted position, t = z x n; the slot
+// holds the position, the momentum (q1, q2, pz), the 15 floats of the local
+// covariance, packed over u = 0 t, 1 z, 2 q1, 3 q2, 4 pz, and the frame's n.
 
 // C_l -= K C_l[{t, z}, :] in place on the slot's local block, row u's gain
 // (kt[u], kz[u]) against the original t and z columns: rows and, within a
@@ -337,66 +275,80 @@ __device__ __forceinline__ void slot_local_downdate(const SlotRef &sl, const R k
         }
 }
 
-// Update in FP64 on the slot, in the local frame: S (n, t, z) and S^-1 by
-// adjugate, the gain's five non-radial rows, x += K r, C -= K C[{t, z}, :]
-// on the local block, chi2 = r^T S^-1 r; then the PSD repair: a local
-// variance that cancellation drove to zero or below is clamped to 1e-12 of
-// the local trace (correlations are left alone).  Returns 2, 3 (repaired) or
-// 1 (S not positive definite).
+// The update in FP64 on the slot: the factorisation and the two scalar
+// updates of update_local (below); then the PSD repair: a variance that
+// cancellation drove to zero or below is clamped to 1e-12 of the trace
+// (correlations are left alone).  Returns 2, 3 (repaired) or 1 (S not positive
+// definite).  The FP64 pipe takes a warp instruction every 16 cycles of the SM,
+// so the form with the fewest of them is used: some 130 and the conversions
+// (an adjugate of S, and a gain with three columns, needed about 250).
 static __device__ __noinline__ int update_fp64(float *slot_p, int stride)
 {
     const SlotRef sl{slot_p, stride};
-    const double X0 = sl.x(0), X1 = sl.x(1);
-    const double ir = 1.0 / sqrt(X0 * X0 + X1 * X1);
-    const double nx = X0 * ir, ny = X1 * ir;
-    slot_to_local<double>(sl, nx, ny);
-    auto L = [&](int i, int j) -> float & { return sl.c(i, j); };  // the slot's local block
-    const double v0 = sl.v(0), v1 = sl.v(1), v2 = sl.v(2), v3 = sl.v(3), v4 = sl.v(4), v5 = sl.v(5);
-    const double a = nx * nx * v0 + 2.0 * nx * ny * v1 + ny * ny * v2;
-    const double b = nx * ny * (v2 - v0) + (nx * nx - ny * ny) * v1;
-    const double cc = (double)L(0, 0) + (ny * ny * v0 - 2.0 * nx * ny * v1 + nx * nx * v2);
-    const double d = nx * v3 + ny * v4, e = (double)L(1, 0) + (nx * v4 - ny * v3), f = (double)L(1, 1) + v5;
-    const double i00 = cc * f - e * e, i10 = d * e - b * f, i11 = a * f - d * d;
-    const double i20 = b * e - cc * d, i21 = b * d - a * e, i22 = a * cc - b * b;
-    const double det = a * i00 + b * i10 + d * i20;
-    if (!(a > 0.0) || !(i22 > 0.0) || !(det > 0.0)) {
-        slot_to_cartesian<double>(sl, nx, ny);
-        return 1;
+    double nx = sl.n(0), ny = sl.n(1);
+    {  // the frame's n, normalised to FP64 (one Newton step)
+        const double h = fma(-0.5, fma(nx, nx, ny * ny), 1.5);
+        nx *= h;
+        ny *= h;
     }
-    const double id = 1.0 / det;
-    const double s00 = i00 * id, s10 = i10 * id, s11 = i11 * id, s20 = i20 * id, s21 = i21 * id, s22 = i22 * id;
+    double vt, vz, l, ia, it, iz;
+    {
+        const double v0 = sl.v(0), v1 = sl.v(1), v2 = sl.v(2), v3 = sl.v(3), v4 = sl.v(4);
+        const double nn = nx * nx, tt = ny * ny, nt = nx * ny;
+        const double vnn = fma(nn, v0, fma(2.0 * nt, v1, tt * v2));
+        const double vnt = fma(nt, v2 - v0, (nn - tt) * v1);
+        const double vtt = fma(tt, v0, fma(-2.0 * nt, v1, nn * v2));
+        const double vnz = fma(nx, v3, ny * v4), vtz = fma(nx, v4, -ny * v3);
+        ia = 1.0 / vnn;
+        vt = vnt * ia;
+        vz = vnz * ia;
+        const double dt = fma(-vnt, vt, (double)sl.c(0, 0) + vtt);
+        it = 1.0 / dt;
+        const double e = fma(-vnt, vz, (double)sl.c(1, 0) + vtz);
+        l = e * it;
+        const double dz = fma(-l, e, fma(-vnz, vz, (double)sl.c(1, 1) + (double)sl.v(5)));
+        if (!(vnn > 0.0 && dt > 0.0 && dz > 0.0 && dz < INFINITY)) return 1;
+        iz = 1.0 / dz;
+    }
+    const double X0 = sl.x(0), X1 = sl.x(1);
     const double d0 = (double)sl.m(0) - X0, d1 = (double)sl.m(1) - X1;
-    const double rn = nx * d0 + ny * d1, rt = nx * d1 - ny * d0, rz = (double)sl.m(2) - sl.x(2);
-    const double q0 = s00 * rn + s10 * rt + s20 * rz, q1 = s10 * rn + s11 * rt + s21 * rz;
-    const double q2 = s20 * rn + s21 * rt + s22 * rz;
-    sl.chi2() = (float)(rn * q0 + rt * q1 + rz * q2);
-    double kt[5], kz[5];
+    const double rn = fma(nx, d0, ny * d1);
+    const double r1 = fma(-vt, rn, fma(nx, d1, -ny * d0));
+    const double r2 = fma(-l, r1, fma(-vz, rn, (double)sl.m(2) - (double)sl.x(2)));
+    const double w1 = r1 * it, w2 = r2 * iz;
+    sl.chi2() = (float)fma(rn * rn, ia, fma(r1, w1, r2 * w2));
+    const double b0 = fma(-l, (double)sl.c(0, 0), (double)sl.c(1, 0));
+    // rows descending and, in a row, columns descending read only entries not
+    // yet rewritten (b0 is kept); rolled, for the callers' registers
 #pragma unroll 1
-    for (int u = 0; u < 5; ++u) {
-        const double ct = L(u, 0), cz = L(u, 1);
-        kt[u] = ct * s11 + cz * s21;
-        kz[u] = ct * s21 + cz * s22;
-        const double dx = (ct * s10 + cz * s20) * rn + kt[u] * rt + kz[u] * rz;
+    for (int u = 4; u >= 0; --u) {
+        const double a = sl.c(u, 0), b = u ? fma(-l, a, (double)sl.c(u, 1)) : b0;
+        const double dx = fma(a, w1, b * w2);
         if (u == 0) {
-            sl.x(0) = (float)(X0 - ny * dx);
-            sl.x(1) = (float)(X1 + nx * dx);
+            sl.x(0) = (float)fma(-ny, dx, X0);
+            sl.x(1) = (float)fma(nx, dx, X1);
         } else {
             sl.x(u + 1) = (float)((double)sl.x(u + 1) + dx);
         }
-    }
-    slot_local_downdate<double>(sl, kt, kz);
-    double tr = 0.0;
+        const double ka = -a * it, kb = -b * iz;
 #pragma unroll 1
-    for (int u = 0; u < 5; ++u) tr += fabs((double)L(u, u));
+        for (int w = u; w >= 0; --w) {
+            const double aw = sl.c(w, 0), bw = w ? fma(-l, aw, (double)sl.c(w, 1)) : b0;
+            sl.c(u, w) = (float)fma(ka, aw, fma(kb, bw, (double)sl.c(u, w)));
+        }
+    }
+    float tr = 0.0f;
     bool rep = false;
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+        tr += fabsf(sl.c(u, u));
+        rep = rep || !(sl.c(u, u) > 0.0f);
+    }
+    if (!rep) return 2;
 #pragma unroll 1
     for (int u = 0; u < 5; ++u)
-        if (!(L(u, u) > 0.0f)) {
-            L(u, u) = (float)(1e-12 * tr);
-            rep = true;
-        }
-    slot_to_cartesian<double>(sl, nx, ny);
-    return rep ? 3 : 2;
+        if (!(sl.c(u, u) > 0.0f)) sl.c(u, u) = 1e-12f * tr;
+    return 3;
 }
 
 // Float-float arithmetic: a value is hi + lo with |lo| <= ulp(hi)/2, about 48
@@ -455,9 +407,7 @@ static __device__ __noinline__ int update_ff(float *slot_p, int stride)
 {
     const SlotRef sl{slot_p, stride};
     const float X0 = sl.x(0), X1 = sl.x(1);
-    const float ir = rsqrtf(X0 * X0 + X1 * X1);
-    const float nx = X0 * ir, ny = X1 * ir;
-    slot_to_local<float>(sl, nx, ny);
+    const float nx = sl.n(0), ny = sl.n(1);
     auto L = [&](int i, int j) -> float & { return sl.c(i, j); };
     const float v0 = sl.v(0), v1 = sl.v(1), v2 = sl.v(2), v3 = sl.v(3), v4 = sl.v(4);
     const ff a{fmaf(nx * nx, v0, fmaf(2.0f * nx * ny, v1, ny * ny * v2)), 0.0f};
@@ -468,10 +418,7 @@ static __device__ __noinline__ int update_ff(float *slot_p, int stride)
     const ff i00 = ff_det2(cc, f, e, e), i10 = ff_det2(d, e, b, f), i11 = ff_det2(a, f, d, d);
     const ff i20 = ff_det2(b, e, cc, d), i21 = ff_det2(b, d, a, e), i22 = ff_det2(a, cc, b, b);
     const ff det = ff_add(ff_mul(a, i00), ff_add(ff_mul(b, i10), ff_mul(d, i20)));
-    if (!(a.hi > 0.0f) || !(i22.hi > 0.0f) || !(det.hi > 0.0f)) {
-        slot_to_cartesian<float>(sl, nx, ny);
-        return 1;
-    }
+    if (!(a.hi > 0.0f) || !(i22.hi > 0.0f) || !(det.hi > 0.0f)) return 1;
     // 1/det: one Newton step on the FP32 reciprocal, r + r (1 - det r)
     const float rc = 1.0f / det.hi;
     const ff one_minus = ff_add(ff{1.0f, 0.0f}, ff_neg(ff_mul(det, ff{rc, 0.0f})));
@@ -504,7 +451,6 @@ static __device__ __noinline__ int update_ff(float *slot_p, int stride)
         }
     }
     slot_local_downdate<float>(sl, kt, kz);
-    slot_to_cartesian<float>(sl, nx, ny);
     return 2;
 }
 
@@ -520,132 +466,339 @@ struct Routing {
     float gain_max;  // information-gain threshold: C_ii / V_ii above it routes the gain
 };
 
+// ---------------------------------------------------------------------------
+// The filter on the covariance of a track's local coordinates.  On a
+// cylinder the crossing cannot move along the radial direction, so the
+// covariance has five dimensions, not six: (t, z, q1, q2, pz), the position
+// along t = z x n and along z, and the momentum.  The transverse momentum is
+// kept in a frame that turns with the track: p = F (q1, q2), F the rotation
+// (f0, -f1; f1, f0).  F is turned by the angle the helix turns the momentum
+// by, so q1 and q2 do not change along a helix and the Jacobian from one layer
+// to the next is the identity but for one row and a rank-one term:
+//   lambda = L . (dt, dq1, dq2)   (the turning angle's change over omega)
+//   t'     = A . (dt, dq1, dq2)
+//   z'     = z + jp pz + lz lambda,  q' = q + W lambda,  pz' = pz,
+// with that, e the unit direction and its left normal before the step, that',
+// e' after it, n0, t0 and n1 the layers' frames, cn = n1 . that',
+// se = n1 . e', W = omega (q2, -q1), jp = s / pT, lz = pz / pT,
+//   A0 = (that' . n0) / cn,  (A1, A2) = (b that + a e) / (pT cn),
+//   L0 = -(n1 . t0) / cn,    (L1, L2) = -((a + b k) that + (a k - b) e) / pT, k = se / cn
+// (that and e in the turning frame: (q1, q2) / pT and (-q2, q1) / pT); the
+// terms in s of the Cartesian Jacobian cancel.  The transport is 67 FP32
+// instructions (178 on the Cartesian block structure), its Jacobian some 30
+// (90), and the update needs no rotation in and out.  F starts along the
+// momentum: the covariance of a stiff track is wide along it (curvature) and
+// narrow across, and entries that mix the two would carry the rounding of the
+// wide one.  Every sum of products below is written with fmaf, so that the
+// rounding does not depend on what the code is inlined into.
+struct Local {
+    float x, y, z, q1, q2, pz;  // position and momentum, p = F (q1, q2)
+    float f0, f1;               // F: cosine and sine
+    float nx, ny;               // n of the last layer reached
+};
+// Packed local covariance: index pk(i, j) over 0 t, 1 z, 2 q1, 3 q2, 4 pz.
+
+struct LocalJac {
+    float A0, A1, A2, L0, L1, L2, W1, W2, jp, lz;
+};
+
+// Step to radius r = 1 / inv_r.  0 and the new position, frames, Jacobian and
+// pn = |p . n| there; or, with p as it was, KF_FLAG_UNREACHABLE, or
+// KF_FLAG_LEFT_BARREL when the crossing lies beyond z_half.
+// With B, the Jacobian of the step back too: the same formulas from n1 to n0
+// by the angle -phi (an inverse of J itself loses its digits near a tangential
+// crossing), and cn_start = n0 . that.
+__device__ __forceinline__ uint32_t step_local(Local &p, float qkb, float r, float inv_r, float z_half, LocalJac &J,
+                                               float &pn, LocalJac *B = nullptr, float *cn_start = nullptr)
+{
+    const float pt2 = fmaf(p.q1, p.q1, p.q2 * p.q2);
+    const float ipt = rsqrtf(pt2);
+    const float om = qkb * ipt;
+    const float tx = fmaf(p.f0, p.q1, -p.f1 * p.q2) * ipt, ty = fmaf(p.f1, p.q1, p.f0 * p.q2) * ipt;
+    Turn t;
+    if (!crossing(p.x, p.y, tx, ty, om, pt2, r, t)) return KF_FLAG_UNREACHABLE;
+    J.jp = t.s * ipt;
+    const float z = fmaf(p.pz, J.jp, p.z);
+    if (fabsf(z) > z_half) return KF_FLAG_LEFT_BARREL;
+    p.z = z;
+    p.x += fmaf(tx, t.a, ty * t.b);
+    p.y += fmaf(ty, t.a, -tx * t.b);
+    const float ux = fmaf(tx, t.c, ty * t.sn), uy = fmaf(ty, t.c, -tx * t.sn);  // that'
+    const float g0 = fmaf(p.f0, t.c, p.f1 * t.sn);
+    p.f1 = fmaf(p.f1, t.c, -p.f0 * t.sn);
+    p.f0 = g0;
+    const float nx = p.x * inv_r, ny = p.y * inv_r;
+    if (B) {
+        const float cn0 = fmaf(p.nx, tx, p.ny * ty), se0 = fmaf(p.ny, tx, -p.nx * ty);
+        const float icn0 = __fdividef(1.0f, cn0), i2 = ipt * ipt, k = se0 * icn0;
+        const float al = -i2 * fmaf(t.b, k, -t.a), be = i2 * fmaf(t.a, k, t.b);
+        const float ga = i2 * icn0 * t.b, de = -i2 * icn0 * t.a;
+        *B = LocalJac{fmaf(tx, nx, ty * ny) * icn0, fmaf(ga, p.q1, -de * p.q2), fmaf(ga, p.q2, de * p.q1),
+                      fmaf(p.nx, ny, -p.ny * nx) * icn0, fmaf(al, p.q1, -be * p.q2), fmaf(al, p.q2, be * p.q1),
+                      om * p.q2, -om * p.q1, -J.jp, p.pz * ipt};
+        *cn_start = cn0;
+    }
+    const float cn = fmaf(nx, ux, ny * uy), se = fmaf(ny, ux, -nx * uy);
+    const float icn = __fdividef(1.0f, cn);
+    J.A0 = fmaf(ux, p.nx, uy * p.ny) * icn;
+    J.L0 = fmaf(nx, p.ny, -ny * p.nx) * icn;
+    p.nx = nx;
+    p.ny = ny;
+    const float i2 = ipt * ipt, k = se * icn;
+    const float al = -i2 * fmaf(t.b, k, t.a), be = i2 * fmaf(-t.a, k, t.b);
+    J.L1 = fmaf(al, p.q1, -be * p.q2);
+    J.L2 = fmaf(al, p.q2, be * p.q1);
+    const float ga = i2 * icn * t.b, de = i2 * icn * t.a;
+    J.A1 = fmaf(ga, p.q1, -de * p.q2);
+    J.A2 = fmaf(ga, p.q2, de * p.q1);
+    J.W1 = om * p.q2;
+    J.W2 = -om * p.q1;
+    J.lz = p.pz * ipt;
+    pn = fabsf(cn) * pt2 * ipt;
+    return 0u;
+}
+
+// c <- J c J^T
+__device__ __forceinline__ void transport_local(const LocalJac &J, float c[15])
+{
+    constexpr int T = 0, Z = 1, U = 2, V = 3, P = 4;
+    auto row = [&](float a0, float a1, float a2, int i) {
+        return fmaf(a0, c[pk(T, i)], fmaf(a1, c[pk(U, i)], a2 * c[pk(V, i)]));
+    };
+    // covariances of lambda and of t' with the old coordinates
+    const float lt = row(J.L0, J.L1, J.L2, T), lz = row(J.L0, J.L1, J.L2, Z), lu = row(J.L0, J.L1, J.L2, U);
+    const float lv = row(J.L0, J.L1, J.L2, V), lp = row(J.L0, J.L1, J.L2, P);
+    const float at = row(J.A0, J.A1, J.A2, T), az = row(J.A0, J.A1, J.A2, Z), au = row(J.A0, J.A1, J.A2, U);
+    const float av = row(J.A0, J.A1, J.A2, V), ap = row(J.A0, J.A1, J.A2, P);
+    const float ll = fmaf(J.L0, lt, fmaf(J.L1, lu, J.L2 * lv));
+    const float tl = fmaf(J.A0, lt, fmaf(J.A1, lu, J.A2 * lv));
+    c[pk(T, T)] = fmaf(J.A0, at, fmaf(J.A1, au, J.A2 * av));
+    c[pk(U, T)] = fmaf(J.W1, tl, au);
+    c[pk(V, T)] = fmaf(J.W2, tl, av);
+    c[pk(P, T)] = ap;
+    c[pk(Z, T)] = fmaf(J.jp, ap, fmaf(J.lz, tl, az));
+    // y = z + jp pz, then z' = y + lz lambda
+    const float yp = fmaf(J.jp, c[pk(P, P)], c[pk(P, Z)]);
+    const float yl = fmaf(J.jp, lp, lz), zl = fmaf(J.lz, ll, yl);
+    const float yy = fmaf(J.jp, c[pk(P, Z)] + yp, c[pk(Z, Z)]);
+    c[pk(Z, Z)] = fmaf(J.lz, yl + zl, yy);
+    c[pk(U, Z)] = fmaf(J.jp, c[pk(P, U)], fmaf(J.lz, lu, fmaf(J.W1, zl, c[pk(U, Z)])));
+    c[pk(V, Z)] = fmaf(J.jp, c[pk(P, V)], fmaf(J.lz, lv, fmaf(J.W2, zl, c[pk(V, Z)])));
+    c[pk(P, Z)] = fmaf(J.lz, lp, yp);
+    const float u1 = fmaf(J.W1, ll, lu), v1 = fmaf(J.W2, ll, lv);  // of lambda with q'
+    c[pk(U, U)] = fmaf(J.W1, lu + u1, c[pk(U, U)]);
+    c[pk(V, U)] = fmaf(J.W2, lu, fmaf(J.W1, v1, c[pk(V, U)]));
+    c[pk(V, V)] = fmaf(J.W2, lv + v1, c[pk(V, V)]);
+    c[pk(P, U)] = fmaf(J.W1, lp, c[pk(P, U)]);
+    c[pk(P, V)] = fmaf(J.W2, lp, c[pk(P, V)]);
+}
+
+// The step from a start anywhere (a seed) with a full 6x6 covariance onto the
+// first layer; the turning frame starts as the laboratory's.  Returns as
+// step_local does (x, c as they were when it fails).
+__device__ __forceinline__ uint32_t enter_local(const float x[6], float c6[21], float qkb, float r, float inv_r,
+                                                float z_half, Local &p, float c[15], float &pn)
+{
+    float xn[6];
+    Jac J;
+    if (!propagate(x, qkb, r, xn, J)) return KF_FLAG_UNREACHABLE;
+    if (fabsf(xn[2]) > z_half) return KF_FLAG_LEFT_BARREL;
+    transport(J, c6);
+    const float pt2 = fmaf(xn[3], xn[3], xn[4] * xn[4]), ipt = rsqrtf(pt2);
+    const float f0 = xn[3] * ipt, f1 = xn[4] * ipt;
+    const float nx = xn[0] * inv_r, ny = xn[1] * inv_r;
+    p = Local{xn[0], xn[1], xn[2], fmaf(f0, xn[3], f1 * xn[4]), fmaf(f0, xn[4], -f1 * xn[3]), xn[5], f0, f1, nx, ny};
+    // rows t, z, pz against (t, z, px, py, pz), then the momentum columns turned
+    auto lt = [&](int j) { return fmaf(nx, c6[pk(j, 1)], -ny * c6[pk(j, 0)]); };
+    auto qu = [&](float a, float b) { return fmaf(f0, a, f1 * b); };
+    auto qv = [&](float a, float b) { return fmaf(f0, b, -f1 * a); };
+    c[pk(0, 0)] = fmaf(ny * ny, c6[pk(0, 0)], fmaf(-2.0f * nx * ny, c6[pk(1, 0)], nx * nx * c6[pk(1, 1)]));
+    c[pk(1, 0)] = lt(2);
+    c[pk(1, 1)] = c6[pk(2, 2)];
+    const float tu = lt(3), tv = lt(4);
+    c[pk(2, 0)] = qu(tu, tv);
+    c[pk(3, 0)] = qv(tu, tv);
+    c[pk(4, 0)] = lt(5);
+    c[pk(2, 1)] = qu(c6[pk(3, 2)], c6[pk(4, 2)]);
+    c[pk(3, 1)] = qv(c6[pk(3, 2)], c6[pk(4, 2)]);
+    c[pk(4, 1)] = c6[pk(5, 2)];
+    const float ux = qu(c6[pk(3, 3)], c6[pk(4, 3)]), uy = qu(c6[pk(4, 3)], c6[pk(4, 4)]);
+    c[pk(2, 2)] = qu(ux, uy);
+    c[pk(3, 2)] = qv(ux, uy);
+    c[pk(3, 3)] = qv(qv(c6[pk(3, 3)], c6[pk(4, 3)]), qv(c6[pk(4, 3)], c6[pk(4, 4)]));
+    c[pk(4, 2)] = qu(c6[pk(5, 3)], c6[pk(5, 4)]);
+    c[pk(4, 3)] = qv(c6[pk(5, 3)], c6[pk(5, 4)]);
+    c[pk(4, 4)] = c6[pk(5, 5)];
+    pn = fabsf(fmaf(xn[3], p.nx, xn[4] * p.ny));
+    return 0u;
+}
+
+// The momentum noise of a thin layer, theta0^2 (|p|^2 I3 - p p^T) (Highland,
+// beta = 1, path x_over_x0 / |cos(incidence)|): theta0^2.
+__device__ __forceinline__ float noise_local(const Local &p, float pn, float x_over_x0)
+{
+    if (!(x_over_x0 > 0.0f)) return 0.0f;
+    const float ip = rsqrtf(fmaf(p.pz, p.pz, fmaf(p.q1, p.q1, p.q2 * p.q2)));
+    const float xx0 = __fdividef(x_over_x0, pn * ip);
+    const float lg = fmaf(0.038f, __logf(xx0), 1.0f);
+    return (0.0136f * 0.0136f) * (ip * ip) * xx0 * (lg * lg);
+}
+
+// That noise, theta2 = theta0^2, added to the momentum block.
+__device__ __forceinline__ void scatter_local(const Local &p, float theta2, float c[15])
+{
+    const float tu = -theta2 * p.q1, tv = -theta2 * p.q2;
+    c[pk(2, 2)] = fmaf(theta2, fmaf(p.q2, p.q2, p.pz * p.pz), c[pk(2, 2)]);
+    c[pk(3, 2)] = fmaf(tu, p.q2, c[pk(3, 2)]);
+    c[pk(3, 3)] = fmaf(theta2, fmaf(p.q1, p.q1, p.pz * p.pz), c[pk(3, 3)]);
+    c[pk(4, 2)] = fmaf(tu, p.pz, c[pk(4, 2)]);
+    c[pk(4, 3)] = fmaf(tv, p.pz, c[pk(4, 3)]);
+    c[pk(4, 4)] = fmaf(theta2, fmaf(p.q1, p.q1, p.q2 * p.q2), c[pk(4, 4)]);
+}
+
 // Update with a 3-D hit (Section 2.1: 3x3 measurement covariance V).
 //   S = C_xx + V, K = C[:, 0:3] S^-1, x += K r, C -= K C[0:3, :],
 //   dchi2 = r^T S^-1 r.
 //
-// The FP32 path works in the local frame of the layer at the predicted
-// position: n = (x, y, 0)/|(x, y)|, t = z x n, z.  Transport onto the cylinder
-// leaves the covariance the exact null vector n (the crossing cannot move off
-// the surface), so in x/y the exactly known radial direction and the
-// uncertain tangential one share every entry and FP32 cannot resolve the gain
-// of an update that shrinks the covariance by orders of magnitude (a hit
-// after a diffuse seed).  In (n, t, z) they decouple: C's radial row is zero
-// (its rounding residue is dropped), S = [[V_nn, V_nt, V_nz], [V_nt, C_tt +
-// V_tt, C_tz + V_tz], [V_nz, C_tz + V_tz, C_zz + V_zz]], the gain's radial
-// row is zero, and only the five non-radial rows (t, z, px, py, pz) are
-// updated, each from the t and z columns.  dx and C are rotated back to x/y.
+// In (n, t, z) C has no radial row, and the exactly known radial direction
+// does not mix with the uncertain tangential one, which in x/y share every
+// entry (FP32 could not resolve the gain of an update that shrinks the
+// covariance by orders of magnitude, a hit after a diffuse seed).  S is
+// factorised in the order n, t, z: with vt = V_nt / V_nn, vz = V_nz / V_nn the
+// hit's t and z given its n, S's t pivot dt, its z pivot dz and l = S_zt' / dt,
+// three residuals rn, r1, r2 with variances V_nn, dt, dz,
+//   chi2 = rn^2 / V_nn + r1^2 / dt + r2^2 / dz,
+// and the gain is two scalar updates with the columns C_t and C_z - l C_t.
+// det S = V_nn dt dz, positive definite when all three pivots are positive.
 // Routing (mode 1):
 //   * the whole update is redone in FP64 with a PSD repair (update_fp64) when
 //     S is not positive definite in FP32, when the determinant of its
 //     correlation matrix R = D^-1/2 S D^-1/2 (D = diag S) is below
-//     27 / (4 cond_max), which keeps cond_2(R) <= cond_max on the FP32 path,
-//     or when pT lies outside [pt_lo, pt_hi];
+//     27 / (4 cond_max) (R's eigenvalues sum to 3, so that this bounds
+//     cond_2(R) by cond_max on the FP32 path; the spread of S's diagonal, V_nn
+//     << C_zz, is harmless), or when pT lies outside [pt_lo, pt_hi];
 //   * with gain_max > 0, the gain is formed in float-float (update_ff) when
-//     C_ii > gain_max V_ii for some i.  Float-float runs on the FP32 pipe,
-//     which on this part is 64 times wider than the FP64 one.
+//     C_ii > gain_max V_ii for some i.
 // Returns 0 updated in FP32, 2 updated with extended-precision arithmetic,
 // 3 updated in FP64 with a PSD repair, 1 failed (S not positive definite).
-__device__ __forceinline__ int update(float x[6], float c[21], const float m[3], const float v[6],
-                                      const Routing &rt, float *dchi2, float *slot, int stride)
+__device__ __forceinline__ int update_local(Local &p, float c[15], const float m[3], const float v[6],
+                                            const Routing &rt, float *dchi2, float *slot, int stride)
 {
-    const float ir = rsqrtf(x[0] * x[0] + x[1] * x[1]);
-    const float nx = x[0] * ir, ny = x[1] * ir;
-    // t column of C in the local frame: C_it = -ny C_i0 + nx C_i1 (i >= 2),
-    // C_tt = t^T C_xy t; the z column is C's own
-    const float ctt = fmaf(ny * ny, c[pk(0, 0)], fmaf(-2.0f * nx * ny, c[pk(1, 0)], nx * nx * c[pk(1, 1)]));
-    float ct[6];  // ct[i] = C_l[i][t] for i = 2..5
-#pragma unroll
-    for (int i = 2; i < 6; ++i) ct[i] = fmaf(nx, c[pk(i, 1)], -ny * c[pk(i, 0)]);
-    const float vnn = fmaf(nx * nx, v[0], fmaf(2.0f * nx * ny, v[1], ny * ny * v[2]));
-    const float vnt = fmaf(nx * ny, v[2] - v[0], (nx * nx - ny * ny) * v[1]);
-    const float vtt = fmaf(ny * ny, v[0], fmaf(-2.0f * nx * ny, v[1], nx * nx * v[2]));
+    const float nx = p.nx, ny = p.ny;
+    const float nn = nx * nx, tt = ny * ny, nt = nx * ny;
+    const float vnn = fmaf(nn, v[0], fmaf(2.0f * nt, v[1], tt * v[2]));
+    const float vnt = fmaf(nt, v[2] - v[0], fmaf(nx, nx, -tt) * v[1]);
+    const float vtt = fmaf(tt, v[0], fmaf(-2.0f * nt, v[1], nn * v[2]));
     const float vnz = fmaf(nx, v[3], ny * v[4]), vtz = fmaf(nx, v[4], -ny * v[3]);
-    const float a = vnn, b = vnt, cc = ctt + vtt;
-    const float d = vnz, e = ct[2] + vtz, f = c[pk(2, 2)] + v[5];
-    const float i00 = cc * f - e * e, i10 = d * e - b * f, i11 = a * f - d * d;
-    const float i20 = b * e - cc * d, i21 = b * d - a * e, i22 = a * cc - b * b;
-    const float det = fmaf(a, i00, fmaf(b, i10, d * i20));
-    const bool pd = a > 0.0f && i22 > 0.0f && det > 0.0f;
+    const float stt = c[pk(0, 0)] + vtt, szz = c[pk(1, 1)] + v[5];
+    const float ia = __fdividef(1.0f, vnn);
+    const float vt = vnt * ia, vz = vnz * ia;
+    const float dt = fmaf(-vnt, vt, stt);
+    const float it = __fdividef(1.0f, dt);
+    const float e = fmaf(-vnt, vz, c[pk(1, 0)] + vtz);
+    const float l = e * it;
+    const float dz = fmaf(-l, e, fmaf(-vnz, vz, szz));
+    // an infinite V_zz must not pass: the caller tells a bad hit by the failure
+    const bool pd = vnn > 0.0f && dt > 0.0f && dz > 0.0f && dz < INFINITY;
     int kind = 0;
     if (rt.mode == 1) {
-        // S's correlation matrix R = D^-1/2 S D^-1/2 (D = diag S): the rounding
-        // of the adjugate's cofactors grows with its condition, not with the
-        // spread of S's diagonal (V_nn << C_zz is harmless).  With eigenvalues
-        // summing to 3, det R >= 27 / (4 cond_max) bounds cond_2(R) by cond_max.
-        const bool ill = !pd || det <= rt.det_min * (a * cc * f);
-        const float pt2 = x[3] * x[3] + x[4] * x[4];
+        const bool ill = !pd || dt * dz <= rt.det_min * (stt * szz);
+        const float pt2 = fmaf(p.q1, p.q1, p.q2 * p.q2);
         if (ill || pt2 < rt.pt_lo * rt.pt_lo || pt2 > rt.pt_hi * rt.pt_hi)
             kind = 2;
-        else if (rt.gain_max > 0.0f &&
-                 (c[0] > rt.gain_max * v[0] || c[2] > rt.gain_max * v[2] || c[5] > rt.gain_max * v[5]))
+        else if (rt.gain_max > 0.0f && (tt * c[pk(0, 0)] > rt.gain_max * v[0] || nn * c[pk(0, 0)] > rt.gain_max * v[2] ||
+                                        c[pk(1, 1)] > rt.gain_max * v[5]))
             kind = 1;
     } else if (!pd) {
         return 1;
     }
     if (kind) {
-        slot_write(slot, stride, x, c, m, v);
+        float *s = slot;
+        const float x[6] = {p.x, p.y, p.z, p.q1, p.q2, p.pz};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) s[(kSlotX + i) * stride] = x[i];
+#pragma unroll
+        for (int i = 0; i < 15; ++i) s[(kSlotC + i) * stride] = c[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) s[(kSlotM + i) * stride] = m[i];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) s[(kSlotV + i) * stride] = v[i];
+        s[(kSlotFrame + 2) * stride] = nx;
+        s[(kSlotFrame + 3) * stride] = ny;
         const int st = update_ext(slot, stride, kind);
         if (st == 1) return 1;
+        p.x = s[kSlotX * stride];
+        p.y = s[(kSlotX + 1) * stride];
+        p.z = s[(kSlotX + 2) * stride];
+        p.q1 = s[(kSlotX + 3) * stride];
+        p.q2 = s[(kSlotX + 4) * stride];
+        p.pz = s[(kSlotX + 5) * stride];
 #pragma unroll
-        for (int i = 0; i < 6; ++i) x[i] = slot[(kSlotX + i) * stride];
-#pragma unroll
-        for (int i = 0; i < 21; ++i) c[i] = slot[(kSlotC + i) * stride];
-        *dchi2 = slot[kSlotChi2 * stride];
+        for (int i = 0; i < 15; ++i) c[i] = s[(kSlotC + i) * stride];
+        *dchi2 = s[kSlotChi2 * stride];
         return st;
     }
-    const float id = __fdividef(1.0f, det);
-    const float s00 = i00 * id, s10 = i10 * id, s11 = i11 * id, s20 = i20 * id, s21 = i21 * id, s22 = i22 * id;
-    const float d0 = m[0] - x[0], d1 = m[1] - x[1];
-    const float rn = fmaf(nx, d0, ny * d1), rt_ = fmaf(nx, d1, -ny * d0), rz = m[2] - x[2];
-    const float q0 = fmaf(s00, rn, fmaf(s10, rt_, s20 * rz));
-    const float q1 = fmaf(s10, rn, fmaf(s11, rt_, s21 * rz));
-    const float q2 = fmaf(s20, rn, fmaf(s21, rt_, s22 * rz));
-    *dchi2 = fmaf(rn, q0, fmaf(rt_, q1, rz * q2));
-    // rows u = t, z, px, py, pz (state indices 1..5 of the local frame):
-    // col_t[u] = C_l[u][t], col_z[u] = C_l[u][z], both before the update
-    float col_t[6], col_z[6];
-    col_t[1] = ctt;
-    col_z[1] = ct[2];
-    col_t[2] = ct[2];
-    col_z[2] = c[pk(2, 2)];
+    const float iz = __fdividef(1.0f, dz);
+    const float d0 = m[0] - p.x, d1 = m[1] - p.y;
+    const float rn = fmaf(nx, d0, ny * d1);
+    const float r1 = fmaf(-vt, rn, fmaf(nx, d1, -ny * d0));
+    const float r2 = fmaf(-l, r1, fmaf(-vz, rn, m[2] - p.z));
+    const float w1 = r1 * it, w2 = r2 * iz;
+    *dchi2 = fmaf(rn * rn, ia, fmaf(r1, w1, r2 * w2));
+    float a[5], b[5];  // the columns of the two scalar updates, and their gains
 #pragma unroll
-    for (int u = 3; u < 6; ++u) {
-        col_t[u] = ct[u];
-        col_z[u] = c[pk(u, 2)];
+    for (int i = 0; i < 5; ++i) {
+        a[i] = c[pk(i, 0)];
+        b[i] = fmaf(-l, a[i], c[pk(i, 1)]);
     }
-    // K_u = (C_ut, C_uz) S^-1[{t, z}, :]; the radial row of K is zero
-    float kt[6], kz[6];
+    const float dx = fmaf(a[0], w1, b[0] * w2);
+    p.x = fmaf(-ny, dx, p.x);
+    p.y = fmaf(nx, dx, p.y);
+    p.z += fmaf(a[1], w1, b[1] * w2);
+    p.q1 += fmaf(a[2], w1, b[2] * w2);
+    p.q2 += fmaf(a[3], w1, b[3] * w2);
+    p.pz += fmaf(a[4], w1, b[4] * w2);
 #pragma unroll
-    for (int u = 1; u < 6; ++u) {
-        const float k0 = fmaf(col_t[u], s10, col_z[u] * s20);
-        kt[u] = fmaf(col_t[u], s11, col_z[u] * s21);
-        kz[u] = fmaf(col_t[u], s21, col_z[u] * s22);
-        const float dxu = fmaf(k0, rn, fmaf(kt[u], rt_, kz[u] * rz));
-        if (u == 1) {  // t: back to x/y
-            x[0] = fmaf(-ny, dxu, x[0]);
-            x[1] = fmaf(nx, dxu, x[1]);
-        } else {
-            x[u] += dxu;
-        }
+    for (int i = 0; i < 5; ++i) {
+        const float ka = -a[i] * it, kb = -b[i] * iz;
+#pragma unroll
+        for (int j = 0; j <= i; ++j) c[pk(i, j)] = fmaf(ka, a[j], fmaf(kb, b[j], c[pk(i, j)]));
     }
-    // C'_uw = C_uw - K_ut C_tw - K_uz C_zw over the non-radial 5x5 block
-    const float ntt = fmaf(-kt[1], col_t[1], fmaf(-kz[1], col_z[1], col_t[1]));
-#pragma unroll
-    for (int u = 2; u < 6; ++u) {
-        const float nt = fmaf(-kt[u], col_t[1], fmaf(-kz[u], col_z[1], col_t[u]));  // C'_u t
-        const float nz = fmaf(-kt[u], col_t[2], fmaf(-kz[u], col_z[2], col_z[u]));  // C'_u z
-        c[pk(u, 0)] = -ny * nt;
-        c[pk(u, 1)] = nx * nt;
-        if (u >= 3) c[pk(u, 2)] = nz;
-        else c[pk(2, 2)] = nz;
-#pragma unroll
-        for (int w = 3; w <= u; ++w) c[pk(u, w)] = fmaf(-kt[u], col_t[w], fmaf(-kz[u], col_z[w], c[pk(u, w)]));
-    }
-    c[pk(0, 0)] = ny * ny * ntt;
-    c[pk(1, 0)] = -nx * ny * ntt;
-    c[pk(1, 1)] = nx * nx * ntt;
     return 0;
+}
+
+// The Cartesian state and covariance (packed 6x6) of local coordinates.
+__device__ __forceinline__ void leave_local(const Local &p, const float c[15], float x[6], float c6[21])
+{
+    const float f0 = p.f0, f1 = p.f1;
+    x[0] = p.x;
+    x[1] = p.y;
+    x[2] = p.z;
+    x[3] = fmaf(f0, p.q1, -f1 * p.q2);
+    x[4] = fmaf(f1, p.q1, f0 * p.q2);
+    x[5] = p.pz;
+    auto px = [&](int j) { return fmaf(f0, c[pk(2, j)], -f1 * c[pk(3, j)]); };
+    auto py = [&](int j) { return fmaf(f1, c[pk(2, j)], f0 * c[pk(3, j)]); };
+    const float lt[4] = {c[pk(1, 0)], px(0), py(0), c[pk(4, 0)]};
+    c6[pk(0, 0)] = p.ny * p.ny * c[pk(0, 0)];
+    c6[pk(1, 0)] = -p.nx * p.ny * c[pk(0, 0)];
+    c6[pk(1, 1)] = p.nx * p.nx * c[pk(0, 0)];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        c6[pk(i + 2, 0)] = -p.ny * lt[i];
+        c6[pk(i + 2, 1)] = p.nx * lt[i];
+    }
+    c6[pk(2, 2)] = c[pk(1, 1)];
+    c6[pk(3, 2)] = px(1);
+    c6[pk(4, 2)] = py(1);
+    c6[pk(5, 2)] = c[pk(4, 1)];
+    const float uu = px(2), uv = px(3), vu = py(2), vv = py(3);
+    c6[pk(3, 3)] = fmaf(f0, uu, -f1 * uv);
+    c6[pk(4, 3)] = fmaf(f0, vu, -f1 * vv);
+    c6[pk(4, 4)] = fmaf(f1, vu, f0 * vv);
+    c6[pk(5, 3)] = px(4);
+    c6[pk(5, 4)] = py(4);
+    c6[pk(5, 5)] = c[pk(4, 4)];
 }
 
 }  // namespace kf

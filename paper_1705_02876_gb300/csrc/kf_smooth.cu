@@ -3,28 +3,22 @@
 // gives at every layer the estimate using all of the track's hits (Section 2
 // names a final fit with a smoother as the step after building).
 //
-// On a cylinder the predicted and filtered covariances are singular (the
-// crossing cannot leave the surface: the radial direction n of the predicted
-// crossing carries no variance), so the backward pass works in each layer's
-// local coordinates (t, z, px, py, pz), t = z x n, where they are 5x5 and
-// positive definite.  With G the Jacobian from layer l's local coordinates to
-// layer l+1's and Q the scattering noise added at layer l+1:
-//   A_l  = Cf_l G^T Cp_{l+1}^-1 = G^-1 (I - Q Cp_{l+1}^-1)  (Cp = G Cf G^T + Q),
-//   xs_l = xf_l + R_l A_l (xs_{l+1} - xp_{l+1}),
+// Both passes work in the local coordinates (t, z, q1, q2, pz) of kf_math.cuh,
+// where the covariances are 5x5 and positive definite.  With G the Jacobian
+// from layer l to layer l+1 and Q the scattering noise added at layer l+1:
+//   A_l  = Cf_l G^T Cp_{l+1}^-1 = G^-1 (I - K), K = Q Cp_{l+1}^-1  (Cp = G Cf G^T + Q),
+//   xs_l = xf_l + A_l (xs_{l+1} - xp_{l+1}),
 //   Cs_l = Cf_l + A_l (Cs_{l+1} - Cp_{l+1}) A_l^T.
-// The second form is the one computed: G^-1 is a 3x3 inverse of the
-// transport's transverse block (well conditioned), and Cp^-1 (a Cholesky
-// factorisation of Cp scaled to unit diagonal) only multiplies the scattering
-// noise, so the FP32 rounding that Cp's correlations amplify enters A scaled
-// by |Q| / |Cp|; the other factor is never formed.  The forward pass writes
-// the filtered state and local covariance (with the frame) of every layer to
-// the output arrays; the backward pass reads them, recomputes the prediction
-// of layer l+1 from the filtered estimate of layer l (the same propagation,
-// transport and scattering as the forward pass, on the same state bits: xp, G
-// and Q come out identical, Cp differs by the rounding of the stored local
-// covariance), and overwrites them with the smoothed ones.  Nothing else is
-// stored: a track's filtered estimates (108 B per layer) are read back while
-// still in L2, and each output line reaches DRAM once, smoothed.
+// The second form is the one computed: Cp^-1 (an L D L^T factorisation) only
+// multiplies the scattering noise, so the FP32 rounding that Cp's correlations
+// amplify enters A scaled by |Q| / |Cp|.  K has the three momentum rows only,
+// and G^-1 has the form of G itself (a step back along the helix), so that
+// the covariance goes through the transport of the forward pass.  The forward pass writes the filtered coordinates, their covariance
+// and frames (25 floats) of every layer to the output arrays; the backward
+// pass reads them, repeats the step to layer l+1 (xp, G and Q come out the
+// same, bit for bit) and overwrites them with the smoothed estimate.  Nothing
+// else is stored: they are read back while still in L2, and each output line
+// reaches DRAM once, smoothed.
 #include "kf.h"
 #include "kf_api_internal.h"
 #include "kf_fit.cuh"
@@ -48,72 +42,10 @@ struct SmoothIO {
     uint32_t *out_flags;
 };
 
-__device__ __forceinline__ void local_of(const float c[21], float nx, float ny, float cl[15])
-{
-    cl[0] = fmaf(ny * ny, c[pk(0, 0)], fmaf(-2.0f * nx * ny, c[pk(1, 0)], nx * nx * c[pk(1, 1)]));
-#pragma unroll
-    for (int k = 2; k < 6; ++k) cl[pk(k - 1, 0)] = fmaf(nx, c[pk(k, 1)], -ny * c[pk(k, 0)]);
-#pragma unroll
-    for (int i = 2; i < 6; ++i)
-#pragma unroll
-        for (int j = 2; j <= i; ++j) cl[pk(i - 1, j - 1)] = c[pk(i, j)];
-}
-
-__device__ __forceinline__ float cart_of(const float cl[15], float nx, float ny, int i, int j)
-{
-    const float wi = i == 0 ? -ny : nx, wj = j == 0 ? -ny : nx;
-    if (i < 2 && j < 2) return wi * wj * cl[0];
-    if (i < 2) return wi * cl[pk(j - 1, 0)];
-    if (j < 2) return wj * cl[pk(i - 1, 0)];
-    return cl[pk(i - 1, j - 1)];
-}
-
-// The 13 non-trivial entries of the local Jacobian from frame n0 to frame n1
-// (rows t, z, px, py, pz; columns the same):
-//   t'  = M00 t + M01 px + M02 py,  px' = M10 t + M11 px + M12 py,
-//   py' = M20 t + M21 px + M22 py,  z' = z + mz0 t + mz1 px + mz2 py + jp pz,
-//   pz' = pz;  stored as M (9, row-major), mz (3), jp.
-__device__ __forceinline__ void local_jacobian(const Jac &J, float nx0, float ny0, float nx1, float ny1, float g[13])
-{
-    float a[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) a[k] = fmaf(nx1, J.T[1][k], -ny1 * J.T[0][k]);
-    g[0] = fmaf(nx0, a[1], -ny0 * a[0]);
-    g[1] = a[2];
-    g[2] = a[3];
-#pragma unroll
-    for (int r = 1; r < 3; ++r) {
-        g[3 * r] = fmaf(nx0, J.T[r + 1][1], -ny0 * J.T[r + 1][0]);
-        g[3 * r + 1] = J.T[r + 1][2];
-        g[3 * r + 2] = J.T[r + 1][3];
-    }
-    g[9] = fmaf(nx0, J.jz[1], -ny0 * J.jz[0]);
-    g[10] = J.jz[2];
-    g[11] = J.jz[3];
-    g[12] = J.jzpz;
-}
-
-// The scattering noise of layer l on the momentum block, packed (px,px)
-// (py,px) (py,py) (pz,px) (pz,py) (pz,pz): theta0^2 (|p|^2 I3 - p p^T).
-__device__ __forceinline__ void scattering_q6(const float xn[6], float inv_r, float x_over_x0, float q6[6])
-{
-#pragma unroll
-    for (int i = 0; i < 6; ++i) q6[i] = 0.0f;
-    if (!(x_over_x0 > 0.0f)) return;
-    float p2;
-    const float t2 = scattering_theta2(xn, inv_r, x_over_x0, p2);
-    const float px = xn[3], py = xn[4], pz = xn[5];
-    q6[0] = t2 * (p2 - px * px);
-    q6[1] = -t2 * px * py;
-    q6[2] = t2 * (p2 - py * py);
-    q6[3] = -t2 * pz * px;
-    q6[4] = -t2 * pz * py;
-    q6[5] = t2 * (p2 - pz * pz);
-}
-
-// Registers capped at 128 (four blocks, 16 warps per SM) with a small spill:
-// 2.23 ms on the fit workload against 2.46 ms uncapped (237 registers, eight
-// warps); caps of 102 and 85 registers spill more and are slower.
+// Registers capped at 128 (four blocks, 16 warps per SM).  Bound by FP32 issue:
+// 1,530 warp instructions per 32 track-layers, 65% of the issue slots (500,000
+// tracks of 10 layers: 0.355 ms on the 6x6 covariance, 0.29 ms now; 1.56 KB
+// per track at the copy bandwidth would take 0.115 ms).
 __global__ void __launch_bounds__(128, 4) smooth_kernel(const FitGeom g, const Routing rt, const SmoothIO io)
 {
     extern __shared__ float slots[];
@@ -123,286 +55,259 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const FitGeom g, const R
     const int L = g.L;
     float *slot = slots + threadIdx.x;
     const int stride = blockDim.x;
-    auto ost = [&](int l, int i) -> float & { return io.out_state[((int64_t)l * 6 + i) * T + t]; };
-    auto ocv = [&](int l, int i) -> float & { return io.out_cov[((int64_t)l * 21 + i) * T + t]; };
+    float *os = io.out_state + t, *oc = io.out_cov + t;  // layer l, component i: os[(6 l + i) T], oc[(21 l + i) T]
 
     // ---- forward: the fit, keeping every layer
-    float x[6], c[21];
-    bool finite = true;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        x[i] = __ldcs(io.seed_state + i * T + t);
-        finite = finite && isfinite(x[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 21; ++i) {
-        c[i] = __ldcs(io.seed_cov + i * T + t);
-        finite = finite && isfinite(c[i]);
-    }
     const float qkb = (float)io.charge[t] * g.qk;
     const uint32_t mask = io.hit_mask[t];
-    uint32_t flags = finite ? 0u : (uint32_t)KF_FLAG_NAN_INPUT;
+    float m[3] = {0, 0, 0}, v[6] = {0, 0, 0, 0, 0, 0};
+    const float *hp = io.hit_pos + t, *hc = io.hit_cov + t;
+    auto load_hit = [&](float mm[3], float vv[6]) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) mm[i] = __ldcs(hp + i * T);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) vv[i] = __ldcs(hc + i * T);
+    };
+    Local p{};
+    float c[15], pn;
+    uint32_t flags;
+    bool go;
+    {
+        float x6[6], c6[21];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) x6[i] = __ldcs(io.seed_state + i * T + t);
+#pragma unroll
+        for (int i = 0; i < 21; ++i) c6[i] = __ldcs(io.seed_cov + i * T + t);
+        if (mask & 1u) load_hit(m, v);
+        flags = (all_finite<6>(x6) && all_finite<21>(c6)) ? 0u : (uint32_t)KF_FLAG_NAN_INPUT;
+        if (!flags) flags = enter_local(x6, c6, qkb, g.r[0], g.inv_r[0], g.z_half, p, c, pn);
+        go = flags == 0u;
+    }
     int K = 0;
-    for (int l = 0; l < L && finite; ++l) {
-        float xn[6], s;
-        Jac J;
-        if (!propagate(x, qkb, g.r[l], xn, s, &J)) {
-            flags |= KF_FLAG_UNREACHABLE;
-            break;
-        }
-        if (fabsf(xn[2]) > g.z_half) {
-            flags |= KF_FLAG_LEFT_BARREL;
-            break;
-        }
-        const float nx1 = xn[0] * g.inv_r[l], ny1 = xn[1] * g.inv_r[l];
-        transport(J, c);
-        {
-            float q6[6];
-            scattering_q6(xn, g.inv_r[l], g.xx0[l], q6);
-            c[pk(3, 3)] += q6[0];
-            c[pk(4, 3)] += q6[1];
-            c[pk(4, 4)] += q6[2];
-            c[pk(5, 3)] += q6[3];
-            c[pk(5, 4)] += q6[4];
-            c[pk(5, 5)] += q6[5];
-        }
-#pragma unroll
-        for (int i = 0; i < 6; ++i) x[i] = xn[i];
-        if ((mask >> l) & 1u) {
-            float m[3], v[6], d = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) m[i] = __ldcs(io.hit_pos + ((int64_t)l * 3 + i) * T + t);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) v[i] = __ldcs(io.hit_cov + ((int64_t)l * 6 + i) * T + t);
-            bool hit_ok = true;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) hit_ok = hit_ok && isfinite(m[i]);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) hit_ok = hit_ok && isfinite(v[i]);
-            if (!hit_ok) {
-                flags |= KF_FLAG_NAN_INPUT;
-                finite = false;
+    for (int l = 0; l < L && go; ++l) {
+        const bool has = (mask >> l) & 1u, has_next = l + 1 < L && ((mask >> (l + 1)) & 1u);
+        float mn[3], vn[6];
+        hp += 3 * T;
+        hc += 6 * T;
+        if (has_next) load_hit(mn, vn);
+        if (l > 0) {
+            LocalJac J;
+            const uint32_t stop = step_local(p, qkb, g.r[l], g.inv_r[l], g.z_half, J, pn);
+            if (stop) {
+                flags |= stop;
                 break;
             }
-            const int st = update(x, c, m, v, rt, &d, slot, stride);
+            transport_local(J, c);
+        }
+        scatter_local(p, noise_local(p, pn, g.xx0[l]), c);
+        if (has) {
+            float d = 0.0f;
+            const int st = update_local(p, c, m, v, rt, &d, slot, stride);
+            // a non-finite hit value fails the update or makes d non-finite
+            if ((st == 1 || !isfinite(d)) && (!all_finite<3>(m) || !all_finite<6>(v))) {
+                flags |= KF_FLAG_NAN_INPUT;
+                K = 0;
+                break;
+            }
             if (st == 1) flags |= KF_FLAG_INVERSION_FAILED;
             if (st >= 2) flags |= KF_FLAG_FP64_PATH;
             if (st == 3) flags |= KF_FLAG_PSD_REPAIRED;
         }
-        // filtered: state, local covariance and its frame into the outputs
-        {
-            float cl[15];
-            local_of(c, nx1, ny1, cl);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) ost(l, i) = x[i];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) ocv(l, i) = cl[i];
-            ocv(l, 15) = nx1;
-            ocv(l, 16) = ny1;
-        }
         K = l + 1;
+        if (K < L) {  // filtered: the coordinates, their covariance and frames
+            const float x[6] = {p.x, p.y, p.z, p.q1, p.q2, p.pz};
+#pragma unroll
+            for (int i = 0; i < 6; ++i) os[(int64_t)(6 * l + i) * T] = x[i];
+#pragma unroll
+            for (int i = 0; i < 15; ++i) oc[(int64_t)(21 * l + i) * T] = c[i];
+            oc[(int64_t)(21 * l + 15) * T] = p.nx;
+            oc[(int64_t)(21 * l + 16) * T] = p.ny;
+            oc[(int64_t)(21 * l + 17) * T] = p.f0;
+            oc[(int64_t)(21 * l + 18) * T] = p.f1;
+        }
+        if (has_next) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) m[i] = mn[i];
+#pragma unroll
+            for (int i = 0; i < 6; ++i) v[i] = vn[i];
+        }
     }
-    if (!finite) K = 0;
     io.out_reached[t] = (int16_t)K;
 
-    // ---- backward
-    float xs[6], cs[15], nx = 1.0f, ny = 0.0f;  // smoothed at layer l+1 and its frame
-    if (K > 0) {
+    // ---- backward: p, c are the smoothed estimate of layer l + 1
+    auto write = [&](int l) {
+        float x6[6], c6[21];
+        leave_local(p, c, x6, c6);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) xs[i] = ost(K - 1, i);
+        for (int i = 0; i < 6; ++i) __stcs(os + (int64_t)(6 * l + i) * T, x6[i]);
 #pragma unroll
-        for (int i = 0; i < 15; ++i) cs[i] = ocv(K - 1, i);
-        nx = ocv(K - 1, 15);
-        ny = ocv(K - 1, 16);
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j <= i; ++j) ocv(K - 1, pk(i, j)) = cart_of(cs, nx, ny, i, j);
-    }
+        for (int i = 0; i < 21; ++i) __stcs(oc + (int64_t)(21 * l + i) * T, c6[i]);
+    };
+    if (K > 0) write(K - 1);
     for (int l = K - 2; l >= 0; --l) {
-        float xf[6], cf[15], cp[15], xp[6], gj[13], q6[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) xf[i] = __ldlu(&ost(l, i));  // the filtered estimate's last read
-#pragma unroll
-        for (int i = 0; i < 15; ++i) cf[i] = __ldlu(&ocv(l, i));
-        const float nxl = __ldlu(&ocv(l, 15)), nyl = __ldlu(&ocv(l, 16));
+        Local f;
+        float cf[15];
         {
-            // the prediction of layer l+1 from the filtered estimate of layer
-            // l, as the forward pass made it (the track reached layer l+1 there)
-            float c21[21];
+            const float *a = os + (int64_t)(6 * l) * T, *b = oc + (int64_t)(21 * l) * T;
+            // the filtered estimate's last read
+            f = Local{__ldlu(a),         __ldlu(a + T),      __ldlu(a + 2 * T),  __ldlu(a + 3 * T),  __ldlu(a + 4 * T),
+                      __ldlu(a + 5 * T), __ldlu(b + 17 * T), __ldlu(b + 18 * T), __ldlu(b + 15 * T), __ldlu(b + 16 * T)};
 #pragma unroll
-            for (int i = 0; i < 6; ++i)
-#pragma unroll
-                for (int j = 0; j <= i; ++j) c21[pk(i, j)] = cart_of(cf, nxl, nyl, i, j);
-            float sd;
-            Jac J;
-            propagate(xf, qkb, g.r[l + 1], xp, sd, &J);
-            const float nx1 = xp[0] * g.inv_r[l + 1], ny1 = xp[1] * g.inv_r[l + 1];
-            local_jacobian(J, nxl, nyl, nx1, ny1, gj);
-            transport(J, c21);
-            scattering_q6(xp, g.inv_r[l + 1], g.xx0[l + 1], q6);
-            c21[pk(3, 3)] += q6[0];
-            c21[pk(4, 3)] += q6[1];
-            c21[pk(4, 4)] += q6[2];
-            c21[pk(5, 3)] += q6[3];
-            c21[pk(5, 4)] += q6[4];
-            c21[pk(5, 5)] += q6[5];
-            local_of(c21, nx1, ny1, cp);
+            for (int i = 0; i < 15; ++i) cf[i] = __ldlu(b + i * T);
         }
-        // Cholesky of Cp scaled to unit diagonal: S = D Cp D, D = diag(Cp)^-1/2
-        float dsc[5], Lc[15];
-        bool ok = true;
+        // the prediction of layer l+1, as the forward pass made it (the track
+        // reached layer l+1 there)
+        Local q = f;
+        LocalJac J, B;
+        float cp[15], cn0;
+        step_local(q, qkb, g.r[l + 1], g.inv_r[l + 1], INFINITY, J, pn, &B, &cn0);
 #pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            ok = ok && cp[pk(i, i)] > 0.0f;
-            dsc[i] = rsqrtf(cp[pk(i, i)]);
-        }
+        for (int i = 0; i < 15; ++i) cp[i] = cf[i];
+        transport_local(J, cp);
+        const float t2 = noise_local(q, pn, g.xx0[l + 1]);
+        scatter_local(q, t2, cp);
+        float D[15];
+#pragma unroll
+        for (int i = 0; i < 15; ++i) D[i] = c[i] - cp[i];
+        // det G, the ratio of the momentum's normal components (a step keeps the
+        // phase-space flux through the layers), must not vanish; pn = pT |cn|
+        bool ok = cn0 * cn0 * fmaf(f.q1, f.q1, f.q2 * f.q2) > 1e-12f * pn * pn;
+        // Cp = Lc diag(dg) Lc^T (unit lower Lc, kept in cp's strict triangle)
+        float idg[5];
 #pragma unroll
         for (int j = 0; j < 5; ++j) {
-            float djj = cp[pk(j, j)] * dsc[j] * dsc[j];
+            float dj = cp[pk(j, j)];
 #pragma unroll
-            for (int k = 0; k < j; ++k) djj = fmaf(-Lc[pk(j, k)], Lc[pk(j, k)], djj);
-            ok = ok && djj > 0.0f;
-            const float ljj = sqrtf(fmaxf(djj, 1e-30f)), il = 1.0f / ljj;
-            Lc[pk(j, j)] = ljj;
+            for (int k = 0; k < j; ++k) dj = fmaf(-cp[pk(j, k)] * cp[pk(j, k)], cp[pk(k, k)], dj);
+            ok = ok && dj > 0.0f;
+            cp[pk(j, j)] = dj;
+            idg[j] = __fdividef(1.0f, dj);
 #pragma unroll
             for (int i = j + 1; i < 5; ++i) {
-                float sij = cp[pk(i, j)] * dsc[i] * dsc[j];
+                float u = cp[pk(i, j)];
 #pragma unroll
-                for (int k = 0; k < j; ++k) sij = fmaf(-Lc[pk(i, k)], Lc[pk(j, k)], sij);
-                Lc[pk(i, j)] = sij * il;
+                for (int k = 0; k < j; ++k) u = fmaf(-cp[pk(i, k)] * cp[pk(k, k)], cp[pk(j, k)], u);
+                cp[pk(i, j)] = u * idg[j];
             }
         }
-        // M^-1 of the transverse block (t, px, py) by adjugate
-        const float m00 = gj[0], m01 = gj[1], m02 = gj[2], m10 = gj[3], m11 = gj[4], m12 = gj[5];
-        const float m20 = gj[6], m21 = gj[7], m22 = gj[8];
-        const float a00 = m11 * m22 - m12 * m21, a01 = m02 * m21 - m01 * m22, a02 = m01 * m12 - m02 * m11;
-        const float a10 = m12 * m20 - m10 * m22, a11 = m00 * m22 - m02 * m20, a12 = m02 * m10 - m00 * m12;
-        const float a20 = m10 * m21 - m11 * m20, a21 = m01 * m20 - m00 * m21, a22 = m00 * m11 - m01 * m10;
-        const float detm = m00 * a00 + m01 * a10 + m02 * a20;
-        ok = ok && fabsf(detm) > 1e-6f;
         if (!ok) {  // no smoothing across this layer: keep the filtered estimate
             flags |= KF_FLAG_INVERSION_FAILED;
+            p = f;
 #pragma unroll
-            for (int i = 0; i < 6; ++i) xs[i] = xf[i];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) cs[i] = cf[i];
+            for (int i = 0; i < 15; ++i) c[i] = cf[i];
         } else {
-            const float idet = 1.0f / detm;
-            // G^-1 (5x5): (t, px, py) = Mi (t', px', py'); pz = pz';
-            // z = z' - (mz Mi) . (t', px', py') - jp pz'
-            float Gi[5][5];
-#pragma unroll
-            for (int i = 0; i < 5; ++i)
-#pragma unroll
-                for (int j = 0; j < 5; ++j) Gi[i][j] = 0.0f;
-            const float Mi[3][3] = {{a00 * idet, a01 * idet, a02 * idet},
-                                    {a10 * idet, a11 * idet, a12 * idet},
-                                    {a20 * idet, a21 * idet, a22 * idet}};
-            constexpr int Q3[3] = {0, 2, 3};
-#pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int c3 = 0; c3 < 3; ++c3) Gi[Q3[r]][Q3[c3]] = Mi[r][c3];
-#pragma unroll
-            for (int c3 = 0; c3 < 3; ++c3)
-                Gi[1][Q3[c3]] = -fmaf(gj[9], Mi[0][c3], fmaf(gj[10], Mi[1][c3], gj[11] * Mi[2][c3]));
-            Gi[1][1] = 1.0f;
-            Gi[1][4] = -gj[12];
-            Gi[4][4] = 1.0f;
-            // W = Cp^-1 Q (only Q's momentum columns are non-zero): three
-            // solves with the scaled factor, Cp^-1 b = D S^-1 D b
-            float W[5][3];
+            // K = Q Cp^-1, rows q1, q2, pz: one solve per row
+            const float tu = -t2 * q.q1, tv = -t2 * q.q2;
+            const float q6[6] = {t2 * fmaf(q.q2, q.q2, q.pz * q.pz), tu * q.q2, t2 * fmaf(q.q1, q.q1, q.pz * q.pz),
+                                 tu * q.pz, tv * q.pz, t2 * fmaf(q.q1, q.q1, q.q2 * q.q2)};
+            float Kr[3][5];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                // column 2 + k of the local Q (rows px, py, pz; packed q6 is
-                // (px,px) (py,px) (py,py) (pz,px) (pz,py) (pz,pz))
-                const float b5[5] = {0.0f, 0.0f, q6[k == 0 ? 0 : k == 1 ? 1 : 3], q6[k == 0 ? 1 : k == 1 ? 2 : 4],
-                                     q6[k == 0 ? 3 : k == 1 ? 4 : 5]};
-                float y[5];
+                float w[5] = {0.0f, 0.0f, q6[k == 0 ? 0 : k == 1 ? 1 : 3], q6[k == 0 ? 1 : k == 1 ? 2 : 4],
+                              q6[k == 0 ? 3 : k == 1 ? 4 : 5]};
 #pragma unroll
-                for (int i = 0; i < 5; ++i) {
-                    float acc = dsc[i] * b5[i];
+                for (int i = 3; i < 5; ++i)
 #pragma unroll
-                    for (int j = 0; j < i; ++j) acc = fmaf(-Lc[pk(i, j)], y[j], acc);
-                    y[i] = acc / Lc[pk(i, i)];
-                }
+                    for (int j = 2; j < i; ++j) w[i] = fmaf(-cp[pk(i, j)], w[j], w[i]);
 #pragma unroll
-                for (int i = 4; i >= 0; --i) {
-                    float acc = y[i];
+                for (int i = 2; i < 5; ++i) w[i] *= idg[i];
 #pragma unroll
-                    for (int j = i + 1; j < 5; ++j) acc = fmaf(-Lc[pk(j, i)], y[j], acc);
-                    y[i] = acc / Lc[pk(i, i)];
-                }
+                for (int i = 3; i >= 0; --i)
 #pragma unroll
-                for (int i = 0; i < 5; ++i) W[i][k] = dsc[i] * y[i];
+                    for (int j = i + 1; j < 5; ++j) w[i] = fmaf(-cp[pk(j, i)], w[j], w[i]);
+#pragma unroll
+                for (int i = 0; i < 5; ++i) Kr[k][i] = w[i];
             }
-            // A = G^-1 (I - Q Cp^-1), (Q Cp^-1)[2 + k][j] = W[j][k]; kept as At = A^T
-            float At[5][5];
+            // state: d = (I - K) (xs' - xp), then the step back
+            const float e0 = p.x - q.x, e1 = p.y - q.y;
+            const float dl[5] = {fmaf(q.nx, e1, -q.ny * e0), p.z - q.z, p.q1 - q.q1, p.q2 - q.q2, p.pz - q.pz};
+            float d[5] = {dl[0], dl[1], dl[2], dl[3], dl[4]};
 #pragma unroll
-            for (int i = 0; i < 5; ++i)
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int j = 0; j < 5; ++j) d[2 + k] = fmaf(-Kr[k][j], dl[j], d[2 + k]);
+            const float dt = fmaf(B.A0, d[0], fmaf(B.A1, d[2], B.A2 * d[3]));
+            const float la = fmaf(B.L0, d[0], fmaf(B.L1, d[2], B.L2 * d[3]));
+            // covariance: (I - K) (Cs' - Cp) (I - K)^T, then the step back.
+            // Where layer l + 1 is crossed almost along its surface, t at layer
+            // l is a small difference of large terms: its row is taken from
+            // A's row a as a whole, u = D a (from (I - K) D (I - K)^T, whose
+            // roundings B's entries scale, the t variance of a looper came out
+            // 4% off).
+            float ct[5];
+            {
+                float a[5], b[5], u[5];  // t = a . delta, lambda = b . delta
 #pragma unroll
                 for (int j = 0; j < 5; ++j) {
-                    float acc = Gi[i][j];
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) acc = fmaf(-Gi[i][2 + k], W[j][k], acc);
-                    At[j][i] = acc;
+                    a[j] = fmaf(-B.A1, Kr[0][j], fmaf(-B.A2, Kr[1][j], j == 0 ? B.A0 : j == 2 ? B.A1 : j == 3 ? B.A2 : 0.0f));
+                    b[j] = fmaf(-B.L1, Kr[0][j], fmaf(-B.L2, Kr[1][j], j == 0 ? B.L0 : j == 2 ? B.L1 : j == 3 ? B.L2 : 0.0f));
                 }
-            // state: delta = local(n_{l+1}) of (xs - xp)
-            const float d0 = xs[0] - xp[0], d1 = xs[1] - xp[1];
-            const float dl[5] = {fmaf(nx, d1, -ny * d0), xs[2] - xp[2], xs[3] - xp[3], xs[4] - xp[4],
-                                 xs[5] - xp[5]};
-            float e[5];
+                float ul = 0.0f;
+                ct[0] = 0.0f;
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                float acc = 0.0f;
+                for (int i = 0; i < 5; ++i) {
+                    u[i] = 0.0f;
 #pragma unroll
-                for (int k = 0; k < 5; ++k) acc = fmaf(At[k][i], dl[k], acc);
-                e[i] = acc;
+                    for (int j = 0; j < 5; ++j) u[i] = fmaf(a[j], D[pk(i, j)], u[i]);
+                    ct[0] = fmaf(a[i], u[i], ct[0]);
+                    ul = fmaf(b[i], u[i], ul);
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    ct[2 + k] = u[2 + k];
+#pragma unroll
+                    for (int i = 0; i < 5; ++i) ct[2 + k] = fmaf(-Kr[k][i], u[i], ct[2 + k]);
+                }
+                ct[1] = fmaf(B.jp, ct[4], fmaf(B.lz, ul, u[1]));
+                ct[2] = fmaf(B.W1, ul, ct[2]);
+                ct[3] = fmaf(B.W2, ul, ct[3]);
             }
-            xs[0] = fmaf(-nyl, e[0], xf[0]);
-            xs[1] = fmaf(nxl, e[0], xf[1]);
+            float E[3][5];
 #pragma unroll
-            for (int i = 1; i < 5; ++i) xs[i + 1] = xf[i + 1] + e[i];
-            // covariance: Cs = Cf + A (Cs' - Cp) A^T
-            float D5[15];
-#pragma unroll
-            for (int i = 0; i < 15; ++i) D5[i] = cs[i] - cp[i];
-            float AD[5][5];  // A D
-#pragma unroll
-            for (int i = 0; i < 5; ++i)
+            for (int k = 0; k < 3; ++k)
 #pragma unroll
                 for (int j = 0; j < 5; ++j) {
                     float acc = 0.0f;
 #pragma unroll
-                    for (int k = 0; k < 5; ++k) acc = fmaf(At[k][i], D5[pk(k, j)], acc);
-                    AD[i][j] = acc;
+                    for (int i = 0; i < 5; ++i) acc = fmaf(Kr[k][i], D[pk(i, j)], acc);
+                    E[k][j] = acc;
                 }
 #pragma unroll
-            for (int i = 0; i < 5; ++i)
+            for (int k = 0; k < 3; ++k) {
 #pragma unroll
-                for (int j = 0; j <= i; ++j) {
-                    float acc = cf[pk(i, j)];
+                for (int j = 0; j < 2; ++j) D[pk(2 + k, j)] -= E[k][j];
 #pragma unroll
-                    for (int k = 0; k < 5; ++k) acc = fmaf(AD[i][k], At[k][j], acc);
-                    cs[pk(i, j)] = acc;
+                for (int h = 0; h <= k; ++h) {
+                    float acc = D[pk(2 + k, 2 + h)] - E[k][2 + h] - E[h][2 + k];
+#pragma unroll
+                    for (int i = 0; i < 5; ++i) acc = fmaf(E[k][i], Kr[h][i], acc);
+                    D[pk(2 + k, 2 + h)] = acc;
                 }
+            }
+            transport_local(B, D);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) D[pk(i, 0)] = ct[i];
+            p = Local{fmaf(-f.ny, dt, f.x),
+                      fmaf(f.nx, dt, f.y),
+                      f.z + fmaf(B.jp, d[4], fmaf(B.lz, la, d[1])),
+                      f.q1 + fmaf(B.W1, la, d[2]),
+                      f.q2 + fmaf(B.W2, la, d[3]),
+                      f.pz + d[4],
+                      f.f0,
+                      f.f1,
+                      f.nx,
+                      f.ny};
+#pragma unroll
+            for (int i = 0; i < 15; ++i) c[i] = cf[i] + D[i];
         }
-        nx = nxl;
-        ny = nyl;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) __stcs(&ost(l, i), xs[i]);  // final: streamed out
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j <= i; ++j) __stcs(&ocv(l, pk(i, j)), cart_of(cs, nx, ny, i, j));
+        write(l);
     }
     // layers not reached (and every layer of a track with a non-finite input)
     for (int l = K; l < L; ++l) {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) ost(l, i) = NAN;
+        for (int i = 0; i < 6; ++i) os[(int64_t)(6 * l + i) * T] = NAN;
 #pragma unroll
-        for (int i = 0; i < 21; ++i) ocv(l, i) = NAN;
+        for (int i = 0; i < 21; ++i) oc[(int64_t)(21 * l + i) * T] = NAN;
     }
     io.out_flags[t] = flags;
 }
