@@ -75,7 +75,7 @@ typedef struct CUstream_st *kf_stream; /* a cudaStream_t; NULL is the legacy def
 #define KF_PRECISION_ROUTED 1 /* FP32, with ill-conditioned updates redone in FP64 */
 
 /* launch_mode */
-#define KF_LAUNCH_AUTO 0      /* one persistent launch over all events, graph-captured */
+#define KF_LAUNCH_AUTO 0      /* all events in one launch, and one for the tracks that need FP64 */
 #define KF_LAUNCH_PER_EVENT 1 /* one plain launch per event (needs event_offsets) */
 #define KF_LAUNCH_FLAT 2      /* one plain launch over all tracks */
 
@@ -105,9 +105,9 @@ typedef struct {
     /* launch shape (fit) */
     int launch_mode;         /* KF_LAUNCH_* */
     int tracks_per_block;    /* 0 = autotuned, else 32, 64, 128 or 256 */
-    int reg_cap;             /* registers per thread of the persistent fit: 0 = autotuned,
+    int reg_cap;             /* registers per thread of the fit: 0 = autotuned,
                                 -1 = uncapped, 168, 128, 96 or 80 */
-    int hit_prefetch;        /* layers of hits the persistent fit loads ahead of their
+    int hit_prefetch;        /* layers of hits the fit loads ahead of their
                                 update: 0 = autotuned, 1 = the next layer into registers,
                                 2 or 4 = through a ring in shared memory (cp.async) */
     /* building */
@@ -183,11 +183,11 @@ int kf_fit_tracks(kf_context *ctx, const kf_geometry *geom, int64_t n_tracks,
  * finds host-device transfers about half of the GPU build's wall time).
  *
  * chunk_tracks = 0 and every array page-locked memory the device can address
- * (cudaMallocHost, cudaHostAlloc, cudaHostRegister): one persistent fit
- * launch reads the inputs and writes the outputs where they are, over the
- * host link; nothing is staged.  Otherwise the batch is cut into chunks of
- * chunk_tracks tracks (0: 262,144); each chunk is copied in, fitted (the
- * persistent fit, all of the chunk's events in one launch) and copied out on
+ * (cudaMallocHost, cudaHostAlloc, cudaHostRegister): the fit
+ * reads the inputs and writes the outputs where they are, over the host
+ * link; nothing is staged.  Otherwise the batch is cut into chunks of
+ * chunk_tracks tracks (0: 262,144); each chunk is copied in, fitted (all of
+ * the chunk's events in one launch) and copied out on
  * one of three internal streams, so the transfers of one chunk overlap the
  * fit of another.
  *
@@ -506,7 +506,7 @@ int kf_smooth_tracks(kf_context *ctx, const kf_geometry *geom, int64_t n_tracks,
 int kf_transport_batch(kf_context *ctx, int64_t n, const float *J, float *C, kf_stream stream);
 
 /*
- * Launch shape the autotuner picked for the persistent fit of n_layers layers
+ * Launch shape the autotuner picked for the fit of n_layers layers
  * and a batch of n_tracks' size class (powers of two), once a KF_LAUNCH_AUTO
  * fit of that class has run on ctx.  Writes tracks per block, the register
  * cap per thread (-1: uncapped) and the hit prefetch depth (kf_options).
@@ -523,24 +523,21 @@ int kf_fit_tuned_shape(kf_context *ctx, int n_layers, int64_t n_tracks, int *tra
  * Callers that work inside a device-memory pool they do not own, loops that
  * must not touch the allocator after start-up, or hosts that forbid
  * allocation while their own work is in flight can call this instead.  It
- * runs the same persistent fit kernel (same steps, inputs, outputs and flags
- * as kf_fit_tracks, all events in one launch) and allocates nothing: the
- * kernel's only scratch, the 4-byte counter from which its warps claim
- * 32-track units, is a fixed array in the library's device memory that every
- * GPU loading the library holds until the process exits.
+ * runs the same fit kernels (same steps, inputs, outputs and flags
+ * as kf_fit_tracks, all events in one launch and the tracks that need FP64 in
+ * another) and allocates nothing: the kernels' only scratch, two 4-byte
+ * counters, is a fixed array in the library's device memory that every GPU
+ * loading the library holds until the process exits.
  *
  *   - Runs on the current CUDA device.  The first call on a device looks up
  *     that array's device address once (cudaGetSymbolAddress); make that
  *     first call before any stream capture.
- *   - Each call clears the counter on `stream` before its launch.  All calls
- *     on a device share the counter, so calls whose work overlaps on the GPU
+ *   - The counters read 0 between calls: the second launch clears them.  All
+ *     calls on a device share them, so calls whose work overlaps on the GPU
  *     (different streams, not ordered) race and give wrong results: order
  *     them on one stream or synchronise.
  *   - n_tracks must be at most KF_NOALLOC_MAX_TRACKS (2^36, the limit of
- *     kf_fit_tracks too); larger batches return KF_ERR_TOO_LARGE, and so does
- *     a launch that would hold more than 16,384 resident warps (the 32-bit
- *     counter must not wrap while every warp makes its last claim; a GB300
- *     holds at most 152 x 64 = 9,728).
+ *kf_fit_tracks too); larger batches return KF_ERR_TOO_LARGE.
  *   - No tuning runs.  The shape is opt->tracks_per_block, opt->reg_cap and
  *     opt->hit_prefetch where set, else 64 tracks per block, no register cap
  *     and the register prefetch (depth 1).  Only the (block, cap, depth)
@@ -551,8 +548,7 @@ int kf_fit_tuned_shape(kf_context *ctx, int n_layers, int64_t n_tracks, int *tra
  *     returns KF_ERR_ARG.  opt->launch_mode is ignored.  There is no context,
  *     so failures are reported by the return code only: KF_ERR_ARG (a bad
  *     argument or an uncompiled shape), KF_ERR_TOO_LARGE, KF_ERR_CUDA (a CUDA
- *     call failed, including the shape's shared-memory opt-in or occupancy
- *     query).
+ *     call failed, including the shape's shared-memory opt-in).
  */
 #define KF_NOALLOC_MAX_TRACKS (68719476736LL)
 int kf_fit_tracks_noalloc(const kf_geometry *geom, int64_t n_tracks, const float *seed_state,

@@ -1,6 +1,5 @@
 // C interface (include/kf.h): argument checks, launch-shape selection (an
-// autotuner over tracks per block), CUDA-graph capture of the persistent fit
-// launch, and the context that owns scratch memory.
+// autotuner over tracks per block), and the context that owns scratch memory.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -18,32 +17,13 @@
 
 using namespace kf;
 
-namespace {
-
-struct GraphEntry {
-    FitGeom g;
-    Routing rt;
-    FitIO io;
-    FitShape shape;
-    int grid;
-    cudaGraphExec_t exec;
-    uint64_t last_use;
-};
-
-bool same_bytes(const void *a, const void *b, size_t n) { return std::memcmp(a, b, n) == 0; }
-
-}  // namespace
-
 struct kf_context {
     int device = 0;
     int sm_count = 0;
-    unsigned *d_counter = nullptr;  // persistent-kernel work counter
-    cudaStream_t capture_stream = nullptr;
+    unsigned *d_work = nullptr;  // the fit's counters (kFitWorkBytes), 0 between fits
     std::string err;
     // (L, log2 size, precision, fixed block, fixed cap, fixed depth) -> shape
     std::map<std::tuple<int, int, int, int, int, int>, kf::FitShape> tuned;
-    std::vector<GraphEntry> graphs;
-    uint64_t clock = 0;
     kf::BuildState *build = nullptr;
     kf::MlpState *mlp = nullptr;
     kf::HostPipe *host = nullptr;
@@ -186,12 +166,12 @@ int kf_context_create(kf_context **out, int device)
     kf_context *ctx = new kf_context;
     ctx->device = device;
     ctx->sm_count = prop.multiProcessorCount;
-    if (cudaMalloc(&ctx->d_counter, 256) != cudaSuccess) {
+    if (cudaMalloc(&ctx->d_work, kFitWorkBytes) != cudaSuccess) {
         delete ctx;
         return KF_ERR_NOMEM;
     }
-    if (cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaFree(ctx->d_counter);
+    if (cudaMemset(ctx->d_work, 0, kFitWorkBytes) != cudaSuccess) {
+        cudaFree(ctx->d_work);
         delete ctx;
         return KF_ERR_CUDA;
     }
@@ -204,14 +184,12 @@ void kf_context_destroy(kf_context *ctx)
     if (!ctx) return;
     DeviceGuard dg(ctx->device);
     cudaDeviceSynchronize();
-    for (auto &e : ctx->graphs) cudaGraphExecDestroy(e.exec);
     kf::destroy_build_state(ctx->build);
     kf::destroy_mlp_state(ctx->mlp);
     kf::destroy_host_state(ctx->host);
     kf::destroy_smooth_state(ctx->smooth);
     kf::destroy_seed_state(ctx->seed);
-    if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
-    cudaFree(ctx->d_counter);
+    cudaFree(ctx->d_work);
     delete ctx;
 }
 
@@ -228,59 +206,21 @@ int size_class(int64_t n)
     return c;
 }
 
-// Enqueue the persistent fit: counter reset + kernel, replayed from a cached
-// CUDA graph when this exact launch was captured before.
-cudaError_t enqueue_persistent(kf_context *ctx, const FitGeom &g, const Routing &rt, const FitIO &io,
-                               const FitShape &sh, cudaStream_t stream, bool use_graph)
+// Routed fits of fewer tracks than this run in one launch, warps of 32 tracks
+// with the FP64 update in line, and are not tuned: the launch for the tracks
+// put off costs the host 3 us (19.7 against 16.4 us a call at 1,000 tracks,
+// whose kernel takes 8.7 us either way), and with at most two warps on an SM
+// they hardly wait for each other's FP64 updates.  With one track in eight in
+// FP64 the lines cross between 10,000 tracks (103 us in line, 121 put off) and
+// 20,000 (134 and 123).  A power of two, as the tuner's size classes.
+constexpr int64_t kOneLaunchTracks = 8192;
+
+cudaError_t enqueue_fit(kf_context *ctx, const FitGeom &g, const Routing &rt, const FitIO &io, const FitShape &sh,
+                        cudaStream_t stream)
 {
-    const int block = sh.block;
-    const int per_sm = persistent_blocks_per_sm(block, sh.cap, sh.depth);
-    if (per_sm <= 0) return cudaErrorInvalidConfiguration;
-    const int64_t units = (io.T + 31) / 32;
-    const int64_t want = (units * 32 + block - 1) / block;
-    const int grid = (int)std::min<int64_t>((int64_t)ctx->sm_count * per_sm, std::max<int64_t>(want, 1));
-    cudaStreamCaptureStatus capst = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(stream, &capst);
-    if (!use_graph || capst != cudaStreamCaptureStatusNone) {
-        cudaError_t e = cudaMemsetAsync(ctx->d_counter, 0, sizeof(unsigned), stream);
-        if (e != cudaSuccess) return e;
-        return launch_fit_persistent(g, rt, io, block, sh.cap, sh.depth, grid, ctx->d_counter, stream);
-    }
-    for (auto &e : ctx->graphs) {
-        if (e.shape.block == block && e.shape.cap == sh.cap && e.shape.depth == sh.depth && e.grid == grid &&
-            same_bytes(&e.g, &g, sizeof g) &&
-            same_bytes(&e.rt, &rt, sizeof rt) && same_bytes(&e.io, &io, sizeof io)) {
-            e.last_use = ++ctx->clock;
-            return cudaGraphLaunch(e.exec, stream);
-        }
-    }
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return e;
-    cudaError_t e1 = cudaMemsetAsync(ctx->d_counter, 0, sizeof(unsigned), ctx->capture_stream);
-    cudaError_t e2 = e1 == cudaSuccess
-                         ? launch_fit_persistent(g, rt, io, block, sh.cap, sh.depth, grid, ctx->d_counter,
-                                                 ctx->capture_stream)
-                         : e1;
-    e = cudaStreamEndCapture(ctx->capture_stream, &graph);
-    if (e2 != cudaSuccess) e = e2;
-    if (e != cudaSuccess) {
-        if (graph) cudaGraphDestroy(graph);
-        return e;
-    }
-    cudaGraphExec_t exec = nullptr;
-    e = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) return e;
-    if (ctx->graphs.size() >= 16) {  // evict the least recently used
-        size_t lru = 0;
-        for (size_t i = 1; i < ctx->graphs.size(); ++i)
-            if (ctx->graphs[i].last_use < ctx->graphs[lru].last_use) lru = i;
-        cudaGraphExecDestroy(ctx->graphs[lru].exec);
-        ctx->graphs.erase(ctx->graphs.begin() + lru);
-    }
-    ctx->graphs.push_back(GraphEntry{g, rt, io, sh, grid, exec, ++ctx->clock});
-    return cudaGraphLaunch(exec, stream);
+    const int ok = fit_shape_usable(sh.block, sh.cap, sh.depth);
+    if (ok <= 0) return cudaErrorInvalidConfiguration;
+    return launch_fit_tuned(g, rt, io, sh.block, sh.cap, sh.depth, ctx->sm_count, ctx->d_work, stream);
 }
 
 // Time every compiled (tracks per block, register cap, hit prefetch depth)
@@ -299,7 +239,7 @@ FitShape tune_shape(kf_context *ctx, const FitGeom &g, const Routing &rt, const 
     int n = 0;
     {
         int all_b[64], all_c[64], all_d[64];
-        const int m = persistent_shapes(all_b, all_c, all_d, 64);
+        const int m = fit_shapes(all_b, all_c, all_d, 64);
         for (int i = 0; i < m; ++i)
             if ((!fixed.block || all_b[i] == fixed.block) &&
                 (!fixed.cap || all_c[i] == (fixed.cap < 0 ? 0 : fixed.cap)) &&
@@ -317,9 +257,9 @@ FitShape tune_shape(kf_context *ctx, const FitGeom &g, const Routing &rt, const 
     FitShape best = cand[0];
     float best_ms = 1e30f;
     for (int i = 0; i < n; ++i) {
-        if (enqueue_persistent(ctx, g, rt, io, cand[i], stream, false) != cudaSuccess) continue;
+        if (enqueue_fit(ctx, g, rt, io, cand[i], stream) != cudaSuccess) continue;
         cudaEventRecord(a, stream);
-        for (int rep = 0; rep < 3; ++rep) enqueue_persistent(ctx, g, rt, io, cand[i], stream, false);
+        for (int rep = 0; rep < 3; ++rep) enqueue_fit(ctx, g, rt, io, cand[i], stream);
         cudaEventRecord(b, stream);
         if (cudaEventSynchronize(b) != cudaSuccess) break;
         float ms = 0.0f;
@@ -389,10 +329,15 @@ int kf_fit_tracks(kf_context *ctx, const kf_geometry *geom, int64_t n_tracks, co
             e = launch_fit_plain(g, rt, io, event_offsets[ev], event_offsets[ev + 1], block ? block : 128, stream);
         break;
     default: {
+        if (rt.mode == 1 && n_tracks < kOneLaunchTracks && !block && !o.reg_cap && !o.hit_prefetch) {
+            e = launch_fit_plain(g, rt, io, 0, n_tracks, 32, stream);
+            ctx->tuned.emplace(std::make_tuple(g.L, size_class(n_tracks), rt.mode, 0, 0, 0), FitShape{32, 0, 1});
+            break;
+        }
         FitShape shape{block, o.reg_cap < 0 ? 0 : o.reg_cap, o.hit_prefetch};
         if (!block || !o.reg_cap || !o.hit_prefetch)
             shape = tune_shape(ctx, g, rt, io, stream, FitShape{block, o.reg_cap, o.hit_prefetch});
-        e = enqueue_persistent(ctx, g, rt, io, shape, stream, true);
+        e = enqueue_fit(ctx, g, rt, io, shape, stream);
     }
     }
     if (e != cudaSuccess) return cuda_error(ctx, e, "fit launch");

@@ -1,6 +1,7 @@
 // Kalman-filter track fit on sm_103a: one thread per track (Section 4.2),
 // state and packed local covariance (kf_math.cuh) in registers, structure-of-arrays inputs read
 // coalesced (Section 4.1: element (i, j) of consecutive tracks is contiguous).
+#include <algorithm>
 #include <mutex>
 #include <set>
 #include <utility>
@@ -12,8 +13,6 @@ namespace kf {
 
 namespace {
 
-constexpr uint32_t kStop = KF_FLAG_UNREACHABLE | KF_FLAG_LEFT_BARREL | KF_FLAG_NAN_INPUT;
-
 __device__ __forceinline__ void cp_async4(float *dst, const float *src)
 {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -23,8 +22,10 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Fit track t over every layer in order (the steps and stop rules are those of
-// kf_fit_tracks in kf.h).  Hits are loaded DEPTH layers ahead of their update:
+// Fit track base + off over every layer in order (the steps and stop rules are
+// those of kf_fit_tracks in kf.h).  base is the block's: the addresses of every
+// array are then a uniform pointer and the thread's offset.  Hits are loaded
+// DEPTH layers ahead of their update:
 // DEPTH = 1 into registers, through pointers advanced by one layer's stride;
 // DEPTH >= 2 by asynchronous copies (cp.async, one commit group per layer,
 // empty for a layer without a hit) into this thread's column of a ring of
@@ -32,111 +33,114 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // so that the loads in flight hold no registers.  A non-finite value in a
 // used hit makes the chi2 increment non-finite, or makes S fail its positive
 // definiteness test, so the hit is tested only then.
-template <int DEPTH>
-__device__ __forceinline__ void fit_track(const FitGeom &g, const Routing &rt, const FitIO &io, int64_t t,
+// DEFER: at the first update that needs extended precision the track is given
+// up and true returned (nothing is written).
+template <int DEPTH, bool DEFER, class OFF>
+__device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, const FitIO &io, int64_t base, OFF off,
                                           float *slot, int stride, float *ring = nullptr)
 {
     const int64_t T = io.T;
-    float sx[6], sc[21];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) sx[i] = __ldcs(io.seed_state + i * T + t);
-#pragma unroll
-    for (int i = 0; i < 21; ++i) sc[i] = __ldcs(io.seed_cov + i * T + t);
-    const float qkb = (float)io.charge[t] * g.qk;
-    const uint32_t mask = __ldcs(io.hit_mask + t);
-    uint32_t flags = (all_finite<6>(sx) && all_finite<21>(sc)) ? 0u : (uint32_t)KF_FLAG_NAN_INPUT;
-    float chi2 = 0.0f;
-    int nhits = 0;
-    const float *hp = io.hit_pos + t;  // layer l, component i: hp[(3 l + i) T]
-    const float *hc = io.hit_cov + t;
-    const int64_t T3 = 3 * T, T6 = 6 * T;
+    const float *seed_state = io.seed_state + base, *seed_cov = io.seed_cov + base;
+    const float *hp = io.hit_pos + base;  // layer l, component i: hp[(3 l + i) T + off]
+    const float *hc = io.hit_cov + base;
+    const uint32_t mask = __ldcs(io.hit_mask + base + off);
     float m[3] = {0, 0, 0}, v[6] = {0, 0, 0, 0, 0, 0};
     auto load_hit = [&](float mm[3], float vv[6]) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) mm[i] = __ldcs(hp + i * T);
+        for (int i = 0; i < 3; ++i) mm[i] = __ldcs(hp + i * T + off);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) vv[i] = __ldcs(hc + i * T);
+        for (int i = 0; i < 6; ++i) vv[i] = __ldcs(hc + i * T + off);
+        hp += 3 * T;
+        hc += 6 * T;
     };
     // DEPTH >= 2: layer l's hit goes to stage l % (DEPTH + 1); stage_in is the
     // stage of the next layer to issue, stage_out that of the next to use
     int stage_in = 0, stage_out = 0, l_in = 0;
     auto issue = [&]() {
         if (l_in < g.L && ((mask >> l_in) & 1u)) {
-            const float *p = io.hit_pos + (int64_t)(3 * l_in) * T + t;
-            const float *q = io.hit_cov + (int64_t)(6 * l_in) * T + t;
             float *st = ring + stage_in * 9 * stride;
 #pragma unroll
-            for (int i = 0; i < 3; ++i) cp_async4(st + i * stride, p + i * T);
+            for (int i = 0; i < 3; ++i) cp_async4(st + i * stride, hp + i * T + off);
 #pragma unroll
-            for (int i = 0; i < 6; ++i) cp_async4(st + (3 + i) * stride, q + i * T);
+            for (int i = 0; i < 6; ++i) cp_async4(st + (3 + i) * stride, hc + i * T + off);
         }
         cp_async_commit();
         ++l_in;
+        hp += 3 * T;
+        hc += 6 * T;
         stage_in = stage_in == DEPTH ? 0 : stage_in + 1;
     };
+    float sx[6], sc[21];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) sx[i] = __ldcs(seed_state + i * T + off);
+#pragma unroll
+    for (int i = 0; i < 21; ++i) sc[i] = __ldcs(seed_cov + i * T + off);
+    const float qkb = (float)(io.charge + base)[off] * g.qk;
     if constexpr (DEPTH == 1) {
-        if (mask & 1u) load_hit(m, v);
+        load_hit(m, v);  // whether or not it is there, without waiting for the mask
     } else {
 #pragma unroll
         for (int k = 0; k < DEPTH; ++k) issue();
     }
+    uint32_t flags = (all_finite<6>(sx) && all_finite<21>(sc)) ? 0u : (uint32_t)KF_FLAG_NAN_INPUT;
+    float chi2 = 0.0f;
+    int nhits = 0;
     Local p;
     float c[15], pn;
-    bool at_seed = true;  // no layer reached
-    if (!flags) {
-        flags = enter_local(sx, sc, qkb, g.r[0], g.inv_r[0], g.z_half, p, c, pn);
-        at_seed = flags != 0u;
-    }
-    for (int l = 0; l < g.L && !(flags & kStop); ++l) {
-        const bool has = (mask >> l) & 1u;
-        const bool has_next = l + 1 < g.L && ((mask >> (l + 1)) & 1u);
-        float mn[3], vn[6];
-        if constexpr (DEPTH == 1) {
-            hp += T3;
-            hc += T6;
-            if (has_next) load_hit(mn, vn);
-        } else {
-            issue();                      // layer l + DEPTH
-            cp_async_wait<DEPTH>();       // layer l's group has landed
-            if (has) {
-                const float *st = ring + stage_out * 9 * stride;
+    bool deferred = false;
+    if (!flags) flags = enter_local(sx, sc, qkb, g.r[0], g.inv_r[0], g.z_half, p, c, pn);
+    const bool at_seed = flags != 0u;  // no layer reached
+    if (!at_seed) {
+        for (int l = 0; l < g.L; ++l) {
+            const bool has = (mask >> l) & 1u;
+            float mn[3] = {0, 0, 0}, vn[6] = {0, 0, 0, 0, 0, 0};
+            if constexpr (DEPTH == 1) {
+                if (l + 1 < g.L) load_hit(mn, vn);
+            } else {
+                issue();                 // layer l + DEPTH
+                cp_async_wait<DEPTH>();  // layer l's group has landed
+                if (has) {
+                    const float *st = ring + stage_out * 9 * stride;
 #pragma unroll
-                for (int i = 0; i < 3; ++i) m[i] = st[i * stride];
+                    for (int i = 0; i < 3; ++i) m[i] = st[i * stride];
 #pragma unroll
-                for (int i = 0; i < 6; ++i) v[i] = st[(3 + i) * stride];
+                    for (int i = 0; i < 6; ++i) v[i] = st[(3 + i) * stride];
+                }
+                stage_out = stage_out == DEPTH ? 0 : stage_out + 1;
             }
-            stage_out = stage_out == DEPTH ? 0 : stage_out + 1;
-        }
-        if (l > 0) {
-            LocalJac J;
-            const uint32_t stop = step_local(p, qkb, g.r[l], g.inv_r[l], g.z_half, J, pn);
-            if (stop) {
-                flags |= stop;
-                break;
-            }
-            transport_local(J, c);
-        }
-        scatter_local(p, noise_local(p, pn, g.xx0[l]), c);
-        if (has) {
-            float d = 0.0f;
-            const int st = update_local(p, c, m, v, rt, &d, slot, stride);
-            if (st == 1 || !isfinite(d)) {
-                if (!all_finite<3>(m) || !all_finite<6>(v)) {
-                    flags |= KF_FLAG_NAN_INPUT;
+            if (l > 0) {
+                LocalJac J;
+                const uint32_t stop = step_local(p, qkb, g.r[l], g.inv_r[l], g.z_half, J, pn);
+                if (stop) {
+                    flags |= stop;
                     break;
                 }
+                transport_local(J, c);
             }
-            if (st == 1) {
-                flags |= KF_FLAG_INVERSION_FAILED;
-            } else {
-                chi2 += d;
-                ++nhits;
-                if (st >= 2) flags |= KF_FLAG_FP64_PATH;
-                if (st == 3) flags |= KF_FLAG_PSD_REPAIRED;
+            scatter_local(p, noise_local(p, pn, g.xx0[l]), c);
+            if (has) {
+                float d = 0.0f;
+                const int st = update_local<DEFER>(p, c, m, v, rt, &d, slot, stride);
+                if (DEFER && st == 4) {
+                    deferred = true;
+                    break;
+                }
+                if (st == 1 || !isfinite(d)) {
+                    if (!all_finite<3>(m) || !all_finite<6>(v)) {
+                        flags |= KF_FLAG_NAN_INPUT;
+                        break;
+                    }
+                }
+                if (st == 1) {
+                    flags |= KF_FLAG_INVERSION_FAILED;
+                } else {
+                    chi2 += d;
+                    ++nhits;
+                    if (st >= 2) flags |= KF_FLAG_FP64_PATH;
+                    if (st == 3) flags |= KF_FLAG_PSD_REPAIRED;
+                }
             }
-        }
-        if constexpr (DEPTH == 1) {
-            if (has_next) {
+            if constexpr (DEPTH == 1) {
 #pragma unroll
                 for (int i = 0; i < 3; ++i) m[i] = mn[i];
 #pragma unroll
@@ -144,25 +148,28 @@ __device__ __forceinline__ void fit_track(const FitGeom &g, const Routing &rt, c
             }
         }
     }
-    if constexpr (DEPTH > 1) cp_async_wait<0>();  // no copy of this track may land in the next one's ring
+    if constexpr (DEPTH > 1) cp_async_wait<0>();
+    if (DEFER && deferred) return true;
     float x[6], c6[21];
     if (at_seed || (flags & KF_FLAG_NAN_INPUT)) {  // a track with bad input returns its seed
 #pragma unroll
-        for (int i = 0; i < 6; ++i) x[i] = io.seed_state[i * T + t];
+        for (int i = 0; i < 6; ++i) x[i] = seed_state[i * T + off];
 #pragma unroll
-        for (int i = 0; i < 21; ++i) c6[i] = io.seed_cov[i * T + t];
+        for (int i = 0; i < 21; ++i) c6[i] = seed_cov[i * T + off];
         chi2 = 0.0f;
         nhits = 0;
     } else {
         leave_local(p, c, x, c6);
     }
+    float *out_state = io.out_state + base, *out_cov = io.out_cov + base;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) __stcs(io.out_state + i * T + t, x[i]);
+    for (int i = 0; i < 6; ++i) __stcs(out_state + i * T + off, x[i]);
 #pragma unroll
-    for (int i = 0; i < 21; ++i) __stcs(io.out_cov + i * T + t, c6[i]);
-    __stcs(io.out_chi2 + t, chi2);
-    io.out_ndof[t] = (int16_t)(3 * nhits - 6);
-    io.out_flags[t] = flags;
+    for (int i = 0; i < 21; ++i) __stcs(out_cov + i * T + off, c6[i]);
+    __stcs(io.out_chi2 + base + off, chi2);
+    (io.out_ndof + base)[off] = (int16_t)(3 * nhits - 6);
+    (io.out_flags + base)[off] = flags;
+    return false;
 }
 
 // One thread per track over [t_begin, t_end).
@@ -171,34 +178,74 @@ __global__ void __launch_bounds__(256) fit_plain_kernel(const FitGeom g, const R
 {
     extern __shared__ float slots[];
     const int64_t t = t_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < t_end) fit_track<1>(g, rt, io, t, slots + threadIdx.x, blockDim.x);
+    if (t < t_end) fit_track<1, false>(g, rt, io, t - threadIdx.x, threadIdx.x, slots + threadIdx.x, blockDim.x);
 }
 
-// Persistent kernel: each warp claims 32-track units from *counter until the
-// batch is exhausted (Section 4.2: fill the GPU with the tracks of many events
-// in one launch).  Warps schedule themselves, so a warp slowed by an
-// extended-precision update does not hold the rest of its block.  MINB > 1
-// caps the registers per thread at 65536 / (BLOCK * MINB) to raise occupancy.
-// DEPTH >= 2 keeps the hit ring in dynamic shared memory (ring_floats(...)).
+// One thread per track over the whole batch (Section 4.2: fill the GPU with the
+// tracks of many events in one launch).  MINB > 1 caps the registers per
+// thread at 65536 / (BLOCK * MINB) to raise occupancy.  DEPTH >= 2 keeps the
+// hit ring in dynamic shared memory (ring_bytes(...)).
+//
+// The FP64 pipe is 64 times narrower than the FP32 one and takes as long for
+// one lane of a warp as for 32, so a track that needs it is put off: its flags
+// are set to kPutOff and it is counted in work[0], and fit_extended_kernel,
+// launched behind, fits these tracks from their seeds in full warps (none: it
+// returns at once).  With one track in eight above pt_hi (1,000,000 tracks, pT
+// log-uniform 0.24 to 500 GeV) nearly every warp held one and stopped for it
+// at every layer: 7.09 ms before, 1.03 ms now.  Without the FP64 code
+// this kernel also needs fewer registers (96 with the ring, no spills).
+constexpr uint32_t kPutOff = 0x80000000u;
+
 template <int BLOCK, int MINB, int DEPTH>
-__global__ void __launch_bounds__(BLOCK, MINB) fit_persistent_kernel(const FitGeom g, const Routing rt,
-                                                                      const FitIO io, unsigned *counter)
+__global__ void __launch_bounds__(BLOCK, MINB) fit_kernel(const FitGeom g, const Routing rt, const FitIO io,
+                                                           unsigned *work)
 {
-    __shared__ float slots[kSlotSize * BLOCK];
     extern __shared__ float ring[];
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned n_units = (unsigned)((io.T + 31) / 32);
-    for (;;) {
-        unsigned u = 0;
-        if (lane == 0) u = atomicAdd(counter, 1u);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        if (u >= n_units) break;
-        const int64_t t = (int64_t)u * 32 + lane;
-        if (t < io.T) fit_track<DEPTH>(g, rt, io, t, slots + threadIdx.x, BLOCK, ring + threadIdx.x);
-    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int64_t base = (int64_t)blockIdx.x * BLOCK;
+    const unsigned off = threadIdx.x;
+    bool put_off = false;
+    if (base + off < io.T) put_off = fit_track<DEPTH, true>(g, rt, io, base, off, nullptr, BLOCK, ring + off);
+    if (put_off) (io.out_flags + base)[off] = kPutOff;
+    const unsigned n = __popc(__ballot_sync(0xffffffffu, put_off));
+    if (n && (off & 31u) == 0) atomicAdd(work, n);
 }
 
-using PersistentFn = void (*)(FitGeom, Routing, FitIO, unsigned *);
+// The tracks put off by the launch before: a block gathers them from the flags
+// of its chunks of the batch until it has one per thread, and fits those.
+constexpr int kExtBlock = 128;
+__global__ void __launch_bounds__(kExtBlock, 4) fit_extended_kernel(const FitGeom g, const Routing rt, const FitIO io,
+                                                                     unsigned *work)
+{
+    __shared__ float slots[kSlotSize * kExtBlock];
+    __shared__ int64_t queue[2 * kExtBlock];
+    __shared__ int queued;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (__ldcg(work) == 0) return;
+    if (threadIdx.x == 0) queued = 0;
+    __syncthreads();
+    const int64_t chunks = (io.T + kExtBlock - 1) / kExtBlock;
+    for (int64_t ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+        const int64_t t = ch * kExtBlock + threadIdx.x;
+        if (t < io.T && __ldcg(io.out_flags + t) == kPutOff) queue[atomicAdd(&queued, 1)] = t;
+        __syncthreads();
+        const bool last = ch + gridDim.x >= chunks;
+        int n = queued;
+        while (n >= kExtBlock || (last && n > 0)) {  // uniform over the block
+            const int take = min(n, kExtBlock);
+            n -= take;
+            if ((int)threadIdx.x < take)
+                fit_track<1, false>(g, rt, io, 0, queue[n + threadIdx.x], slots + threadIdx.x, kExtBlock);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) queued = n;
+        __syncthreads();
+    }
+    // the last block to end clears the count: every block has read it
+    if (threadIdx.x == 0 && atomicInc(work + 1, gridDim.x - 1) == gridDim.x - 1) work[0] = 0u;
+}
+
+using FitFn = void (*)(FitGeom, Routing, FitIO, unsigned *);
 
 // Dynamic shared memory of a shape: DEPTH + 1 stages of 9 floats per thread.
 constexpr size_t ring_bytes(int block, int depth) { return depth > 1 ? (size_t)(depth + 1) * 9 * block * 4 : 0; }
@@ -208,25 +255,25 @@ constexpr size_t ring_bytes(int block, int depth) { return depth > 1 ? (size_t)(
 // __launch_bounds__(BLOCK, 65536 / (R * BLOCK)).
 struct Shape {
     int block, cap, depth;
-    PersistentFn fn;
+    FitFn fn;
 };
 const Shape kShapes[] = {
-    {32, 0, 1, fit_persistent_kernel<32, 1, 1>},     {64, 0, 1, fit_persistent_kernel<64, 1, 1>},
-    {128, 0, 1, fit_persistent_kernel<128, 1, 1>},   {256, 0, 1, fit_persistent_kernel<256, 1, 1>},
-    {32, 168, 1, fit_persistent_kernel<32, 12, 1>},  {64, 168, 1, fit_persistent_kernel<64, 6, 1>},
-    {128, 168, 1, fit_persistent_kernel<128, 3, 1>}, {32, 128, 1, fit_persistent_kernel<32, 16, 1>},
-    {64, 128, 1, fit_persistent_kernel<64, 8, 1>},   {128, 128, 1, fit_persistent_kernel<128, 4, 1>},
-    {256, 128, 1, fit_persistent_kernel<256, 2, 1>}, {32, 96, 1, fit_persistent_kernel<32, 20, 1>},
-    {64, 96, 1, fit_persistent_kernel<64, 10, 1>},   {128, 96, 1, fit_persistent_kernel<128, 5, 1>},
-    {32, 80, 1, fit_persistent_kernel<32, 24, 1>},   {64, 80, 1, fit_persistent_kernel<64, 12, 1>},
-    {128, 80, 1, fit_persistent_kernel<128, 6, 1>},  {256, 80, 1, fit_persistent_kernel<256, 3, 1>},
-    {32, 128, 2, fit_persistent_kernel<32, 16, 2>},  {64, 128, 2, fit_persistent_kernel<64, 8, 2>},
-    {128, 128, 2, fit_persistent_kernel<128, 4, 2>}, {256, 128, 2, fit_persistent_kernel<256, 2, 2>},
-    {32, 96, 2, fit_persistent_kernel<32, 20, 2>},   {64, 96, 2, fit_persistent_kernel<64, 10, 2>},
-    {128, 96, 2, fit_persistent_kernel<128, 5, 2>},  {32, 128, 4, fit_persistent_kernel<32, 16, 4>},
-    {64, 128, 4, fit_persistent_kernel<64, 8, 4>},   {128, 128, 4, fit_persistent_kernel<128, 4, 4>},
-    {256, 128, 4, fit_persistent_kernel<256, 2, 4>}, {32, 96, 4, fit_persistent_kernel<32, 20, 4>},
-    {64, 96, 4, fit_persistent_kernel<64, 10, 4>},   {128, 96, 4, fit_persistent_kernel<128, 5, 4>},
+    {32, 0, 1, fit_kernel<32, 1, 1>},     {64, 0, 1, fit_kernel<64, 1, 1>},
+    {128, 0, 1, fit_kernel<128, 1, 1>},   {256, 0, 1, fit_kernel<256, 1, 1>},
+    {32, 168, 1, fit_kernel<32, 12, 1>},  {64, 168, 1, fit_kernel<64, 6, 1>},
+    {128, 168, 1, fit_kernel<128, 3, 1>}, {32, 128, 1, fit_kernel<32, 16, 1>},
+    {64, 128, 1, fit_kernel<64, 8, 1>},   {128, 128, 1, fit_kernel<128, 4, 1>},
+    {256, 128, 1, fit_kernel<256, 2, 1>}, {32, 96, 1, fit_kernel<32, 20, 1>},
+    {64, 96, 1, fit_kernel<64, 10, 1>},   {128, 96, 1, fit_kernel<128, 5, 1>},
+    {32, 80, 1, fit_kernel<32, 24, 1>},   {64, 80, 1, fit_kernel<64, 12, 1>},
+    {128, 80, 1, fit_kernel<128, 6, 1>},  {256, 80, 1, fit_kernel<256, 3, 1>},
+    {32, 128, 2, fit_kernel<32, 16, 2>},  {64, 128, 2, fit_kernel<64, 8, 2>},
+    {128, 128, 2, fit_kernel<128, 4, 2>}, {256, 128, 2, fit_kernel<256, 2, 2>},
+    {32, 96, 2, fit_kernel<32, 20, 2>},   {64, 96, 2, fit_kernel<64, 10, 2>},
+    {128, 96, 2, fit_kernel<128, 5, 2>},  {32, 128, 4, fit_kernel<32, 16, 4>},
+    {64, 128, 4, fit_kernel<64, 8, 4>},   {128, 128, 4, fit_kernel<128, 4, 4>},
+    {256, 128, 4, fit_kernel<256, 2, 4>}, {32, 96, 4, fit_kernel<32, 20, 4>},
+    {64, 96, 4, fit_kernel<64, 10, 4>},   {128, 96, 4, fit_kernel<128, 5, 4>},
 };
 
 const Shape *find_shape(int block, int cap, int depth)
@@ -267,18 +314,14 @@ cudaError_t launch_fit_plain(const FitGeom &g, const Routing &rt, const FitIO &i
     return cudaGetLastError();
 }
 
-int persistent_blocks_per_sm(int block, int cap, int depth)
+int fit_shape_usable(int block, int cap, int depth)
 {
     const Shape *sh = find_shape(block, cap, depth);
     if (!sh) return 0;
-    int n = 0;
-    if (prepare_shape(sh) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sh->fn, block, ring_bytes(block, depth)) != cudaSuccess)
-        return -1;
-    return n;
+    return prepare_shape(sh) == cudaSuccess ? 1 : -1;
 }
 
-int persistent_shapes(int *blocks, int *caps, int *depths, int max_n)
+int fit_shapes(int *blocks, int *caps, int *depths, int max_n)
 {
     int n = 0;
     for (const Shape &sh : kShapes)
@@ -291,15 +334,27 @@ int persistent_shapes(int *blocks, int *caps, int *depths, int max_n)
     return n;
 }
 
-cudaError_t launch_fit_persistent(const FitGeom &g, const Routing &rt, const FitIO &io, int block, int cap, int depth,
-                                  int grid, unsigned *counter, cudaStream_t stream)
+cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &io, int block, int cap, int depth,
+                                  int sm_count, unsigned *work, cudaStream_t stream)
 {
     const Shape *sh = find_shape(block, cap, depth);
     if (!sh) return cudaErrorInvalidValue;
-    const cudaError_t e = prepare_shape(sh);
+    cudaError_t e = prepare_shape(sh);
     if (e != cudaSuccess) return e;
-    sh->fn<<<grid, block, ring_bytes(block, depth), stream>>>(g, rt, io, counter);
-    return cudaGetLastError();
+    const int64_t grid = (io.T + block - 1) / block;
+    if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
+    sh->fn<<<(unsigned)grid, block, ring_bytes(block, depth), stream>>>(g, rt, io, work);
+    if ((e = cudaGetLastError()) != cudaSuccess || rt.mode == 0) return e;  // without routing no track is put off
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>((io.T + kExtBlock - 1) / kExtBlock, (int64_t)sm_count * 4));
+    cfg.blockDim = dim3(kExtBlock);
+    cfg.stream = stream;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fit_extended_kernel, g, rt, io, work);
 }
 
 }  // namespace kf

@@ -34,29 +34,28 @@ struct FitIO {
     uint32_t *out_flags;
 };
 
-// A persistent-fit launch shape: threads per block, register cap (0 = none)
+// A launch shape of the fit: threads per block, register cap (0 = none)
 // and hit prefetch depth (layers ahead).
 struct FitShape {
     int block, cap, depth;
 };
 
-// status word bits written by the persistent kernels (device scratch)
-constexpr unsigned kStatusTimeout = 1u;
-
 // Launchers (kf_fit.cu).  All enqueue on `stream` and return the launch error.
 cudaError_t launch_fit_plain(const FitGeom &g, const Routing &rt, const FitIO &io, int64_t t_begin,
                              int64_t t_end, int block, cudaStream_t stream);
-// Persistent kernel: grid = `grid` blocks of `block` threads with registers
-// capped at `cap` per thread (0 = no cap), hits loaded `depth` layers ahead
-// (1: registers; 2, 4: a cp.async ring in shared memory); warps claim 32-track
-// units from *counter, which must read 0 at launch.
-cudaError_t launch_fit_persistent(const FitGeom &g, const Routing &rt, const FitIO &io, int block, int cap,
-                                  int depth, int grid, unsigned *counter, cudaStream_t stream);
-// Blocks of the persistent kernel of this shape that fit on one SM at once on
-// the current device: 0 if the shape is not compiled in, -1 if a CUDA call
-// (the shared-memory opt-in or the occupancy query) failed.
-int persistent_blocks_per_sm(int block, int cap, int depth);
+// The fit of the whole batch: a kernel of blocks of `block` threads with
+// registers capped at `cap` per thread (0 = no cap), hits loaded `depth` layers
+// ahead (1: registers; 2, 4: a cp.async ring in shared memory), which counts
+// the tracks that need extended precision in work[0], and with routing a
+// second one for those.  `work` (kFitWorkBytes) must read 0 at launch, and does
+// again when the fit has run.
+cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &io, int block, int cap, int depth,
+                             int sm_count, unsigned *work, cudaStream_t stream);
+constexpr size_t kFitWorkBytes = 2 * sizeof(unsigned);
+// 1 if this shape can be launched on the current device, 0 if it is not
+// compiled in, -1 if its shared-memory opt-in failed.
+int fit_shape_usable(int block, int cap, int depth);
 // The (block, cap, depth) shapes compiled in; returns how many were written.
-int persistent_shapes(int *blocks, int *caps, int *depths, int max_n);
+int fit_shapes(int *blocks, int *caps, int *depths, int max_n);
 
 }  // namespace kf

@@ -1,7 +1,7 @@
 // The fit from host buffers (the paper's multi-stream event transfers, Section
 // 4.2; its builds spent about half their wall time on host-device transfers,
 // Section 4.3).  Page-locked buffers the device can address are read and
-// written in place by one persistent launch: on this part the kernel's loads
+// written in place by the fit itself: on this part the kernel's loads
 // over the host link run as fast as the copy engines (about 210 GB/s), and the
 // inputs' reads and the outputs' writes share the link in both directions
 // with no pipeline fill or drain.  Other buffers go through chunks copied in,
@@ -19,7 +19,7 @@ constexpr int kHostStreams = 3;
 
 struct HostPipe {
     cudaStream_t stream[kHostStreams] = {};
-    unsigned *counter = nullptr;  // one work counter per stream
+    char *work = nullptr;  // the work counters of one launch per stream
     char *buf[kHostStreams] = {};  // staging for one chunk per stream
     size_t buf_bytes = 0;
 };
@@ -31,7 +31,7 @@ void destroy_host_state(HostPipe *s)
         if (s->stream[i]) cudaStreamDestroy(s->stream[i]);
         cudaFree(s->buf[i]);
     }
-    cudaFree(s->counter);
+    cudaFree(s->work);
     delete s;
 }
 
@@ -99,11 +99,9 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
     const int cap = o.reg_cap < 0 ? 0 : (o.reg_cap ? o.reg_cap : 128);
     DeviceGuard dg(context_device(ctx));
     const int depth = o.hit_prefetch ? o.hit_prefetch : 1;
-    const int per_sm = persistent_blocks_per_sm(block, cap, depth);
-    if (per_sm < 1)
-        return set_error(ctx, KF_ERR_ARG, "no persistent fit of %d tracks per block, cap %d, hit prefetch %d", block,
-                         cap, depth);
-    const int grid = per_sm * context_sm_count(ctx);
+    const int usable = fit_shape_usable(block, cap, depth);
+    if (usable < 1)
+        return set_error(ctx, KF_ERR_ARG, "no fit of %d tracks per block, cap %d, hit prefetch %d", block, cap, depth);
     int64_t C = chunk_tracks ? chunk_tracks : (int64_t(1) << 18);
     C = std::min<int64_t>(C, n_tracks);
     C = (C + 31) / 32 * 32;
@@ -113,7 +111,8 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
     HostPipe *&hp = context_host_state(ctx);
     if (!hp) {
         hp = new HostPipe;
-        bool ok = cudaMalloc(&hp->counter, kHostStreams * sizeof(unsigned)) == cudaSuccess;
+        bool ok = cudaMalloc(&hp->work, kHostStreams * kFitWorkBytes) == cudaSuccess &&
+                  cudaMemset(hp->work, 0, kHostStreams * kFitWorkBytes) == cudaSuccess;
         for (int i = 0; ok && i < kHostStreams; ++i)
             ok = cudaStreamCreateWithFlags(&hp->stream[i], cudaStreamNonBlocking) == cudaSuccess;
         if (!ok) {
@@ -154,10 +153,8 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
                            static_cast<int16_t *>(dev[9]),
                            static_cast<uint32_t *>(dev[10])};
             cudaStream_t s = hp->stream[0];
-            const int64_t units = (n_tracks + 31) / 32;
-            const int grid_n = (int)std::min<int64_t>(grid, std::max<int64_t>((units * 32 + block - 1) / block, 1));
-            cudaError_t e = cudaMemsetAsync(hp->counter, 0, sizeof(unsigned), s);
-            if (e == cudaSuccess) e = launch_fit_persistent(g, rt, io, block, cap, depth, grid_n, hp->counter, s);
+            const cudaError_t e = launch_fit_tuned(g, rt, io, block, cap, depth, context_sm_count(ctx),
+                                                   reinterpret_cast<unsigned *>(hp->work), s);
             const cudaError_t e2 = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return cuda_error(ctx, e, "host-buffer fit");
             if (e2 != cudaSuccess) return cuda_error(ctx, e2, "host-buffer fit");
@@ -203,7 +200,6 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
         in(lay.hit_pos, hit_pos, 4, (size_t)L * 3);
         in(lay.hit_cov, hit_cov, 4, (size_t)L * 6);
         in(lay.mask, hit_mask, 4, 1);
-        if (e == cudaSuccess) e = cudaMemsetAsync(hp->counter + k, 0, sizeof(unsigned), s);
         if (e == cudaSuccess) {
             FitIO io{n,
                      reinterpret_cast<const float *>(b + lay.seed_state),
@@ -217,7 +213,8 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
                      reinterpret_cast<float *>(b + lay.out_chi2),
                      reinterpret_cast<int16_t *>(b + lay.out_ndof),
                      reinterpret_cast<uint32_t *>(b + lay.out_flags)};
-            e = launch_fit_persistent(g, rt, io, block, cap, depth, grid, hp->counter + k, s);
+            e = launch_fit_tuned(g, rt, io, block, cap, depth, context_sm_count(ctx),
+                                 reinterpret_cast<unsigned *>(hp->work + k * kFitWorkBytes), s);
         }
         out(out_state, lay.out_state, 4, 6);
         out(out_cov, lay.out_cov, 4, 21);

@@ -681,6 +681,8 @@ __device__ __forceinline__ void scatter_local(const Local &p, float theta2, floa
 //     C_ii > gain_max V_ii for some i.
 // Returns 0 updated in FP32, 2 updated with extended-precision arithmetic,
 // 3 updated in FP64 with a PSD repair, 1 failed (S not positive definite).
+// DEFER: an update that needs extended precision is left undone, 4 returned.
+template <bool DEFER = false>
 __device__ __forceinline__ int update_local(Local &p, float c[15], const float m[3], const float v[6],
                                             const Routing &rt, float *dchi2, float *slot, int stride)
 {
@@ -711,6 +713,9 @@ __device__ __forceinline__ int update_local(Local &p, float c[15], const float m
             kind = 1;
     } else if (!pd) {
         return 1;
+    }
+    if constexpr (DEFER) {
+        if (kind) return 4;
     }
     if (kind) {
         float *s = slot;
