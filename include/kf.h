@@ -65,7 +65,7 @@ typedef struct CUstream_st *kf_stream; /* a cudaStream_t; NULL is the legacy def
 #define KF_FLAG_INVERSION_FAILED 4u  /* S = H C H^T + V not positive definite: update skipped */
 #define KF_FLAG_NAN_INPUT 8u         /* non-finite seed or used hit: outputs are the seed */
 #define KF_FLAG_FP64_PATH 16u        /* at least one update used extended precision: a float-float
-                                        gain or the FP64 update */
+                                        gain, the float-float or the FP64 update */
 #define KF_FLAG_PSD_REPAIRED 32u     /* the FP64 path clamped the covariance */
 
 #define KF_MAX_LAYERS 32
@@ -75,7 +75,7 @@ typedef struct CUstream_st *kf_stream; /* a cudaStream_t; NULL is the legacy def
 #define KF_PRECISION_ROUTED 1 /* FP32, with ill-conditioned updates redone in FP64 */
 
 /* launch_mode */
-#define KF_LAUNCH_AUTO 0      /* all events in one launch, and one for the tracks that need FP64 */
+#define KF_LAUNCH_AUTO 0      /* all events in one launch, and one for those in extended precision */
 #define KF_LAUNCH_PER_EVENT 1 /* one plain launch per event (needs event_offsets) */
 #define KF_LAUNCH_FLAT 2      /* one plain launch over all tracks */
 
@@ -99,7 +99,8 @@ typedef struct {
     float cond_max;          /* an update whose S has a correlation matrix R (S scaled to unit
                                 diagonal) with det R < 27 / (4 cond_max) runs in FP64, so
                                 every FP32 update has cond_2(R) <= cond_max */
-    float pt_lo, pt_hi;      /* tracks with pT outside [pt_lo, pt_hi] GeV update in FP64 */
+    float pt_lo, pt_hi;      /* tracks with pT outside [pt_lo, pt_hi] GeV update in float-float
+                                (46 bits and more throughout) where S is well conditioned */
     float gain_max;          /* > 0: an update with C_ii > gain_max V_ii (i = x, y, z) forms
                                 its gain (S^-1 and K) in float-float; 0 = off */
     /* launch shape (fit) */
@@ -524,7 +525,7 @@ int kf_fit_tuned_shape(kf_context *ctx, int n_layers, int64_t n_tracks, int *tra
  * must not touch the allocator after start-up, or hosts that forbid
  * allocation while their own work is in flight can call this instead.  It
  * runs the same fit kernels (same steps, inputs, outputs and flags
- * as kf_fit_tracks, all events in one launch and the tracks that need FP64 in
+ * as kf_fit_tracks, all events in one launch and those in extended precision in
  * another) and allocates nothing: the kernels' only scratch, two 4-byte
  * counters, is a fixed array in the library's device memory that every GPU
  * loading the library holds until the process exits.

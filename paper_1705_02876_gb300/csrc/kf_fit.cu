@@ -186,14 +186,16 @@ __global__ void __launch_bounds__(256) fit_plain_kernel(const FitGeom g, const R
 // thread at 65536 / (BLOCK * MINB) to raise occupancy.  DEPTH >= 2 keeps the
 // hit ring in dynamic shared memory (ring_bytes(...)).
 //
-// The FP64 pipe is 64 times narrower than the FP32 one and takes as long for
-// one lane of a warp as for 32, so a track that needs it is put off: its flags
-// are set to kPutOff and it is counted in work[0], and fit_extended_kernel,
-// launched behind, fits these tracks from their seeds in full warps (none: it
-// returns at once).  With one track in eight above pt_hi (1,000,000 tracks, pT
+// An update in extended precision (float-float: some 1,100 instructions; FP64:
+// a pipe 64 times narrower than the FP32 one) takes as long for one lane of a
+// warp as for 32, so a track that needs one is put off: its flags are set to
+// kPutOff and it is counted in work[0], and fit_extended_kernel, launched
+// behind, fits these tracks from their seeds in full warps (none: it returns
+// at once).  With one track in eight above pt_hi (1,000,000 tracks, pT
 // log-uniform 0.24 to 500 GeV) nearly every warp held one and stopped for it
-// at every layer: 7.09 ms before, 1.03 ms now.  Without the FP64 code
-// this kernel also needs fewer registers (96 with the ring, no spills).
+// at every layer: 7.09 ms in line in FP64, 1.03 ms put off in FP64, 0.32 ms
+// in float-float.  Without that code this kernel also needs fewer registers
+// (96 with the ring, no spills).
 constexpr uint32_t kPutOff = 0x80000000u;
 
 template <int BLOCK, int MINB, int DEPTH>

@@ -454,9 +454,113 @@ static __device__ __noinline__ int update_ff(float *slot_p, int stride)
     return 2;
 }
 
+// The whole update in float-float: update_fp64 to 2^-46 instead of 2^-53, for
+// well-conditioned S (cond_2(R) <= cond_max, the caller's test), where the
+// FP32 results it leaves are the same but for rounding ties.  Some 1,100 FP32
+// instructions, about a tenth of the time of the FP64 pipe's 280.  Returns 2 or
+// 3 (repaired).
+__device__ __forceinline__ ff ff_sub(ff x, ff y) { return ff_add(x, ff_neg(y)); }
+__device__ __forceinline__ ff ff_addf(ff x, float y)
+{
+    const ff s = two_sum(x.hi, y);
+    return fast_two_sum(s.hi, __fadd_rn(s.lo, x.lo));
+}
+__device__ __forceinline__ ff ff_mulf(ff x, float y)
+{
+    const ff p = two_prod(x.hi, y);
+    return fast_two_sum(p.hi, __fmaf_rn(x.lo, y, p.lo));
+}
+__device__ __forceinline__ ff ff_rcp(ff x)  // Newton from the FP32 reciprocal r: r (1 + e + e^2), e = 1 - x r
+{
+    const float r = __fdividef(1.0f, x.hi);
+    const float e = __fmaf_rn(-x.lo, r, __fmaf_rn(-x.hi, r, 1.0f));
+    return fast_two_sum(r, __fmul_rn(r, __fmaf_rn(e, e, e)));
+}
+__device__ __forceinline__ float ff_round(ff x, float y) { return ff_addf(x, y).hi; }  // x + y to FP32
+
+static __device__ __noinline__ int update_wide(float *slot_p, int stride)
+{
+    const SlotRef sl{slot_p, stride};
+    ff nx{sl.n(0), 0.0f}, ny{sl.n(1), 0.0f};
+    {  // the frame's n, normalised (one Newton step)
+        const ff a = two_prod(nx.hi, nx.hi), b = two_prod(ny.hi, ny.hi);
+        const ff s = ff_addf(ff_add(a, b), -1.0f);
+        const float h = -0.5f * s.hi;
+        nx = fast_two_sum(nx.hi, __fmul_rn(nx.hi, h));
+        ny = fast_two_sum(ny.hi, __fmul_rn(ny.hi, h));
+    }
+    ff vt, vz, l, ia, it, iz;
+    {
+        const float v0 = sl.v(0), v1 = sl.v(1), v2 = sl.v(2), v3 = sl.v(3), v4 = sl.v(4);
+        const ff nn = ff_mul(nx, nx), tt = ff_mul(ny, ny), nt = ff_mul(nx, ny);
+        const ff x2 = ff_mulf(nt, 2.0f * v1);
+        const ff vnn = ff_add(ff_add(ff_mulf(nn, v0), ff_mulf(tt, v2)), x2);
+        const ff vnt = ff_add(ff_mul(nt, two_sum(v2, -v0)), ff_mulf(ff_sub(nn, tt), v1));
+        const ff vtt = ff_sub(ff_add(ff_mulf(tt, v0), ff_mulf(nn, v2)), x2);
+        const ff vnz = ff_add(ff_mulf(nx, v3), ff_mulf(ny, v4)), vtz = ff_sub(ff_mulf(nx, v4), ff_mulf(ny, v3));
+        ia = ff_rcp(vnn);
+        vt = ff_mul(vnt, ia);
+        vz = ff_mul(vnz, ia);
+        it = ff_rcp(ff_sub(ff_addf(vtt, sl.c(0, 0)), ff_mul(vnt, vt)));
+        const ff e = ff_sub(ff_addf(vtz, sl.c(1, 0)), ff_mul(vnt, vz));
+        l = ff_mul(e, it);
+        iz = ff_rcp(ff_sub(ff_sub(two_sum(sl.c(1, 1), sl.v(5)), ff_mul(vnz, vz)), ff_mul(l, e)));
+    }
+    const float X0 = sl.x(0), X1 = sl.x(1), X2 = sl.x(2);
+    ff w1, w2;
+    {
+        const ff d0 = two_sum(sl.m(0), -X0), d1 = two_sum(sl.m(1), -X1);
+        const ff rn = ff_add(ff_mul(nx, d0), ff_mul(ny, d1));
+        const ff r1 = ff_sub(ff_sub(ff_mul(nx, d1), ff_mul(ny, d0)), ff_mul(vt, rn));
+        const ff r2 = ff_sub(ff_sub(two_sum(sl.m(2), -X2), ff_mul(vz, rn)), ff_mul(l, r1));
+        w1 = ff_mul(r1, it);
+        w2 = ff_mul(r2, iz);
+        const ff chi = ff_add(ff_mul(ff_mul(rn, rn), ia), ff_add(ff_mul(r1, w1), ff_mul(r2, w2)));
+        sl.chi2() = __fadd_rn(chi.hi, chi.lo);
+    }
+    float a[5];
+    ff b[5];
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+        a[u] = sl.c(u, 0);
+        b[u] = ff_addf(ff_neg(ff_mulf(l, a[u])), sl.c(u, 1));
+        const ff dx = ff_add(ff_mulf(w1, a[u]), ff_mul(b[u], w2));
+        if (u == 0) {
+            sl.x(0) = ff_round(ff_neg(ff_mul(ny, dx)), X0);
+            sl.x(1) = ff_round(ff_mul(nx, dx), X1);
+        } else {
+            sl.x(u + 1) = ff_round(dx, u == 1 ? X2 : sl.x(u + 1));
+        }
+    }
+    float tr = 0.0f;
+    bool rep = false;
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+        const ff ka = ff_mulf(it, -a[u]), kb = ff_mul(ff_neg(b[u]), iz);
+#pragma unroll
+        for (int w = 0; w <= u; ++w) {
+            const ff p = two_prod(ka.hi, a[w]), q = two_prod(kb.hi, b[w].hi);
+            const ff s = two_sum(sl.c(u, w), p.hi), t = two_sum(s.hi, q.hi);
+            const float lo = __fadd_rn(__fadd_rn(s.lo, t.lo), __fadd_rn(__fmaf_rn(ka.lo, a[w], p.lo),
+                                                                        __fmaf_rn(kb.hi, b[w].lo, __fmaf_rn(kb.lo, b[w].hi, q.lo))));
+            const float v = __fadd_rn(t.hi, lo);
+            sl.c(u, w) = v;
+            if (u == w) {
+                tr += fabsf(v);
+                rep = rep || !(v > 0.0f);
+            }
+        }
+    }
+    if (!rep) return 2;
+#pragma unroll 1
+    for (int u = 0; u < 5; ++u)
+        if (!(sl.c(u, u) > 0.0f)) sl.c(u, u) = 1e-12f * tr;
+    return 3;
+}
+
 static __device__ __noinline__ int update_ext(float *slot, int stride, int kind)
 {
-    return kind == 2 ? update_fp64(slot, stride) : update_ff(slot, stride);
+    return kind == 2 ? update_fp64(slot, stride) : kind == 3 ? update_wide(slot, stride) : update_ff(slot, stride);
 }
 
 struct Routing {
@@ -676,7 +780,9 @@ __device__ __forceinline__ void scatter_local(const Local &p, float theta2, floa
 //     correlation matrix R = D^-1/2 S D^-1/2 (D = diag S) is below
 //     27 / (4 cond_max) (R's eigenvalues sum to 3, so that this bounds
 //     cond_2(R) by cond_max on the FP32 path; the spread of S's diagonal, V_nn
-//     << C_zz, is harmless), or when pT lies outside [pt_lo, pt_hi];
+//     << C_zz, is harmless);
+//   * else, when pT lies outside [pt_lo, pt_hi], it is redone in float-float
+//     (update_wide);
 //   * with gain_max > 0, the gain is formed in float-float (update_ff) when
 //     C_ii > gain_max V_ii for some i.
 // Returns 0 updated in FP32, 2 updated with extended-precision arithmetic,
@@ -706,8 +812,10 @@ __device__ __forceinline__ int update_local(Local &p, float c[15], const float m
     if (rt.mode == 1) {
         const bool ill = !pd || dt * dz <= rt.det_min * (stt * szz);
         const float pt2 = fmaf(p.q1, p.q1, p.q2 * p.q2);
-        if (ill || pt2 < rt.pt_lo * rt.pt_lo || pt2 > rt.pt_hi * rt.pt_hi)
+        if (ill)
             kind = 2;
+        else if (pt2 < rt.pt_lo * rt.pt_lo || pt2 > rt.pt_hi * rt.pt_hi)
+            kind = 3;
         else if (rt.gain_max > 0.0f && (tt * c[pk(0, 0)] > rt.gain_max * v[0] || nn * c[pk(0, 0)] > rt.gain_max * v[2] ||
                                         c[pk(1, 1)] > rt.gain_max * v[5]))
             kind = 1;
