@@ -206,14 +206,15 @@ int size_class(int64_t n)
     return c;
 }
 
-// Routed fits of fewer tracks than this run in one launch, warps of 32 tracks
-// with the FP64 update in line, and are not tuned: the launch for the tracks
-// put off costs the host 3 us (19.7 against 16.4 us a call at 1,000 tracks,
-// whose kernel takes 8.7 us either way), and with at most two warps on an SM
-// they hardly wait for each other's FP64 updates.  With one track in eight in
-// FP64 the lines cross between 10,000 tracks (103 us in line, 121 put off) and
-// 20,000 (134 and 123).  A power of two, as the tuner's size classes.
-constexpr int64_t kOneLaunchTracks = 8192;
+// Routed fits of fewer tracks than this run in one launch, blocks of 64 tracks
+// with the updates in extended precision in line, and are not tuned: the launch
+// for the tracks put off costs the host 2 to 3 us a call, and few warps share
+// an SM, so that one waiting for its own such update holds up little.  At
+// 10 layers the kernels take 8.9 and 8.8 us for 10,000 tracks (in line, put
+// off), 10.6 and 11.0 for 20,000, 13.0 and 13.2 for 40,000; with one track in
+// eight in extended precision 26 and 33, 30 and 37, 40 and 39.  A power of two,
+// as the tuner's size classes.
+constexpr int64_t kOneLaunchTracks = 32768;
 
 cudaError_t enqueue_fit(kf_context *ctx, const FitGeom &g, const Routing &rt, const FitIO &io, const FitShape &sh,
                         cudaStream_t stream)
@@ -330,8 +331,8 @@ int kf_fit_tracks(kf_context *ctx, const kf_geometry *geom, int64_t n_tracks, co
         break;
     default: {
         if (rt.mode == 1 && n_tracks < kOneLaunchTracks && !block && !o.reg_cap && !o.hit_prefetch) {
-            e = launch_fit_plain(g, rt, io, 0, n_tracks, 32, stream);
-            ctx->tuned.emplace(std::make_tuple(g.L, size_class(n_tracks), rt.mode, 0, 0, 0), FitShape{32, 0, 1});
+            e = launch_fit_plain(g, rt, io, 0, n_tracks, 64, stream);
+            ctx->tuned[std::make_tuple(g.L, size_class(n_tracks), rt.mode, 0, 0, 0)] = FitShape{64, 0, 1};
             break;
         }
         FitShape shape{block, o.reg_cap < 0 ? 0 : o.reg_cap, o.hit_prefetch};

@@ -34,9 +34,16 @@ struct BuildState {
     float4 *bkey = nullptr;  // binned hits: (phi, z, index within the segment as bits, radius)
     int32_t *bin_off = nullptr;
     int32_t *hit_rank = nullptr;  // the binning's rank of each hit within its bin
-    int64_t *seg_off = nullptr;  // device copy of the segment bounds [n_seg + 1]
-    int64_t *ev_off = nullptr;   // device copy of hit_offsets [n_events][L + 1]
-    size_t ev_capacity = 0;
+    int64_t *seg_off = nullptr;  // device copy of the segment bounds [n_seg + 1], then of hit_offsets [n_events][L + 1]
+    // pinned staging of those offsets: a call fills the next slot, once the
+    // copy that last read it is done, and need not wait for its own
+    struct Stage {
+        int64_t *pin = nullptr;
+        size_t elems = 0;
+        cudaEvent_t copied = nullptr;
+        bool used = false;
+    } stage[4];
+    unsigned next_stage = 0;
     // the host-buffer build's pipeline: streams, and per ring slot the batch's device buffers,
     // its pinned offset staging and the events that order the slot's reuse
     cudaStream_t hs_in = nullptr, hs_run = nullptr, hs_out = nullptr;
@@ -74,7 +81,10 @@ void destroy_build_state(BuildState *s)
     cudaFree(s->bin_off);
     cudaFree(s->hit_rank);
     cudaFree(s->seg_off);
-    cudaFree(s->ev_off);
+    for (auto &st : s->stage) {
+        cudaFreeHost(st.pin);
+        if (st.copied) cudaEventDestroy(st.copied);
+    }
     cudaFree(s->seed_flag);
     cudaFree(s->seed_list);
     cudaFree(s->list_count);
@@ -1199,19 +1209,33 @@ int build_impl(kf_context *ctx, const kf_geometry *geom, int n_events, const int
     BuildState *&st = context_build_state(ctx);
     if (!st) st = new BuildState;
     const size_t n_seg = (size_t)n_events * L;
-    if (!grow(&st->seg_off, st->seg_capacity, n_seg + 1) || !grow(&st->ev_off, st->ev_capacity, (size_t)n_events * (L + 1)))
+    const size_t n_off = n_seg + 1 + (size_t)n_events * (L + 1);
+    cudaStreamCaptureStatus capst = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(stream, &capst);
+    if (capst != cudaStreamCaptureStatusNone)  // a replay would read the staging of a later call
+        return cuda_error(ctx, cudaErrorStreamCaptureUnsupported, "offsets copy");
+    BuildState::Stage &sg = st->stage[st->next_stage++ % 4];
+    cudaError_t e = cudaSuccess;
+    if (sg.used && (e = cudaEventSynchronize(sg.copied)) != cudaSuccess) return cuda_error(ctx, e, "offsets copy");
+    if (sg.elems < n_off) {
+        cudaFreeHost(sg.pin);
+        sg.pin = nullptr;
+        sg.elems = 0;
+        sg.used = false;
+        if (cudaMallocHost(&sg.pin, n_off * sizeof(int64_t)) != cudaSuccess)
+            return set_error(ctx, KF_ERR_NOMEM, "could not allocate the build's scratch");
+        sg.elems = n_off;
+    }
+    if (!grow(&st->seg_off, st->seg_capacity, n_off) ||
+        (!sg.copied && cudaEventCreateWithFlags(&sg.copied, cudaEventDisableTiming) != cudaSuccess))
         return set_error(ctx, KF_ERR_NOMEM, "could not allocate the build's scratch");
-    std::vector<int64_t> seg(n_seg + 1);
-    const int64_t max_seg = segment_bounds(hit_offsets, n_events, L, 0, seg.data());
-    cudaError_t e = cudaMemcpyAsync(st->seg_off, seg.data(), (n_seg + 1) * sizeof(int64_t), cudaMemcpyHostToDevice,
-                                    stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(st->ev_off, hit_offsets, (size_t)n_events * (L + 1) * sizeof(int64_t),
-                            cudaMemcpyHostToDevice, stream);
+    const int64_t max_seg = segment_bounds(hit_offsets, n_events, L, 0, sg.pin);
+    std::memcpy(sg.pin + n_seg + 1, hit_offsets, (size_t)n_events * (L + 1) * sizeof(int64_t));
+    e = cudaMemcpyAsync(st->seg_off, sg.pin, n_off * sizeof(int64_t), cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaEventRecord(sg.copied, stream);
     if (e != cudaSuccess) return cuda_error(ctx, e, "offsets copy");
-    // the host vector must outlive the asynchronous copy
-    if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_error(ctx, e, "offsets copy");
-    const BuildBatch bt{n_events, st->ev_off, st->seg_off, max_seg, hit_pos, hit_cov, n_hits, n_seeds, seed_event,
+    sg.used = true;
+    const BuildBatch bt{n_events, st->seg_off + n_seg + 1, st->seg_off, max_seg, hit_pos, hit_cov, n_hits, n_seeds, seed_event,
                         seed_state, seed_cov, seed_charge, out_hit_idx, out_chi2, out_nhits, out_state, out_cov,
                         out_flags, 0, 0};
     return build_run(ctx, g, o, bt, log, stream);

@@ -217,9 +217,18 @@ def _ptr(t: torch.Tensor, dtype, shape=None, name=""):
     if t.dtype != dtype or not t.is_cuda or not t.is_contiguous():
         raise KFError(f"{name}: expected a contiguous CUDA {dtype} tensor, got {t.dtype} "
                       f"{'cuda' if t.is_cuda else 'cpu'} contiguous={t.is_contiguous()}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
-        raise KFError(f"{name}: shape {tuple(t.shape)} != {tuple(shape)}")
-    return t.data_ptr() if t.numel() else None
+    s = t.shape
+    if shape is not None and s != shape:
+        raise KFError(f"{name}: shape {tuple(s)} != {tuple(shape)}")
+    return t.data_ptr() if 0 not in s else None
+
+
+def _raw_stream(stream, device):
+    """The handle of `stream`, or of the device's current one."""
+    if stream is not None:
+        return stream.cuda_stream
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if index is None else index)
 
 
 def fit_outputs(n_tracks: int, device) -> dict:
@@ -257,9 +266,9 @@ def fit_tracks(ctx: Context, geom: GeometryArgs, seed_state, seed_cov, charge, h
         ev = np.ascontiguousarray(event_offsets, dtype=np.int64)
         n_ev = len(ev) - 1
         ev_ptr = ev.ctypes.data
-    s = stream if stream is not None else torch.cuda.current_stream(charge.device)
+    s = _raw_stream(stream, charge.device)
     rc = load().kf_fit_tracks(ctx.handle, ctypes.byref(geom.struct), T, ev_ptr, n_ev, *args,
-                              ctypes.byref(opt) if opt is not None else None, s.cuda_stream)
+                              ctypes.byref(opt) if opt is not None else None, s)
     ctx.check(rc, "kf_fit_tracks")
     return out
 
@@ -356,10 +365,10 @@ def build_tracks(ctx: Context, geom: GeometryArgs, hit_offsets, hit_pos, hit_cov
         _ptr(out["cov"], torch.float32, (21, S * N), "out_cov"),
         _ptr(out["flags"], torch.int32, (S, N), "out_flags"),
     ]
-    s = stream if stream is not None else torch.cuda.current_stream(dev)
+    s = _raw_stream(stream, dev)
     if log is None:
         rc = load().kf_build_tracks(ctx.handle, ctypes.byref(geom.struct), int(off.shape[0]), *args,
-                                    ctypes.byref(opt), s.cuda_stream)
+                                    ctypes.byref(opt), s)
         ctx.check(rc, "kf_build_tracks")
         return out
     cap = int(log["labels"].shape[0])
@@ -368,7 +377,7 @@ def build_tracks(ctx: Context, geom: GeometryArgs, hit_offsets, hit_pos, hit_cov
         _ptr(log["features"], torch.float32, (cap, 12), "log_features"),
         _ptr(log["labels"], torch.float32, (cap,), "log_labels"),
         _ptr(log["ref"], torch.int32, (cap, 4), "log_ref"), cap,
-        _ptr(log["count"], torch.int64, (1,), "log_count"), s.cuda_stream)
+        _ptr(log["count"], torch.int64, (1,), "log_count"), s)
     ctx.check(rc, "kf_build_tracks_logged")
     return out
 
@@ -435,7 +444,7 @@ PROPOSAL_PARAMS = 5057
 
 
 def _cur_stream(t, stream):
-    return (stream if stream is not None else torch.cuda.current_stream(t.device)).cuda_stream
+    return _raw_stream(stream, t.device)
 
 
 def proposal_gradient(ctx: Context, weights, features, labels, stream=None):
@@ -511,12 +520,12 @@ def seed_triplets(ctx: Context, geom: GeometryArgs, hit_offsets, hit_pos, hit_co
     off = np.ascontiguousarray(hit_offsets, dtype=np.int64)
     H = int(hit_pos.shape[1])
     dev = hit_pos.device
-    s = stream if stream is not None else torch.cuda.current_stream(dev)
+    s = _raw_stream(stream, dev)
     n = ctypes.c_int64()
     optp = ctypes.byref(opt) if opt is not None else None
     rc = load().kf_seed_triplets(ctx.handle, ctypes.byref(geom.struct), int(off.shape[0]),
                                  off.ctypes.data if off.size else None, _ptr(hit_pos, torch.float32, (3, H), "hit_pos"),
-                                 H, optp, ctypes.byref(n), s.cuda_stream)
+                                 H, optp, ctypes.byref(n), s)
     ctx.check(rc, "kf_seed_triplets")
     n = int(n.value)
     e = lambda shape, dt: torch.empty(shape, dtype=dt, device=dev)
@@ -527,7 +536,7 @@ def seed_triplets(ctx: Context, geom: GeometryArgs, hit_offsets, hit_pos, hit_co
                               _ptr(hit_cov, torch.float32, (6, H), "hit_cov"), optp, n,
                               *[_ptr(out[k], out[k].dtype, tuple(out[k].shape), k) for k in
                                 ("event", "hits", "seed_state", "seed_cov", "charge", "hit_pos", "hit_cov",
-                                 "hit_mask")], s.cuda_stream)
+                                 "hit_mask")], s)
     ctx.check(rc, "kf_seed_fetch")
     return out
 
@@ -557,9 +566,9 @@ def smooth_tracks(ctx: Context, geom: GeometryArgs, seed_state, seed_cov, charge
         _ptr(out["reached"], torch.int16, (T,), "out_reached"),
         _ptr(out["flags"], torch.int32, (T,), "out_flags"),
     ]
-    s = stream if stream is not None else torch.cuda.current_stream(dev)
+    s = _raw_stream(stream, dev)
     rc = load().kf_smooth_tracks(ctx.handle, ctypes.byref(geom.struct), T, *args,
-                                 ctypes.byref(opt) if opt is not None else None, s.cuda_stream)
+                                 ctypes.byref(opt) if opt is not None else None, s)
     ctx.check(rc, "kf_smooth_tracks")
     return out
 
@@ -603,6 +612,6 @@ def fit_tracks_noalloc(geom: GeometryArgs, seed_state, seed_cov, charge, hit_pos
         _ptr(out["ndof"], torch.int16, (T,), "out_ndof"),
         _ptr(out["flags"], torch.int32, (T,), "out_flags"),
     ]
-    s = stream if stream is not None else torch.cuda.current_stream(charge.device)
+    s = _raw_stream(stream, charge.device)
     return load().kf_fit_tracks_noalloc(ctypes.byref(geom.struct), T, *args,
-                                        ctypes.byref(opt) if opt is not None else None, s.cuda_stream)
+                                        ctypes.byref(opt) if opt is not None else None, s)
