@@ -3,6 +3,7 @@
 // ones are found without scanning the layer).
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -27,7 +28,7 @@ __device__ __forceinline__ int z_bin(float z, const BinGrid &bg)
     return min(max(b, 0), bg.n_z - 1);
 }
 
-// Binning is two kernels.  bin_count_kernel gives each (event, layer)
+// Binning many segments is two kernels.  bin_count_kernel gives each (event, layer)
 // segment one block, which counts the segment's hits into a histogram of its
 // bins in shared memory (shared-memory atomics; the count a hit finds before
 // its own is its rank within the bin, in no fixed order, kept in rank[h]),
@@ -155,6 +156,137 @@ __global__ void __launch_bounds__(kBinThreadsHP, 3) bin_scatter_kernel(const int
     }
 }
 
+// Few segments: a cluster of kBinCluster blocks bins each, in one kernel.  A
+// block counts a contiguous part of the hits into a histogram in its shared
+// memory; the cluster turns the histograms, each block a slice of the bins,
+// into the segment's bin offsets and every block's first place in every bin
+// (through distributed shared memory); then a block reads its part again and
+// places each key at the next place of its bin (a shared-memory atomic: the
+// order within a bin is not fixed).  The azimuths of a part are kept in shared
+// memory between the passes up to kBinCache hits, and computed again beyond.
+// One event (14 segments of 55,000 hits): 21 us with 1,024 threads, 29 with 512,
+// against 54 for the two kernels above, whose count runs on one SM per segment.
+// Beyond one wave of clusters (19 segments at one 1,024-thread block per SM, 38
+// at two of 512) those are faster (896 segments: 0.73 ms against 1.0 to 1.3),
+// since they keep more loads in flight.
+constexpr int kBinCluster = 8;
+constexpr int kBinUnroll = 4;    // hits per thread loaded together
+constexpr int kBinCache = 8192;  // azimuths a block keeps (32 KB)
+constexpr int kBinSlice = 4;     // bins per thread of a block's slice
+
+template <int THREADS>
+__global__ void __cluster_dims__(kBinCluster, 1, 1) __launch_bounds__(THREADS, 1024 / THREADS)
+    bin_cluster_kernel(const int64_t *seg_off, const float *hit_pos, int64_t H, BinGrid bg, int32_t *bin_off, float4 *bkey)
+{
+    static_assert(kMaxBins <= kBinCluster * THREADS * kBinSlice, "a slice is one pass of the block");
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) int32_t hist[];  // [nb] (to a multiple of 4), then the azimuths [kBinCache]
+    constexpr int W = THREADS / 32;
+    __shared__ int warp_tot[W];
+    __shared__ int slice_tot;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nb = bg.n_phi * bg.n_z;
+    const int nb4 = (nb + 3) & ~3;
+    float *cache = reinterpret_cast<float *>(hist + nb4);
+    const int64_t seg = blockIdx.x / kBinCluster;
+    const int64_t lo = seg_off[seg], hi = seg_off[seg + 1];
+    const int64_t part = (hi - lo + kBinCluster - 1) / kBinCluster;
+    const int64_t p0 = min(lo + rank * part, hi), p1 = min(p0 + part, hi);
+    for (int i = tid; i < nb4; i += THREADS) hist[i] = 0;
+    __syncthreads();
+    for (int64_t h0 = p0 + tid; h0 < p1; h0 += kBinUnroll * THREADS) {
+        float x[kBinUnroll], y[kBinUnroll], z[kBinUnroll];
+#pragma unroll
+        for (int k = 0; k < kBinUnroll; ++k) {
+            const int64_t h = h0 + k * THREADS;
+            if (h < p1) {
+                x[k] = hit_pos[h];
+                y[k] = hit_pos[H + h];
+                z[k] = hit_pos[2 * H + h];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kBinUnroll; ++k) {
+            const int64_t h = h0 + k * THREADS;
+            if (h < p1) {
+                const float phi = atan2f(y[k], x[k]);
+                if (h - p0 < kBinCache) cache[h - p0] = phi;
+                atomicAdd(&hist[hit_bin(phi, z[k], bg)], 1);
+            }
+        }
+    }
+    cluster.sync();
+    // this block's slice of the bins, four to a thread: each block's counts
+    // become its first place within the bin
+    const int per = ((nb + kBinCluster - 1) / kBinCluster + 3) & ~3;
+    const int b0 = rank * per + tid * kBinSlice;
+    const bool mine = tid * kBinSlice < per && b0 < nb4;
+    int4 tot = make_int4(0, 0, 0, 0);
+    if (mine) {
+#pragma unroll
+        for (int c = 0; c < kBinCluster; ++c) {
+            int4 *p = reinterpret_cast<int4 *>(cluster.map_shared_rank(hist, c) + b0);
+            const int4 n = *p;
+            *p = tot;
+            tot = make_int4(tot.x + n.x, tot.y + n.y, tot.z + n.z, tot.w + n.w);
+        }
+    }
+    const int sum = tot.x + tot.y + tot.z + tot.w;
+    int incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += o;
+    }
+    if (lane == 31) warp_tot[warp] = incl;
+    __syncthreads();
+    int at = incl - sum, all = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        if (w < warp) at += warp_tot[w];
+        all += warp_tot[w];
+    }
+    if (tid == 0) slice_tot = all;
+    cluster.sync();
+    for (int c = 0; c < rank; ++c) at += *cluster.map_shared_rank(&slice_tot, c);
+    int32_t *bo = bin_off + seg * (nb + 1);
+    if (mine) {
+        const int o[kBinSlice] = {at, at + tot.x, at + tot.x + tot.y, at + tot.x + tot.y + tot.z};
+#pragma unroll
+        for (int i = 0; i < kBinSlice; ++i)
+            if (b0 + i < nb) bo[b0 + i] = o[i];
+    }
+    if (rank == 0 && tid == 0) bo[nb] = (int)(hi - lo);
+    cluster.sync();
+    for (int i = tid; i < nb; i += THREADS) hist[i] += __ldcg(bo + i);
+    __syncthreads();
+    for (int64_t h0 = p0 + tid; h0 < p1; h0 += kBinUnroll * THREADS) {
+        float x[kBinUnroll], y[kBinUnroll], z[kBinUnroll];
+#pragma unroll
+        for (int k = 0; k < kBinUnroll; ++k) {
+            const int64_t h = h0 + k * THREADS;
+            if (h < p1) {
+                x[k] = hit_pos[h];
+                y[k] = hit_pos[H + h];
+                z[k] = hit_pos[2 * H + h];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kBinUnroll; ++k) {
+            const int64_t h = h0 + k * THREADS;
+            if (h < p1) {
+                const float phi = h - p0 < kBinCache ? cache[h - p0] : atan2f(y[k], x[k]);
+                const int p = atomicAdd(&hist[hit_bin(phi, z[k], bg)], 1);
+                if (p < (int)(hi - lo))  // always true: both passes bin a hit alike
+                    bkey[lo + p] = make_float4(phi, z[k], __int_as_float((int)(h - lo)),
+                                               sqrtf(x[k] * x[k] + y[k] * y[k]));
+            }
+        }
+    }
+}
+
 // Bin the hits of n_seg segments (seg_off on the device, [n_seg + 1], within
 // hit_pos [3][H]; max_seg the largest segment's hit count) into bkey and
 // bin_off [n_seg][nb + 1]; rank is scratch of H int32.
@@ -165,6 +297,15 @@ inline cudaError_t bin_hits(const int64_t *seg_off, int64_t n_seg, int64_t max_s
     if (n_seg <= 0) return cudaSuccess;
     const int nb = bg.n_phi * bg.n_z;
     if (nb < 1 || nb > kMaxBins) return cudaErrorInvalidValue;
+    if (n_seg * kBinCluster <= 2 * (int64_t)sm_count) {  // one wave of clusters
+        const bool wide = n_seg * kBinCluster <= sm_count;
+        const auto kern = wide ? bin_cluster_kernel<1024> : bin_cluster_kernel<512>;
+        const int bytes = ((nb + 3) / 4 * 4 + kBinCache) * (int)sizeof(int32_t);
+        const cudaError_t ec = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (ec != cudaSuccess) return ec;
+        kern<<<(unsigned)(n_seg * kBinCluster), wide ? 1024 : 512, bytes, stream>>>(seg_off, hit_pos, H, bg, bin_off, bkey);
+        return cudaGetLastError();
+    }
     const int smem = nb * (int)sizeof(int32_t);
     // the dynamic shared memory opt-in is a per-device attribute: set on every call
     cudaError_t e = cudaFuncSetAttribute(bin_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
