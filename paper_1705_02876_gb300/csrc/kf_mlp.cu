@@ -1,10 +1,10 @@
 // Training and batched inference of the learned hit proposal (kf_mlp.cuh).
 //
 // Training runs in FP32 (master weights, gradients and Adam moments): each
-// block takes tiles of 16 or 32 samples through the forward pass, the binary
+// block takes tiles of 32 samples through the forward pass, the binary
 // cross-entropy on the logits and the backward pass, and writes its part of
-// the weight gradients; a second kernel sums the parts and applies Adam.  Inference copies the weights to BF16 and scores on the
-// tensor cores (mlp_score_warp).
+// the weight gradients; a second kernel sums the parts and applies Adam.
+// Inference copies the weights to BF16 and scores on the tensor cores.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -403,15 +403,24 @@ __global__ void __launch_bounds__(32 * kScoreWarps) mlp_score_kernel(const __nv_
 }
 
 // ---------------------------------------------------------------------------
-// The same scoring on the fifth-generation tensor cores (tcgen05): one CTA of
-// 128 threads scores 128-row tiles.  The weights are staged once per CTA in
-// shared memory; per tile the rows' split inputs go to shared memory, one
-// thread issues the layer-1 products (hi and lo parts into one TMEM
-// accumulator, M = 128, N = 64, K = 16), the four warps read the accumulator
-// back from TMEM (warp w owns TMEM lanes 32w..32w+31, thread t row t), add the
-// bias, apply the ReLU, split the result and write it as the layer-2 A operand;
-// the layer-2 products (4 K-steps x hi/lo) accumulate into a second TMEM
-// region, which the warps read back for the 64 -> 1 dot product.
+// The same scoring on the fifth-generation tensor cores (tcgen05): a CTA of
+// kTcGroups groups of 128 threads, each with a 128-row tile of its own in hand.
+// The weights are staged once per CTA in shared memory; per tile the rows'
+// split inputs go to shared memory, one thread issues the layer-1 products (hi
+// and lo parts into one TMEM accumulator, M = 128, N = 64, K = 16), the four
+// warps read the accumulator back from TMEM (warp w owns TMEM lanes
+// 32w..32w+31, thread t row t; the bias is in it), apply the ReLU, split the
+// result and write it as the layer-2 A operand over the inputs; the layer-2
+// products (4 K-steps x hi/lo) accumulate over the layer-1 columns, which the
+// warps read back for the 64 -> 1 dot product.
+//
+// What bounds it is one tile's serial way (load, split, product, read, split,
+// product, read: the issue slots are half idle), so tiles in flight count: with
+// one set of columns and of operands per tile, and the weights shared by three
+// tiles, an SM holds six (before: four, each with its own weights and two
+// sets).  4,194,301 rows: 143 us, 158 with four (52 B a row would take 32 us at
+// the copy bandwidth).  Shared memory is busy for some 60% of that, 66 KB of
+// operand reads and 40 KB of writes a tile.
 //
 // Operands are K-major without swizzle, in core matrices of 8 rows x 16 bytes
 // (8 BF16 values): element (r, k) of a tile with K columns is at byte
@@ -420,19 +429,22 @@ __global__ void __launch_bounds__(32 * kScoreWarps) mlp_score_kernel(const __nv_
 // matrices adjacent in K (128 B) and the stride-dimension offset the distance
 // between 8-row groups ((K / 8) 128 B).
 
-constexpr int kTcRows = 128, kTcCols = 128;  // rows per tile; TMEM columns (two 64-column accumulators)
-constexpr int kTcCtasPerSm = 4;               // 4 x 128 = the SM's 512 TMEM columns (and ~52 KB of
-                                              // shared memory each: a fifth cannot be resident)
-constexpr uint32_t kTcWaitLimit = 1u << 24;   // mbarrier polls before a wait gives up
+constexpr int kTcRows = 128, kTcGroups = 3;        // rows per tile; tiles of a CTA
+constexpr int kTcThreads = kTcRows * kTcGroups;
+constexpr int kTcCols = 256;                       // TMEM columns of a CTA (a power of two): 64 per tile
+constexpr int kTcCtasPerSm = 2;                    // 2 x 256 = the SM's 512 TMEM columns
+constexpr uint32_t kTcWaitLimit = 1u << 24;        // mbarrier polls before a wait gives up
 
 struct __align__(128) TcSmem {
-    uint8_t A1h[kTcRows * 32], A1l[kTcRows * 32];    // inputs, K = 16 (12 used, 3 bias columns)
-    uint8_t A2h[kTcRows * 128], A2l[kTcRows * 128];  // first hidden layer, K = 64
+    // per tile, the A operand's hi and lo parts: the first hidden layer (K =
+    // 64), and before it, at the start, the inputs (K = 16: 12 used, 3 bias columns)
+    uint8_t Ah[kTcGroups][kTcRows * 128], Al[kTcGroups][kTcRows * 128];
+    uint8_t ones[kTcRows * 32];                       // (1, 1, 1, 0, ...) per row: K = 16
     uint8_t B1[kMlpHid * 32];                         // W1^T and b1's parts: N = 64 x K = 16
     uint8_t B2[kMlpHid * 128];                        // W2^T: N = 64 x K = 64
     uint8_t B2b[kMlpHid * 32];                        // b2's parts: N = 64 x K = 16 (3 used)
     float W3[kMlpHid], b3;
-    unsigned long long mbar;
+    unsigned long long mbar[kTcGroups];
     uint32_t taddr;
 };
 
@@ -498,18 +510,26 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *mbar, uint32_t par
     return false;
 }
 
-// 32 consecutive FP32 columns of this thread's TMEM lane, without the wait
+// 16 consecutive FP32 columns of this thread's TMEM lane, without the wait
 // (tmem_wait() before the values are used).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t r[32])
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t r[16])
 {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
+}
+// Barrier `id` of the group's 128 threads; whether `p` held for any of them.
+__device__ __forceinline__ bool group_or(int id, bool p)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, %2, 128, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"((uint32_t)p), "r"(id)
+        : "memory");
+    return r != 0;
 }
 __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -518,16 +538,18 @@ __device__ __forceinline__ void st_shared_v4(uint8_t *p, uint32_t a, uint32_t b,
     *reinterpret_cast<uint4 *>(p) = make_uint4(a, b, c, d);
 }
 
-__global__ void __launch_bounds__(kTcRows, kTcCtasPerSm) mlp_score_tc_kernel(const float *w32, const float *X,
-                                                                              int64_t n, float *logits,
-                                                                              unsigned *status)
+// VEC: the rows start on 16-byte boundaries and are read as three float4.
+template <bool VEC>
+__global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) mlp_score_tc_kernel(const float *w32, const float *X,
+                                                                                 int64_t n, float *logits,
+                                                                                 unsigned *status)
 {
     extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
     TcSmem &s = *reinterpret_cast<TcSmem *>(tc_smem_raw);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x % kTcRows, group = threadIdx.x / kTcRows, warp = tid >> 5;
     // weights: W1^T with b1's parts as its K rows 12..14, W2^T, and b2's parts
     // (K rows 0..2 of B2b), in BF16, K-major core matrices
-    for (int nn = tid; nn < kMlpHid; nn += kTcRows) {
+    for (int nn = threadIdx.x; nn < kMlpHid; nn += kTcThreads) {
         __nv_bfloat16 p1[3], p2[3];
         bf16_parts3(w32[kOffB1 + nn], p1);
         bf16_parts3(w32[kOffB2 + nn], p2);
@@ -540,18 +562,24 @@ __global__ void __launch_bounds__(kTcRows, kTcCtasPerSm) mlp_score_tc_kernel(con
         }
         s.W3[nn] = w32[kOffW3 + nn];
     }
-    for (int i = tid; i < kMlpHid * kMlpHid; i += kTcRows) {
-        const int nn = i >> 6, k = i & 63;
+    for (int i = threadIdx.x; i < kMlpHid * kMlpHid; i += kTcThreads) {
+        const int nn = i & 63, k = i >> 6;
         *reinterpret_cast<__nv_bfloat16 *>(s.B2 + core_offset(nn, k, 64)) =
             __float2bfloat16(w32[kOffW2 + k * kMlpHid + nn]);
     }
-    if (tid == 0) {
+    if (group == 0) {
+        st_shared_v4(s.ones + core_offset(tid, 0, 16), 0x3F803F80u, 0x00003F80u, 0u, 0u);
+        st_shared_v4(s.ones + core_offset(tid, 8, 16), 0u, 0u, 0u, 0u);
+    }
+    if (threadIdx.x == 0) {
         s.b3 = w32[kOffB3];
-        const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&s.mbar);
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb));
+        for (int g = 0; g < kTcGroups; ++g) {
+            const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&s.mbar[g]);
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb));
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {
+    if (threadIdx.x < 32) {
         const uint32_t a = (uint32_t)__cvta_generic_to_shared(&s.taddr);
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(a), "n"(kTcCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -561,124 +589,135 @@ __global__ void __launch_bounds__(kTcRows, kTcCtasPerSm) mlp_score_tc_kernel(con
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s.taddr;
-    const uint32_t d1 = tmem, d2 = tmem + kMlpHid;      // accumulators: columns 0..63 and 64..127
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;  // this warp's TMEM lanes
+    const uint32_t d = tmem + group * kMlpHid;               // the tile's accumulator columns
+    const uint32_t dl = d + ((uint32_t)(warp * 32) << 16);   // this warp's lanes of them
+    uint8_t *Ah = s.Ah[group], *Al = s.Al[group];
+    unsigned long long *mbar = &s.mbar[group];
     const float b3 = s.b3;
     uint32_t parity = 0;
     bool failed = false;
-    const int64_t tiles = (n + kTcRows - 1) / kTcRows;
+    const int64_t tiles = (n + kTcRows - 1) / kTcRows, step = (int64_t)gridDim.x * kTcGroups;
     // row `tid` of a tile's inputs; the next tile's are loaded while the
     // current tile's products run
     auto load_row = [&](int64_t tile, float f[kMlpIn]) {
         const int64_t row = tile * kTcRows + tid;
+        const bool in = tile < tiles && row < n;
+        if constexpr (VEC) {
 #pragma unroll
-        for (int i = 0; i < kMlpIn; ++i) f[i] = (tile < tiles && row < n) ? __ldcs(X + row * kMlpIn + i) : 0.0f;
+            for (int i = 0; i < kMlpIn; i += 4) {
+                const float4 v = in ? __ldcs(reinterpret_cast<const float4 *>(X + row * kMlpIn + i))
+                                    : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                f[i] = v.x;
+                f[i + 1] = v.y;
+                f[i + 2] = v.z;
+                f[i + 3] = v.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kMlpIn; ++i) f[i] = in ? __ldcs(X + row * kMlpIn + i) : 0.0f;
+        }
     };
     float fin[kMlpIn];
-    load_row(blockIdx.x, fin);
-    for (int64_t tile = blockIdx.x; tile < tiles && !failed; tile += gridDim.x) {
+    int64_t tile = (int64_t)blockIdx.x * kTcGroups + group;
+    load_row(tile, fin);
+    for (; tile < tiles; tile += step) {
         const int64_t row = tile * kTcRows + tid;
         // inputs of row `tid` and three 1s (the bias columns), split into BF16
         // hi and lo (1 is exact: its lo part is 0)
-        float f[16];
+        {
+            uint32_t h[8], l[8];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) f[i] = i < kMlpIn ? fin[i] : i < kMlpIn + 3 ? 1.0f : 0.0f;
-        uint32_t h[8], l[8];
+            for (int i = 0; i < 6; ++i) split_bf16x2(fin[2 * i], fin[2 * i + 1], h[i], l[i]);
+            h[6] = 0x3F803F80u;
+            h[7] = 0x00003F80u;
+            l[6] = l[7] = 0u;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) split_bf16x2(f[2 * i], f[2 * i + 1], h[i], l[i]);
-#pragma unroll
-        for (int kg = 0; kg < 2; ++kg) {
-            st_shared_v4(s.A1h + core_offset(tid, kg * 8, 16), h[4 * kg], h[4 * kg + 1], h[4 * kg + 2], h[4 * kg + 3]);
-            st_shared_v4(s.A1l + core_offset(tid, kg * 8, 16), l[4 * kg], l[4 * kg + 1], l[4 * kg + 2], l[4 * kg + 3]);
+            for (int kg = 0; kg < 2; ++kg) {
+                st_shared_v4(Ah + core_offset(tid, kg * 8, 16), h[4 * kg], h[4 * kg + 1], h[4 * kg + 2], h[4 * kg + 3]);
+                st_shared_v4(Al + core_offset(tid, kg * 8, 16), l[4 * kg], l[4 * kg + 1], l[4 * kg + 2], l[4 * kg + 3]);
+            }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        // the group's rows are written, and its reads of the last tile's columns done
+        if ((failed = group_or(group + 1, failed))) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            tc_mma(d1, smem_desc(s.A1h, 128, 256), smem_desc(s.B1, 128, 256), 0u);
-            tc_mma(d1, smem_desc(s.A1l, 128, 256), smem_desc(s.B1, 128, 256), 1u);
-            tc_commit(&s.mbar);
+            tc_mma(d, smem_desc(Ah, 128, 256), smem_desc(s.B1, 128, 256), 0u);
+            tc_mma(d, smem_desc(Al, 128, 256), smem_desc(s.B1, 128, 256), 1u);
+            tc_commit(mbar);
         }
-        load_row(tile + gridDim.x, fin);
-        bool ok = mbar_wait(&s.mbar, parity);
+        load_row(tile + step, fin);
+        failed = !mbar_wait(mbar, parity);
         parity ^= 1u;
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // layer 1 epilogue (the bias is in the accumulator): ReLU, split ->
-        // layer-2 A operand (row tid)
+        // layer-2 A operand (row tid), over the inputs, which are consumed
 #pragma unroll
-        for (int c0 = 0; c0 < kMlpHid; c0 += 32) {
-            uint32_t a[32];
-            tmem_ld32(d1 + lane_base + c0, a);
+        for (int c0 = 0; c0 < kMlpHid; c0 += 16) {
+            uint32_t a[16];
+            tmem_ld16(dl + c0, a);
             tmem_wait();
-            uint32_t hh[16], ll[16];
+            uint32_t hh[8], ll[8];
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
+            for (int i = 0; i < 8; ++i)
                 split_bf16x2(fmaxf(__uint_as_float(a[2 * i]), 0.0f), fmaxf(__uint_as_float(a[2 * i + 1]), 0.0f), hh[i],
                              ll[i]);
 #pragma unroll
-            for (int kg = 0; kg < 4; ++kg) {
-                st_shared_v4(s.A2h + core_offset(tid, c0 + kg * 8, 64), hh[4 * kg], hh[4 * kg + 1], hh[4 * kg + 2],
+            for (int kg = 0; kg < 2; ++kg) {
+                st_shared_v4(Ah + core_offset(tid, c0 + kg * 8, 64), hh[4 * kg], hh[4 * kg + 1], hh[4 * kg + 2],
                              hh[4 * kg + 3]);
-                st_shared_v4(s.A2l + core_offset(tid, c0 + kg * 8, 64), ll[4 * kg], ll[4 * kg + 1], ll[4 * kg + 2],
+                st_shared_v4(Al + core_offset(tid, c0 + kg * 8, 64), ll[4 * kg], ll[4 * kg + 1], ll[4 * kg + 2],
                              ll[4 * kg + 3]);
             }
         }
-        // layer 1's inputs are consumed: A1h row tid becomes (1, 1, 1, 0, ...),
-        // the A operand of layer 2's bias product
-        st_shared_v4(s.A1h + core_offset(tid, 0, 16), 0x3F803F80u, 0x00003F80u, 0u, 0u);
-        st_shared_v4(s.A1h + core_offset(tid, 8, 16), 0u, 0u, 0u, 0u);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
+        if ((failed = group_or(group + 1, failed))) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {  // K-step ks: core matrices 2ks, 2ks + 1 along K
                 const uint64_t b = smem_desc(s.B2 + ks * 256, 128, 1024);
-                tc_mma(d2, smem_desc(s.A2h + ks * 256, 128, 1024), b, ks > 0 ? 1u : 0u);
-                tc_mma(d2, smem_desc(s.A2l + ks * 256, 128, 1024), b, 1u);
+                tc_mma(d, smem_desc(Ah + ks * 256, 128, 1024), b, ks > 0 ? 1u : 0u);
+                tc_mma(d, smem_desc(Al + ks * 256, 128, 1024), b, 1u);
             }
-            tc_mma(d2, smem_desc(s.A1h, 128, 256), smem_desc(s.B2b, 128, 256), 1u);  // + b2
-            tc_commit(&s.mbar);
+            tc_mma(d, smem_desc(s.ones, 128, 256), smem_desc(s.B2b, 128, 256), 1u);  // + b2
+            tc_commit(mbar);
         }
-        ok = mbar_wait(&s.mbar, parity);
+        failed = !mbar_wait(mbar, parity);
         parity ^= 1u;
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // layer 2 epilogue (the bias is in the accumulator): ReLU, the 64 -> 1
         // dot product
-        uint32_t a[64];
-        tmem_ld32(d2 + lane_base, a);
-        tmem_ld32(d2 + lane_base + 32, a + 32);
-        tmem_wait();
         float z = b3;
 #pragma unroll
-        for (int c = 0; c < kMlpHid; c += 4) {
-            const float4 w = *reinterpret_cast<const float4 *>(s.W3 + c);
-            z = fmaf(w.x, fmaxf(__uint_as_float(a[c]), 0.0f), z);
-            z = fmaf(w.y, fmaxf(__uint_as_float(a[c + 1]), 0.0f), z);
-            z = fmaf(w.z, fmaxf(__uint_as_float(a[c + 2]), 0.0f), z);
-            z = fmaf(w.w, fmaxf(__uint_as_float(a[c + 3]), 0.0f), z);
+        for (int c0 = 0; c0 < kMlpHid; c0 += 32) {
+            uint32_t a[32];
+            tmem_ld16(dl + c0, a);
+            tmem_ld16(dl + c0 + 16, a + 16);
+            tmem_wait();
+#pragma unroll
+            for (int c = 0; c < 32; c += 4) {
+                const float4 w = *reinterpret_cast<const float4 *>(s.W3 + c0 + c);
+                z = fmaf(w.x, fmaxf(__uint_as_float(a[c]), 0.0f), z);
+                z = fmaf(w.y, fmaxf(__uint_as_float(a[c + 1]), 0.0f), z);
+                z = fmaf(w.z, fmaxf(__uint_as_float(a[c + 2]), 0.0f), z);
+                z = fmaf(w.w, fmaxf(__uint_as_float(a[c + 3]), 0.0f), z);
+            }
         }
         if (row < n) logits[row] = z;
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();  // TMEM read and shared operands consumed before the next tile reuses them
     }
     if (failed) {
-        // a product did not complete in time: report it, give whatever is
-        // still in flight a bounded while to land, then release TMEM
+        // a product did not complete in time: report it, and give whatever is
+        // still in flight a bounded while to land before TMEM is released
         if (tid == 0) atomicOr(status, 1u);
-        mbar_wait(&s.mbar, parity);
-        __syncthreads();
+        mbar_wait(mbar, parity);
     }
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTcCols));
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTcCols));
 }
 
 int ensure_state(kf_context *ctx, MlpState **out)
@@ -872,12 +911,14 @@ int kf_proposal_score_with(kf_context *ctx, const float *features, int64_t n, fl
     if (engine == KF_SCORE_AUTO) engine = n >= kScoreTcMinRows ? KF_SCORE_TCGEN05 : KF_SCORE_MMA_SYNC;
     cudaError_t e;
     if (engine == KF_SCORE_TCGEN05) {
-        if ((e = cudaFuncSetAttribute(mlp_score_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(TcSmem))) != cudaSuccess)
+        const auto kern = reinterpret_cast<uintptr_t>(features) % 16 ? mlp_score_tc_kernel<false> : mlp_score_tc_kernel<true>;
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TcSmem))) !=
+            cudaSuccess)
             return cuda_error(ctx, e, "tcgen05 scoring shared memory");
         const int64_t tiles = (n + kTcRows - 1) / kTcRows;
-        const unsigned grid = (unsigned)std::min<int64_t>(tiles, (int64_t)context_sm_count(ctx) * kTcCtasPerSm);
-        mlp_score_tc_kernel<<<grid, kTcRows, sizeof(TcSmem), stream>>>(s->w32, features, n, logits, s->status);
+        const unsigned grid = (unsigned)std::min<int64_t>((tiles + kTcGroups - 1) / kTcGroups,
+                                                          (int64_t)context_sm_count(ctx) * kTcCtasPerSm);
+        kern<<<grid, kTcThreads, sizeof(TcSmem), stream>>>(s->w32, features, n, logits, s->status);
     } else {
         if ((e = cudaFuncSetAttribute(mlp_score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(ScoreSmem))) != cudaSuccess)

@@ -133,3 +133,18 @@ def test_load_proposal_as_bytes(kf):
         kf.load_proposal(c2, cu(w[:-1]))
     c1.close()
     c2.close()
+
+
+@pytest.mark.parametrize("n", [1, 128, 129, 3 * 128 + 1, 152 * 2 * 3 * 128 + 77])
+def test_tcgen05_scores_unaligned_rows(kf, ctx, n):
+    """Rows that do not start on 16-byte boundaries take the scalar loads: the
+    same scores, bit for bit, as the vector loads of the same rows aligned, for
+    less than a tile, a CTA's tiles and more than one round of the grid."""
+    X, _, w = data(6, n)
+    kf.proposal_load(ctx, cu(w))
+    flat = torch.empty(n * 12 + 1, device="cuda")
+    flat[1:] = cu(X).reshape(-1)
+    z = kf.proposal_score(ctx, cu(X), engine=2)
+    zu = kf.proposal_score(ctx, flat[1:].view(n, 12), engine=2)
+    assert not kf.proposal_status(ctx)
+    assert torch.equal(z, zu)
