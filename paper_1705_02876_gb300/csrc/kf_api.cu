@@ -96,8 +96,8 @@ Routing make_routing(const kf_options &o)
     Routing rt;
     rt.mode = o.precision_mode;
     rt.det_min = 6.75f / o.cond_max;
-    rt.pt_lo = o.pt_lo;
-    rt.pt_hi = o.pt_hi;
+    rt.pt_lo2 = o.pt_lo * o.pt_lo;
+    rt.pt_hi2 = o.pt_hi * o.pt_hi;
     rt.gain_max = o.gain_max;
     return rt;
 }

@@ -24,10 +24,11 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 // Fit track base + off over every layer in order (the steps and stop rules are
 // those of kf_fit_tracks in kf.h).  base is the block's: the addresses of every
-// array are then a uniform pointer and the thread's offset.  Hits are loaded
-// DEPTH layers ahead of their update:
-// DEPTH = 1 into registers, through pointers advanced by one layer's stride;
-// DEPTH >= 2 by asynchronous copies (cp.async, one commit group per layer,
+// array are then a uniform pointer and the thread's offset.  A layer's hit is
+// loaded ahead of its update: DEPTH = 1 into registers, at the start of the
+// layer (the step and the transport, 250 instructions, cover the latency; a
+// layer earlier cost nine registers and as many moves a layer); DEPTH >= 2
+// layers ahead, by asynchronous copies (cp.async, one commit group per layer,
 // empty for a layer without a hit) into this thread's column of a ring of
 // DEPTH + 1 shared-memory stages of 9 floats each ([stage * 9 + i][stride]),
 // so that the loads in flight hold no registers.  A non-finite value in a
@@ -93,9 +94,8 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
     if (!at_seed) {
         for (int l = 0; l < g.L; ++l) {
             const bool has = (mask >> l) & 1u;
-            float mn[3] = {0, 0, 0}, vn[6] = {0, 0, 0, 0, 0, 0};
             if constexpr (DEPTH == 1) {
-                if (l + 1 < g.L) load_hit(mn, vn);
+                if (l > 0) load_hit(m, v);
             } else {
                 issue();                 // layer l + DEPTH
                 cp_async_wait<DEPTH>();  // layer l's group has landed
@@ -139,12 +139,6 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
                     if (st >= 2) flags |= KF_FLAG_FP64_PATH;
                     if (st == 3) flags |= KF_FLAG_PSD_REPAIRED;
                 }
-            }
-            if constexpr (DEPTH == 1) {
-#pragma unroll
-                for (int i = 0; i < 3; ++i) m[i] = mn[i];
-#pragma unroll
-                for (int i = 0; i < 6; ++i) v[i] = vn[i];
             }
         }
     }

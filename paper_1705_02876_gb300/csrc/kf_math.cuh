@@ -69,27 +69,27 @@ __device__ __forceinline__ bool crossing(float x, float y, float tx, float ty, f
     const float D = fmaf(r, r, -fmaf(x, x, y * y));
     const float Bp = fmaf(-0.25f * om * om, D, fmaf(om, w, 1.0f));
     const float Qd = fmaf(u, u, D * Bp);
-    if (!(Qd >= 0.0f) || !(pt2 > 0.0f)) return false;
-    const float sq = sqrtf(Qd);
-    float s, tau, sigma;
-    if (u + sq > 0.0f) {
-        sigma = __fdividef(D, u + sq);
-        tau = 0.5f * om * sigma;
-        const float t2 = tau * tau;
+    const float sq = sqrtf(Qd), den = u + sq;
+    // one test for the common case: a missed cylinder (Qd < 0) or no transverse
+    // momentum makes den NaN
+    float sigma = __fdividef(D, den);
+    float tau = 0.5f * om * sigma;
+    const float t2 = tau * tau;
+    float s;
+    if (den > 0.0f && t2 < 0.0625f) {
         // atan(tau)/tau: its Taylor series sum_k (-t2)^k / (2k+1) to t2^6 for
-        // |tau| < 1/4 (truncation below 3e-10), else the library atanf
-        float ratio;
-        if (t2 < 0.0625f) {
-            ratio = fmaf(t2, -1.0f / 13.0f, 1.0f / 11.0f);
-            ratio = fmaf(t2, -ratio, 1.0f / 9.0f);
-            ratio = fmaf(t2, -ratio, 1.0f / 7.0f);
-            ratio = fmaf(t2, -ratio, 1.0f / 5.0f);
-            ratio = fmaf(t2, -ratio, 1.0f / 3.0f);
-            ratio = fmaf(t2, -ratio, 1.0f);
-        } else {
-            ratio = atanf(tau) / tau;
-        }
+        // |tau| < 1/4 (truncation below 3e-10)
+        float ratio = fmaf(t2, -1.0f / 13.0f, 1.0f / 11.0f);
+        ratio = fmaf(t2, -ratio, 1.0f / 9.0f);
+        ratio = fmaf(t2, -ratio, 1.0f / 7.0f);
+        ratio = fmaf(t2, -ratio, 1.0f / 5.0f);
+        ratio = fmaf(t2, -ratio, 1.0f / 3.0f);
+        ratio = fmaf(t2, -ratio, 1.0f);
         s = sigma * ratio;
+    } else if (!(Qd >= 0.0f) || !(pt2 > 0.0f)) {
+        return false;
+    } else if (den > 0.0f) {
+        s = sigma * (atanf(tau) / tau);  // a wide turn
     } else {
         // A start moving inwards: both roots of the quadratic, each mapped to
         // its smallest positive path length.
@@ -566,7 +566,7 @@ static __device__ __noinline__ int update_ext(float *slot, int stride, int kind)
 struct Routing {
     int mode;        // 0 FP32, 1 routed
     float det_min;   // 27 / (4 cond_max): the least det of S's correlation matrix done in FP32
-    float pt_lo, pt_hi;
+    float pt_lo2, pt_hi2;  // squares of the pT bounds
     float gain_max;  // information-gain threshold: C_ii / V_ii above it routes the gain
 };
 
@@ -814,7 +814,7 @@ __device__ __forceinline__ int update_local(Local &p, float c[15], const float m
         const float pt2 = fmaf(p.q1, p.q1, p.q2 * p.q2);
         if (ill)
             kind = 2;
-        else if (pt2 < rt.pt_lo * rt.pt_lo || pt2 > rt.pt_hi * rt.pt_hi)
+        else if (pt2 < rt.pt_lo2 || pt2 > rt.pt_hi2)
             kind = 3;
         else if (rt.gain_max > 0.0f && (tt * c[pk(0, 0)] > rt.gain_max * v[0] || nn * c[pk(0, 0)] > rt.gain_max * v[2] ||
                                         c[pk(1, 1)] > rt.gain_max * v[5]))

@@ -85,11 +85,10 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const FitGeom g, const R
     }
     int K = 0;
     for (int l = 0; l < L && go; ++l) {
-        const bool has = (mask >> l) & 1u, has_next = l + 1 < L && ((mask >> (l + 1)) & 1u);
-        float mn[3], vn[6];
+        const bool has = (mask >> l) & 1u;
+        if (l > 0 && has) load_hit(m, v);  // the step and the transport cover the latency
         hp += 3 * T;
         hc += 6 * T;
-        if (has_next) load_hit(mn, vn);
         if (l > 0) {
             LocalJac J;
             const uint32_t stop = step_local(p, qkb, g.r[l], g.inv_r[l], g.z_half, J, pn);
@@ -124,12 +123,6 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const FitGeom g, const R
             oc[(int64_t)(21 * l + 16) * T] = p.ny;
             oc[(int64_t)(21 * l + 17) * T] = p.f0;
             oc[(int64_t)(21 * l + 18) * T] = p.f1;
-        }
-        if (has_next) {
-#pragma unroll
-            for (int i = 0; i < 3; ++i) m[i] = mn[i];
-#pragma unroll
-            for (int i = 0; i < 6; ++i) v[i] = vn[i];
         }
     }
     io.out_reached[t] = (int16_t)K;
