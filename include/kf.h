@@ -198,8 +198,9 @@ int kf_fit_tracks(kf_context *ctx, const kf_geometry *geom, int64_t n_tracks,
  * Device staging (about 3 x 591 B x chunk_tracks at 10 layers) is kept by the
  * context and grown on demand (KF_ERR_NOMEM).  opt->launch_mode is ignored;
  * the shape is opt->tracks_per_block / opt->reg_cap / opt->hit_prefetch when
- * set, else 64 tracks per block, 128 registers and the register prefetch (no
- * tuning runs).
+ * set (the others then 64 tracks per block, 128 registers and the register
+ * prefetch); with none set, 128 registers and, in place, hits four layers
+ * ahead and 64 tracks per block, 256 from 20,000 tracks on (no tuning runs).
  */
 int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int64_t n_tracks, const float *seed_state,
                        const float *seed_cov, const int8_t *charge, const float *hit_pos, const float *hit_cov,

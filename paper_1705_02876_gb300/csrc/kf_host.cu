@@ -95,10 +95,12 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
         (rc = check_ptr(ctx, out_chi2, 4, "out_chi2")) || (rc = check_ptr(ctx, out_ndof, 2, "out_ndof")) ||
         (rc = check_ptr(ctx, out_flags, 4, "out_flags")))
         return rc;
-    const int block = o.tracks_per_block ? o.tracks_per_block : 64;
-    const int cap = o.reg_cap < 0 ? 0 : (o.reg_cap ? o.reg_cap : 128);
+    // the shape asked for, or with none of its parts asked for the path's own
+    const bool own_shape = !o.tracks_per_block && !o.reg_cap && !o.hit_prefetch;
+    int block = o.tracks_per_block ? o.tracks_per_block : 64;
+    int cap = o.reg_cap < 0 ? 0 : (o.reg_cap ? o.reg_cap : 128);
+    int depth = o.hit_prefetch ? o.hit_prefetch : 1;
     DeviceGuard dg(context_device(ctx));
-    const int depth = o.hit_prefetch ? o.hit_prefetch : 1;
     const int usable = fit_shape_usable(block, cap, depth);
     if (usable < 1)
         return set_error(ctx, KF_ERR_ARG, "no fit of %d tracks per block, cap %d, hit prefetch %d", block, cap, depth);
@@ -153,6 +155,16 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
                            static_cast<int16_t *>(dev[9]),
                            static_cast<uint32_t *>(dev[10])};
             cudaStream_t s = hp->stream[0];
+            if (own_shape) {
+                // the link's latency is a layer's work several times over: hits
+                // four layers ahead, and for large batches blocks wide enough
+                // that their rows are 1 KB each (10 layers: 1,000 tracks 34.5 us
+                // with 64 tracks, one layer ahead, 31.5 four ahead; 131,071
+                // tracks 452, 426, and 408 us with 256 tracks; 64 and 256 tracks
+                // meet at 20,000)
+                block = n_tracks < 20000 ? 64 : 256;
+                depth = 4;
+            }
             const cudaError_t e = launch_fit_tuned(g, rt, io, block, cap, depth, context_sm_count(ctx),
                                                    reinterpret_cast<unsigned *>(hp->work), s);
             const cudaError_t e2 = cudaStreamSynchronize(s);
