@@ -103,6 +103,7 @@ struct BuildParams {
     int N;
     float chi2_cut, nsigma, sig_rphi2, sig_z2, max_dphi, max_dz;
     int64_t S, H;
+    int seeds_per_warp;  // at most 32 / G
     int n_events;
     int event_base;    // seed_event values are event_base + the event's index in ev_off
     int64_t hit_base;  // added to the written hit indices (ev_off holds batch-local offsets)
@@ -437,7 +438,6 @@ __global__ void flagged_seeds_kernel(const int32_t *flag, int64_t S, int32_t *li
 template <int G, int MODE>
 __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
 {
-    constexpr int SEEDS_PER_WARP = 32 / G;
     // a lane's child list (it gives at most N <= kMaxN hit children) and the
     // first scan's buffer: kMaxN entries each (lists sized to G measured no
     // faster: their shorter loops cost the plain kernel spills at 128 registers)
@@ -455,9 +455,9 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int slot = lane % G, gbase = lane - slot;
-    // G = 6: five groups per warp; lanes 30 and 31 form an idle group of two
-    const bool lane_ok = lane < SEEDS_PER_WARP * G;
-    const int64_t k_seed = ((int64_t)blockIdx.x * 4 + warp) * SEEDS_PER_WARP + lane / G;
+    // lanes beyond the warp's seeds idle (G = 6: at least 30 and 31)
+    const bool lane_ok = lane < p.seeds_per_warp * G;
+    const int64_t k_seed = ((int64_t)blockIdx.x * 4 + warp) * p.seeds_per_warp + lane / G;
     int64_t s = k_seed;
     bool seed_ok = lane_ok && k_seed < p.S;
     if (p.seed_list) {  // the listed seeds only; a warp without one has nothing to do
@@ -1018,7 +1018,14 @@ int build_run(kf_context *ctx, const FitGeom &g, const kf_options &o, const Buil
     // lanes per seed: the smallest group that holds N candidates (6 for N = 5
     // or 6, so that a warp holds five seeds instead of four)
     const int G = p.N == 1 ? 1 : p.N <= 2 ? 2 : p.N <= 4 ? 4 : p.N <= 6 ? 6 : 8;
-    const int64_t seeds_per_block = 4 * (32 / G);
+    // Seeds per warp: all that fit, 32 / G, but no more than fill the GPU once
+    // (four blocks of four warps per SM).  A warp takes as long as its slowest
+    // lane at every step of every layer, so with SMs to spare fewer seeds share
+    // one: an event of 5,000 seeds, its seed fit included, takes 150 us with three
+    // per warp (417 blocks) and 156 with five (250).
+    p.seeds_per_warp = (int)std::min<int64_t>(
+        32 / G, std::max<int64_t>(1, (b.n_seeds + 16 * context_sm_count(ctx) - 1) / (16 * context_sm_count(ctx))));
+    const int64_t seeds_per_block = 4 * p.seeds_per_warp;
     const unsigned grid = (unsigned)((b.n_seeds + seeds_per_block - 1) / seeds_per_block);
     const int mode = o.use_proposal ? kModeProposal : log ? kModeLog : kModePlain;
     const int smem_plain = (int)build_smem_base(L);
