@@ -133,8 +133,8 @@ typedef struct {
 void kf_options_default(kf_options *opt);
 
 /* Create a context on CUDA device `device` (requires compute capability
- * 10.3).  The context owns scratch memory, the autotuner's choices, captured
- * CUDA graphs and the proposal network's weights. */
+ * 10.3).  The context owns scratch memory, the autotuner's choices
+ * and the proposal network's weights. */
 int kf_context_create(kf_context **ctx, int device);
 void kf_context_destroy(kf_context *ctx);
 
@@ -475,7 +475,7 @@ int kf_seed_fetch(kf_context *ctx, const kf_geometry *geom, const float *hit_pos
  * forward pass is kf_fit_tracks' per-track fit (routed precision as set in
  * opt); the backward pass is the Rauch-Tung-Striebel recursion in each layer's
  * local coordinates (t, z, px, py, pz), where the covariances are positive
- * definite, with Cp^-1 from a Cholesky factorisation scaled to unit diagonal.
+ * definite, with Cp^-1 from an L D L^T factorisation.
  *
  * Inputs: the layouts of kf_fit_tracks (device, caller-owned).
  * Outputs (device, caller-owned): out_state [L][6][T] and out_cov [L][21][T]
