@@ -369,9 +369,10 @@ __global__ void to_bf16_kernel(float *w32, __nv_bfloat16 *W1t, __nv_bfloat16 *W2
 
 constexpr int kScoreWarps = 4, kScoreLd = 12;
 // kf_proposal_score's engine (KF_SCORE_AUTO), chosen by measurement on one
-// GB300: mma.sync below this many rows (at 65,536 rows 0.015 against 0.025
-// ms), tcgen05 from it on (1.24x faster at 2^20 rows, 1.68x at 2^24)
-constexpr int64_t kScoreTcMinRows = 262144;
+// GB300: mma.sync below this many rows (65,536 rows 9.3 against 11.2 us), tcgen05
+// from it on (131,072 rows 12.9 against 13.3 us, 163,840 12.9 and 16.6, 262,144
+// 17.4 and 24.0, 2^24 537 and 1,146)
+constexpr int64_t kScoreTcMinRows = 131072;
 
 struct ScoreSmem {
     MlpSmemWeights w;

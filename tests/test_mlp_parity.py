@@ -148,3 +148,13 @@ def test_tcgen05_scores_unaligned_rows(kf, ctx, n):
     zu = kf.proposal_score(ctx, flat[1:].view(n, 12), engine=2)
     assert not kf.proposal_status(ctx)
     assert torch.equal(z, zu)
+
+
+@pytest.mark.parametrize("n,engine", [(131_071, 1), (131_072, 2)])
+def test_automatic_engine_line(kf, ctx, n, engine):
+    """The automatic choice takes mma.sync below 131,072 rows and tcgen05 from
+    there on: the scores are that engine's, bit for bit."""
+    X, _, w = data(7, n)
+    kf.proposal_load(ctx, cu(w))
+    x = cu(X)
+    assert torch.equal(kf.proposal_score(ctx, x), kf.proposal_score(ctx, x, engine=engine))
