@@ -108,9 +108,10 @@ typedef struct {
     int tracks_per_block;    /* 0 = autotuned, else 32, 64, 128 or 256 */
     int reg_cap;             /* registers per thread of the fit: 0 = autotuned,
                                 -1 = uncapped, 168, 128, 96 or 80 */
-    int hit_prefetch;        /* layers of hits the fit loads ahead of their
-                                update: 0 = autotuned, 1 = the next layer into registers,
-                                2 or 4 = through a ring in shared memory (cp.async) */
+    int hit_prefetch;        /* how far ahead of its update the fit loads a hit:
+                                0 = autotuned, 1 = at the start of its layer, into registers,
+                                2 or 4 = that many layers, through a ring in shared memory
+                                (cp.async) */
     /* building */
     int max_cands;           /* N candidates kept per seed, 1 (best hit) .. 8 */
     float chi2_cut;          /* hits with a larger chi2 increment are incompatible */

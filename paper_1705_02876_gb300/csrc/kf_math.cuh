@@ -1,6 +1,7 @@
 // Per-track Kalman-filter arithmetic in registers (Sections 2, 2.1 and 4.2 of
-// arXiv:1705.02876): one thread owns one track's state x[6] and its packed
-// covariance c[21]; every function below works on those registers.
+// arXiv:1705.02876): one thread owns one track, its position, momentum and the
+// packed covariance c[15] of its local coordinates (from a seed, the Cartesian
+// state x[6] and c[21]); every function below works on those registers.
 //
 // Packed symmetric storage: lower triangle row by row, index(i,j) = i(i+1)/2+j.
 #pragma once
