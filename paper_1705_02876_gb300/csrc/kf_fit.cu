@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256) fit_plain_kernel(const FitGeom g, const R
 // behind, fits these tracks from their seeds in full warps (none: it returns
 // at once).  With one track in eight above pt_hi (1,000,000 tracks, pT
 // log-uniform 0.24 to 500 GeV) nearly every warp held one and stopped for it
-// at every layer: 7.09 ms in line in FP64, 1.03 ms put off in FP64, 0.32 ms
+// at every layer: 7.09 ms in line in FP64, 1.03 ms put off in FP64, 0.31 ms
 // in float-float.  Without that code this kernel also needs fewer registers
 // (96 with the ring, no spills).
 constexpr uint32_t kPutOff = 0x80000000u;
@@ -208,9 +208,12 @@ __global__ void __launch_bounds__(BLOCK, MINB) fit_kernel(const FitGeom g, const
 }
 
 // The tracks put off by the launch before: a block gathers them from the flags
-// of its chunks of the batch until it has one per thread, and fits those.
-constexpr int kExtBlock = 128;
-__global__ void __launch_bounds__(kExtBlock, 4) fit_extended_kernel(const FitGeom g, const Routing rt, const FitIO io,
+// of its chunks of the batch until it has one per thread, and fits those.  Two
+// blocks of 256 threads per SM: the fewer blocks gather, the fewer end on a part
+// of one (1,000,000 stress tracks: 307 us in all; 324 with four blocks of 128,
+// 330 and 342 with 64 and 32 threads).
+constexpr int kExtBlock = 256;
+__global__ void __launch_bounds__(kExtBlock, 2) fit_extended_kernel(const FitGeom g, const Routing rt, const FitIO io,
                                                                      unsigned *work)
 {
     __shared__ float slots[kSlotSize * kExtBlock];
@@ -342,7 +345,7 @@ cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &i
     sh->fn<<<(unsigned)grid, block, ring_bytes(block, depth), stream>>>(g, rt, io, work);
     if ((e = cudaGetLastError()) != cudaSuccess || rt.mode == 0) return e;  // without routing no track is put off
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<int64_t>((io.T + kExtBlock - 1) / kExtBlock, (int64_t)sm_count * 4));
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>((io.T + kExtBlock - 1) / kExtBlock, (int64_t)sm_count * 2));
     cfg.blockDim = dim3(kExtBlock);
     cfg.stream = stream;
     cudaLaunchAttribute at;

@@ -1,7 +1,7 @@
 """Tracks put off to the second launch of a fit (those that need FP64) against
 the same tracks with the FP64 update in line (KF_LAUNCH_FLAT): the same
 arithmetic in another launch, so every output is equal bit for bit.  Sizes on
-both sides of the one-launch limit (32,768 tracks), of the gathering blocks (128
+both sides of the one-launch limit (32,768 tracks), of the gathering blocks (256
 tracks) and with every, some, and no track put off; each batch runs twice, and
 the batch after it finds the counters cleared."""
 import numpy as np
@@ -20,7 +20,7 @@ def kf():
     return kf_
 
 
-@pytest.mark.parametrize("n", [1, 127, 32767, 32768, 32897, 40_001])
+@pytest.mark.parametrize("n", [1, 255, 32767, 32768, 33025, 40_001])
 def test_put_off_equals_in_line(kf, n):
     ctx = kf.Context(0)
     for lo, hi, share in ((260.0, 500.0, (0.9, 1.0)), (50.0, 500.0, (0.05, 0.95)), (1.0, 5.0, (0.0, 0.01))):
