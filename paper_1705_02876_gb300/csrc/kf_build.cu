@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(128, 4) build_kernel(const BuildParams p)
         for (int i = 0; i < 6; ++i) x6[i] = p.seed_state[i * p.S + s];
 #pragma unroll
         for (int i = 0; i < 21; ++i) c6[i] = p.seed_cov[i * p.S + s];
-        flags = enter_local(x6, c6, qkb, p.g.r[0], p.g.inv_r[0], p.g.z_half, t, c, pn);
+        flags = enter_local(x6, c6, qkb, p.g.r[0], p.g.inv_r[0], p.g.z_half, p.rt, slots + threadIdx.x, 128, t, c, pn);
         stopped = flags != 0u;
     }
     const bool at_seed = stopped;  // no layer reached: the seed's one candidate, all holes, stays the seed

@@ -34,8 +34,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // so that the loads in flight hold no registers.  A non-finite value in a
 // used hit makes the chi2 increment non-finite, or makes S fail its positive
 // definiteness test, so the hit is tested only then.
-// DEFER: at the first update that needs extended precision the track is given
-// up and true returned (nothing is written).
+// DEFER: a track outside the pT bounds on the first layer, and any other at the
+// first update that needs extended precision, is given up and true returned
+// (nothing is written).
 template <int DEPTH, bool DEFER, class OFF>
 __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, const FitIO &io, int64_t base, OFF off,
                                           float *slot, int stride, float *ring = nullptr)
@@ -89,9 +90,13 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
     Local p;
     float c[15], pn;
     bool deferred = false;
-    if (!flags) flags = enter_local(sx, sc, qkb, g.r[0], g.inv_r[0], g.z_half, p, c, pn);
+    if (!flags) flags = enter_local<DEFER>(sx, sc, qkb, g.r[0], g.inv_r[0], g.z_half, rt, slot, stride, p, c, pn);
+    if (DEFER && flags == kPutOff) {
+        deferred = true;
+        flags = 0u;
+    }
     const bool at_seed = flags != 0u;  // no layer reached
-    if (!at_seed) {
+    if (!at_seed && !deferred) {
         for (int l = 0; l < g.L; ++l) {
             const bool has = (mask >> l) & 1u;
             if constexpr (DEPTH == 1) {
@@ -190,8 +195,6 @@ __global__ void __launch_bounds__(256) fit_plain_kernel(const FitGeom g, const R
 // at every layer: 7.09 ms in line in FP64, 1.03 ms put off in FP64, 0.31 ms
 // in float-float.  Without that code this kernel also needs fewer registers
 // (96 with the ring, no spills).
-constexpr uint32_t kPutOff = 0x80000000u;
-
 template <int BLOCK, int MINB, int DEPTH>
 __global__ void __launch_bounds__(BLOCK, MINB) fit_kernel(const FitGeom g, const Routing rt, const FitIO io,
                                                            unsigned *work)

@@ -29,17 +29,6 @@ __device__ __forceinline__ bool all_finite(const float *v)
 // Divisions on the FP32 path use __fdividef (reciprocal approximation and a
 // multiply, within 2 ulp for divisors of magnitude 2^-126..2^126, which every
 // divisor here is) in place of the IEEE-rounded sequence.
-//
-// Propagation result and the non-trivial part of its Jacobian.  With
-// P = {x, y, px, py} (state indices 0, 1, 3, 4), J has the block structure
-//   J[P][P] = T (4x4), J[z][P] = jz (4), J[z][z] = 1, J[z][pz] = jzpz,
-//   J[P][z] = J[P][pz] = 0, J[pz] = e_pz,
-// because the crossing of a z-parallel cylinder does not depend on z or pz.
-struct Jac {
-    float T[4][4];
-    float jz[4];
-    float jzpz;
-};
 
 // Helix propagation to the first forward crossing of radius r (uniform field
 // along z; transverse path length s, omega = q k Bz / pT).  Writing
@@ -123,113 +112,21 @@ __device__ __forceinline__ bool crossing(float x, float y, float tx, float ty, f
     return true;
 }
 
-__device__ __forceinline__ bool propagate(const float x[6], float qkb, float r, float xn[6], Jac &J)
+struct Routing {
+    int mode;        // 0 FP32, 1 routed
+    float det_min;   // 27 / (4 cond_max): the least det of S's correlation matrix done in FP32
+    float pt_lo2, pt_hi2;  // squares of the pT bounds
+    float gain_max;  // information-gain threshold: C_ii / V_ii above it routes the gain
+};
+
+// A track whose updates run in extended precision whatever its hits are.
+__device__ __forceinline__ bool outside_pt(float pt2, const Routing &rt)
 {
-    const float px = x[3], py = x[4], pz = x[5];
-    const float pt2 = fmaf(px, px, py * py);
-    const float ipt = rsqrtf(pt2);
-    const float tx = px * ipt, ty = py * ipt;
-    const float om = qkb * ipt;
-    Turn t;
-    if (!crossing(x[0], x[1], tx, ty, om, pt2, r, t)) return false;
-    const float s = t.s, a = t.a, b = t.b, sn = t.sn, c = t.c;
-    xn[0] = x[0] + fmaf(tx, a, ty * b);
-    xn[1] = x[1] + fmaf(ty, a, -tx * b);
-    xn[2] = fmaf(pz * s, ipt, x[2]);
-    xn[3] = fmaf(px, c, py * sn);
-    xn[4] = fmaf(py, c, -px * sn);
-    xn[5] = pz;
-    const float phi = om * s;
-    const float txn = xn[3] * ipt, tyn = xn[4] * ipt;
-    // D = dF/dx0 at fixed s (phi depends on pT through omega)
-    const float d03 = fmaf(-s * tx, txn, a) * ipt, d04 = fmaf(-s * ty, txn, b) * ipt;
-    const float d13 = fmaf(-s * tx, tyn, -b) * ipt, d14 = fmaf(-s * ty, tyn, a) * ipt;
-    const float d33 = fmaf(-phi * tx, tyn, c), d34 = fmaf(-phi * ty, tyn, sn);
-    const float d43 = fmaf(phi * tx, txn, -sn), d44 = fmaf(phi * ty, txn, c);
-    const float lz = pz * ipt;  // dz/ds
-    const float d23 = -s * lz * tx * ipt, d24 = -s * lz * ty * ipt;
-    // ds/dx0 from the constraint x'^2 + y'^2 = r^2
-    const float iden = __fdividef(-1.0f, fmaf(xn[0], txn, xn[1] * tyn));
-    const float ds[4] = {xn[0] * iden, xn[1] * iden, fmaf(xn[0], d03, xn[1] * d13) * iden,
-                         fmaf(xn[0], d04, xn[1] * d14) * iden};
-    const float f[4] = {txn, tyn, om * xn[4], -om * xn[3]};  // dF/ds on P
-    const float d[4][4] = {{1.0f, 0.0f, d03, d04}, {0.0f, 1.0f, d13, d14}, {0.0f, 0.0f, d33, d34}, {0.0f, 0.0f, d43, d44}};
-    const float dz[4] = {0.0f, 0.0f, d23, d24};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) J.T[i][j] = fmaf(f[i], ds[j], d[i][j]);
-        J.jz[j] = fmaf(lz, ds[j], dz[j]);
-    }
-    J.jzpz = s * ipt;
-    return true;
+    return rt.mode == 1 && (pt2 < rt.pt_lo2 || pt2 > rt.pt_hi2);
 }
 
-// C <- J C J^T using the block structure of J (178 FMA instead of 432 for a
-// dense 6x6 triple product on the packed lower triangle).
-__device__ __forceinline__ void transport(const Jac &J, float c[21])
-{
-    constexpr int P[4] = {0, 1, 3, 4};
-    float A[4][4];  // A = T C[P][P]
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            float acc = 0.0f;
-#pragma unroll
-            for (int n = 0; n < 4; ++n) acc = fmaf(J.T[k][n], c[pk(P[n], P[m])], acc);
-            A[k][m] = acc;
-        }
-    float w[4], w2 = c[pk(2, 2)], w5 = c[pk(5, 2)];  // W = row z of J times C
-    w2 = fmaf(J.jzpz, c[pk(5, 2)], w2);
-    w5 = fmaf(J.jzpz, c[pk(5, 5)], c[pk(5, 2)]);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        float acc = fmaf(J.jzpz, c[pk(5, P[m])], c[pk(2, P[m])]);
-#pragma unroll
-        for (int n = 0; n < 4; ++n) acc = fmaf(J.jz[n], c[pk(P[n], P[m])], acc);
-        w[m] = acc;
-    }
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-        w2 = fmaf(J.jz[n], c[pk(P[n], 2)], w2);
-        w5 = fmaf(J.jz[n], c[pk(P[n], 5)], w5);
-    }
-    float c5[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int n = 0; n < 4; ++n) acc = fmaf(c[pk(5, P[n])], J.T[m][n], acc);
-        c5[m] = acc;
-    }
-    float nc[21];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int m = 0; m <= k; ++m) {
-            float acc = 0.0f;
-#pragma unroll
-            for (int n = 0; n < 4; ++n) acc = fmaf(A[k][n], J.T[m][n], acc);
-            nc[pk(P[k], P[m])] = acc;
-        }
-    float c22 = w2;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int n = 0; n < 4; ++n) acc = fmaf(w[n], J.T[m][n], acc);
-        nc[pk(2, P[m])] = acc;
-        c22 = fmaf(J.jz[m], w[m], c22);
-    }
-    nc[pk(2, 2)] = fmaf(J.jzpz, w5, c22);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) nc[pk(5, P[m])] = c5[m];
-    nc[pk(5, 2)] = w5;
-    nc[pk(5, 5)] = c[pk(5, 5)];
-#pragma unroll
-    for (int i = 0; i < 21; ++i) c[i] = nc[i];
-}
+// What a fit that puts such tracks off (DEFER below) gets in place of flags.
+constexpr uint32_t kPutOff = 0x80000000u;
 
 // The extended-precision paths are out of line and rare.  A non-inlined
 // function's registers count towards the kernel's allocation, so these work
@@ -564,13 +461,6 @@ static __device__ __noinline__ int update_ext(float *slot, int stride, int kind)
     return kind == 2 ? update_fp64(slot, stride) : kind == 3 ? update_wide(slot, stride) : update_ff(slot, stride);
 }
 
-struct Routing {
-    int mode;        // 0 FP32, 1 routed
-    float det_min;   // 27 / (4 cond_max): the least det of S's correlation matrix done in FP32
-    float pt_lo2, pt_hi2;  // squares of the pT bounds
-    float gain_max;  // information-gain threshold: C_ii / V_ii above it routes the gain
-};
-
 // ---------------------------------------------------------------------------
 // The filter on the covariance of a track's local coordinates.  On a
 // cylinder the crossing cannot move along the radial direction, so the
@@ -698,43 +588,138 @@ __device__ __forceinline__ void transport_local(const LocalJac &J, float c[15])
     c[pk(P, V)] = fmaf(J.W2, lp, c[pk(P, V)]);
 }
 
-// The step from a start anywhere (a seed) with a full 6x6 covariance onto the
-// first layer; the turning frame starts as the laboratory's.  Returns as
-// step_local does (x, c as they were when it fails).
-__device__ __forceinline__ uint32_t enter_local(const float x[6], float c6[21], float qkb, float r, float inv_r,
-                                                float z_half, Local &p, float c[15], float &pn)
+// The bending plane's block of enter_local (tt, q2 t, q2 q2) in float-float, on
+// the slot: the covariance of (x, y, px, py), packed, then the rows t and q2
+// over them; the block is left at the slot's start.
+static __device__ __noinline__ void enter_wide(float *s, int stride)
 {
-    float xn[6];
-    Jac J;
-    if (!propagate(x, qkb, r, xn, J)) return KF_FLAG_UNREACHABLE;
-    if (fabsf(xn[2]) > z_half) return KF_FLAG_LEFT_BARREL;
-    transport(J, c6);
-    const float pt2 = fmaf(xn[3], xn[3], xn[4] * xn[4]), ipt = rsqrtf(pt2);
-    const float f0 = xn[3] * ipt, f1 = xn[4] * ipt;
-    const float nx = xn[0] * inv_r, ny = xn[1] * inv_r;
-    p = Local{xn[0], xn[1], xn[2], fmaf(f0, xn[3], f1 * xn[4]), fmaf(f0, xn[4], -f1 * xn[3]), xn[5], f0, f1, nx, ny};
-    // rows t, z, pz against (t, z, px, py, pz), then the momentum columns turned
-    auto lt = [&](int j) { return fmaf(nx, c6[pk(j, 1)], -ny * c6[pk(j, 0)]); };
-    auto qu = [&](float a, float b) { return fmaf(f0, a, f1 * b); };
-    auto qv = [&](float a, float b) { return fmaf(f0, b, -f1 * a); };
-    c[pk(0, 0)] = fmaf(ny * ny, c6[pk(0, 0)], fmaf(-2.0f * nx * ny, c6[pk(1, 0)], nx * nx * c6[pk(1, 1)]));
-    c[pk(1, 0)] = lt(2);
-    c[pk(1, 1)] = c6[pk(2, 2)];
-    const float tu = lt(3), tv = lt(4);
-    c[pk(2, 0)] = qu(tu, tv);
-    c[pk(3, 0)] = qv(tu, tv);
-    c[pk(4, 0)] = lt(5);
-    c[pk(2, 1)] = qu(c6[pk(3, 2)], c6[pk(4, 2)]);
-    c[pk(3, 1)] = qv(c6[pk(3, 2)], c6[pk(4, 2)]);
-    c[pk(4, 1)] = c6[pk(5, 2)];
-    const float ux = qu(c6[pk(3, 3)], c6[pk(4, 3)]), uy = qu(c6[pk(4, 3)], c6[pk(4, 4)]);
-    c[pk(2, 2)] = qu(ux, uy);
-    c[pk(3, 2)] = qv(ux, uy);
-    c[pk(3, 3)] = qv(qv(c6[pk(3, 3)], c6[pk(4, 3)]), qv(c6[pk(4, 3)], c6[pk(4, 4)]));
-    c[pk(4, 2)] = qu(c6[pk(5, 3)], c6[pk(5, 4)]);
-    c[pk(4, 3)] = qv(c6[pk(5, 3)], c6[pk(5, 4)]);
+    auto dot = [&](const ff m[4], int row) {  // the row . m
+        ff p[4];
+        float lo = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float v = s[(row + j) * stride];
+            p[j] = two_prod(m[j].hi, v);
+            lo = __fadd_rn(lo, __fmaf_rn(m[j].lo, v, p[j].lo));
+        }
+        const ff a = two_sum(p[0].hi, p[1].hi), b = two_sum(a.hi, p[2].hi), c = two_sum(b.hi, p[3].hi);
+        return two_sum(c.hi, __fadd_rn(lo, __fadd_rn(a.lo, __fadd_rn(b.lo, c.lo))));
+    };
+    constexpr int T = 10, Q = 14;
+    float out[3];
+#pragma unroll 1
+    for (int row = T; row <= Q; row += Q - T) {
+        ff m[4];  // the row times the covariance
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const ff col[4] = {{s[pk(0, i) * stride], 0.0f}, {s[pk(1, i) * stride], 0.0f},
+                               {s[pk(2, i) * stride], 0.0f}, {s[pk(3, i) * stride], 0.0f}};
+            m[i] = dot(col, row);
+        }
+        if (row == T) out[0] = dot(m, T).hi;
+        out[row == T ? 1 : 2] = dot(m, Q).hi;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) s[i * stride] = out[i];
+}
+
+// The step from a start anywhere (a seed) with a full 6x6 covariance onto the
+// first layer; the turning frame starts along the seed's momentum.  Returns as
+// step_local does.  The rows of the Jacobian are those of LocalJac with a
+// displacement (dx, dy) in place of the start's dt (lambda = -n1 . (dx, dy) / cn
+// + ..., t' = that' x (dx, dy) / cn + ...), on the Cartesian coordinates, so that
+// an entry of the local covariance comes from the seed's in one pass.
+// A hit after a seed shrinks q2's variance to what t leaves of it, a small
+// difference of the bending plane's three entries: their sums run from the
+// positions' terms to the momenta's, which exceed them, and are in float-float
+// for a track outside the pT bounds, whose updates are too.  (Through the 6x6
+// covariance on the layer, rotated, an entry had some ten roundings.  Error of
+// the fitted covariance against 64 bits, five hits, pT 0.5 to 10 GeV: 11.6e-6,
+// now 9.3e-6; pT 0.24 to 500 GeV: 6.0e-4, with the sums alone 4.7e-4, now
+// 3.9e-4; three hits 3.9e-4, 3.0e-4, 2.5e-4.)
+// DEFER: kPutOff for such a track, which is left where it was.
+template <bool DEFER = false>
+__device__ __forceinline__ uint32_t enter_local(const float x[6], const float c6[21], float qkb, float r, float inv_r,
+                                                float z_half, const Routing &rt, float *slot, int stride, Local &p,
+                                                float c[15], float &pn)
+{
+    const float pt2 = fmaf(x[3], x[3], x[4] * x[4]);
+    const float ipt = rsqrtf(pt2);
+    const float om = qkb * ipt;
+    const float tx = x[3] * ipt, ty = x[4] * ipt;
+    Turn t;
+    if (!crossing(x[0], x[1], tx, ty, om, pt2, r, t)) return KF_FLAG_UNREACHABLE;
+    const float jp = t.s * ipt;
+    const float z1 = fmaf(x[5], jp, x[2]);
+    if (fabsf(z1) > z_half) return KF_FLAG_LEFT_BARREL;
+    const bool wide = outside_pt(pt2, rt);
+    if (DEFER && wide) return kPutOff;
+    const float x1 = x[0] + fmaf(tx, t.a, ty * t.b), y1 = x[1] + fmaf(ty, t.a, -tx * t.b);
+    const float ux = fmaf(tx, t.c, ty * t.sn), uy = fmaf(ty, t.c, -tx * t.sn);  // that'
+    const float nx = x1 * inv_r, ny = y1 * inv_r;
+    const float cn = fmaf(nx, ux, ny * uy), se = fmaf(ny, ux, -nx * uy);
+    const float icn = __fdividef(1.0f, cn), k = se * icn;
+    const float lx = -nx * icn, ly = -ny * icn;
+    const float l1 = -ipt * fmaf(t.b, k, t.a), l2 = -ipt * fmaf(t.a, k, -t.b);
+    const float a1 = ipt * icn * t.b, a2 = ipt * icn * t.a;
+    const float l3 = fmaf(l1, tx, -l2 * ty), l4 = fmaf(l1, ty, l2 * tx);
+    const float lz = x[5] * ipt;
+    // rows over (x, y, px, py): t, q2 and z (which has 1 for z and jp for pz
+    // too); q1's is (tx, ty) over (px, py)
+    const float T[4] = {-uy * icn, ux * icn, fmaf(a1, tx, -a2 * ty), fmaf(a1, ty, a2 * tx)};
+    const float Q[4] = {-qkb * lx, -qkb * ly, fmaf(-qkb, l3, -ty), fmaf(-qkb, l4, tx)};
+    const float Z[4] = {lz * lx, lz * ly, lz * l3, lz * l4};
+    auto row4 = [&](const float *v, int j) {
+        return fmaf(v[3], c6[pk(4, j)], fmaf(v[2], c6[pk(3, j)], fmaf(v[1], c6[pk(1, j)], v[0] * c6[pk(0, j)])));
+    };
+    float tc[6], zc[6], uc[6], vc[6];  // the rows times the covariance
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        tc[j] = row4(T, j);
+        zc[j] = fmaf(jp, c6[pk(5, j)], c6[pk(2, j)] + row4(Z, j));
+        uc[j] = fmaf(ty, c6[pk(4, j)], tx * c6[pk(3, j)]);
+        vc[j] = row4(Q, j);
+    }
+    auto on4 = [&](const float *m, const float *v) {
+        return fmaf(m[4], v[3], fmaf(m[3], v[2], fmaf(m[1], v[1], m[0] * v[0])));
+    };
+    auto onz = [&](const float *m) { return fmaf(m[5], jp, m[2] + on4(m, Z)); };
+    auto onu = [&](const float *m) { return fmaf(m[4], ty, m[3] * tx); };
+    c[pk(0, 0)] = on4(tc, T);
+    c[pk(1, 0)] = onz(tc);
+    c[pk(1, 1)] = onz(zc);
+    c[pk(2, 0)] = onu(tc);
+    c[pk(2, 1)] = onu(zc);
+    c[pk(2, 2)] = onu(uc);
+    c[pk(3, 0)] = on4(tc, Q);
+    c[pk(3, 1)] = on4(zc, Q);
+    c[pk(3, 2)] = on4(uc, Q);
+    c[pk(3, 3)] = on4(vc, Q);
+    c[pk(4, 0)] = tc[5];
+    c[pk(4, 1)] = zc[5];
+    c[pk(4, 2)] = uc[5];
+    c[pk(4, 3)] = vc[5];
     c[pk(4, 4)] = c6[pk(5, 5)];
-    pn = fabsf(fmaf(xn[3], p.nx, xn[4] * p.ny));
+    if constexpr (!DEFER) {
+        if (wide) {
+            constexpr int P[4] = {0, 1, 3, 4};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j <= i; ++j) slot[pk(i, j) * stride] = c6[pk(P[i], P[j])];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                slot[(10 + i) * stride] = T[i];
+                slot[(14 + i) * stride] = Q[i];
+            }
+            enter_wide(slot, stride);
+            c[pk(0, 0)] = slot[0];
+            c[pk(3, 0)] = slot[stride];
+            c[pk(3, 3)] = slot[2 * stride];
+        }
+    }
+    p = Local{x1, y1, z1, pt2 * ipt, 0.0f, x[5], ux, uy, nx, ny};
+    pn = fabsf(cn) * pt2 * ipt;
     return 0u;
 }
 
@@ -815,7 +800,7 @@ __device__ __forceinline__ int update_local(Local &p, float c[15], const float m
         const float pt2 = fmaf(p.q1, p.q1, p.q2 * p.q2);
         if (ill)
             kind = 2;
-        else if (pt2 < rt.pt_lo2 || pt2 > rt.pt_hi2)
+        else if (outside_pt(pt2, rt))
             kind = 3;
         else if (rt.gain_max > 0.0f && (tt * c[pk(0, 0)] > rt.gain_max * v[0] || nn * c[pk(0, 0)] > rt.gain_max * v[2] ||
                                         c[pk(1, 1)] > rt.gain_max * v[5]))

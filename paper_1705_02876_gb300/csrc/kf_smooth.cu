@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const FitGeom g, const R
         for (int i = 0; i < 21; ++i) c6[i] = __ldcs(io.seed_cov + i * T + t);
         if (mask & 1u) load_hit(m, v);
         flags = (all_finite<6>(x6) && all_finite<21>(c6)) ? 0u : (uint32_t)KF_FLAG_NAN_INPUT;
-        if (!flags) flags = enter_local(x6, c6, qkb, g.r[0], g.inv_r[0], g.z_half, p, c, pn);
+        if (!flags) flags = enter_local(x6, c6, qkb, g.r[0], g.inv_r[0], g.z_half, rt, slot, stride, p, c, pn);
         go = flags == 0u;
     }
     int K = 0;

@@ -1,0 +1,48 @@
+// The per-track arithmetic of csrc/kf_math.cuh compiled for the host, for tests
+// of single steps without a GPU: CUDA's qualifiers are empty and its device
+// functions are the C library's (the approximate ones within their error).
+#include <math.h>
+#include <stdint.h>
+
+#define __device__
+#define __host__
+#define __forceinline__ inline
+#define __noinline__
+static inline float __fdividef(float a, float b) { return a / b; }
+static inline float rsqrtf(float a) { return (float)(1.0 / sqrt((double)a)); }
+#define __logf logf
+static inline float __fadd_rn(float a, float b) { return a + b; }
+static inline float __fsub_rn(float a, float b) { return a - b; }
+static inline float __fmul_rn(float a, float b) { return a * b; }
+static inline float __fmaf_rn(float a, float b, float c) { return fmaf(a, b, c); }
+
+#include "kf_math.cuh"
+
+using namespace kf;
+
+static Routing routing(const float *opt)  // routed, cond_max, pt_lo, pt_hi, gain_max
+{
+    Routing rt{};
+    rt.mode = (int)opt[0];
+    rt.det_min = 6.75f / opt[1];
+    rt.pt_lo2 = opt[2] * opt[2];
+    rt.pt_hi2 = opt[3] * opt[3];
+    rt.gain_max = opt[4];
+    return rt;
+}
+
+// enter_local of n seeds [6][n], [21][n] to radius r: flags [n] and the local
+// covariances [15][n].
+extern "C" void host_enter(int64_t n, const float *state, const float *cov, const int8_t *charge, float qk, float r,
+                           float z_half, const float *opt, float *out, uint32_t *flags)
+{
+    const Routing rt = routing(opt);
+    for (int64_t t = 0; t < n; ++t) {
+        float x[6], c6[21], c[15], slot[kSlotSize], pn;
+        for (int i = 0; i < 6; ++i) x[i] = state[i * n + t];
+        for (int i = 0; i < 21; ++i) c6[i] = cov[i * n + t];
+        Local p{};
+        flags[t] = enter_local(x, c6, charge[t] * qk, r, 1.0f / r, z_half, rt, slot, 1, p, c, pn);
+        for (int i = 0; i < 15; ++i) out[i * n + t] = flags[t] ? NAN : c[i];
+    }
+}

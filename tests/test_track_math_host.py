@@ -1,0 +1,72 @@
+"""Single steps of the library's per-track arithmetic (csrc/kf_math.cuh),
+compiled for the host, against the FP64 oracle."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1705_02876_gb300 import synth
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+EPS = 2.0 ** -24  # half an ulp of FP32, relative
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="no g++")
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("host") / "track_math.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-ffp-contract=off", "-w",
+                    "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_1705_02876_gb300", "csrc"),
+                    "-o", so, os.path.join(HERE, "host", "track_math.cpp")], check=True)
+    return ctypes.CDLL(so)
+
+
+def _p(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def _opt(mode=1, cond_max=1e4, pt_lo=0.25, pt_hi=200.0, gain_max=0.0):
+    return np.array([mode, cond_max, pt_lo, pt_hi, gain_max], np.float32)
+
+
+def test_seed_covariance_on_the_first_layer(host, oracle):
+    """What the first hit's t leaves of q2's variance, vv - vt^2 / tt, from a
+    seed's covariance on the first layer: a small difference of terms of size vv
+    (tt and vt^2 / tt are no larger in it), which the fit's covariance inherits.
+    Each entry rounded once, by EPS / sqrt(3) of itself in the root mean square,
+    puts it off by sqrt(1 + 4 + 1) EPS / sqrt(3) = sqrt(2) EPS vv; the sums' own
+    roundings stay below that, in FP32 and further below in float-float (tracks
+    outside the pT bounds)."""
+    n = 3000
+    b = synth.make_fit_batch(5, [n], pt_lo=0.24, pt_hi=500.0, pt_dist="loguniform", eta_max=1.5)
+    g = b.geom
+    r = float(np.float32(g.radii[0]))
+    c, fl = {}, np.empty(n, np.uint32)
+    for name, opt in (("float-float", _opt(pt_lo=1e3, pt_hi=2e3)), ("FP32", _opt(mode=0))):
+        c[name] = np.empty((15, n), np.float32)
+        host.host_enter(ctypes.c_int64(n), _p(b.seed_state), _p(b.seed_cov), _p(b.charge),
+                        ctypes.c_float(0.00299792458 * g.bz), ctypes.c_float(r), ctypes.c_float(g.z_half), _p(opt),
+                        _p(c[name]), _p(fl))
+    rel = {k: [] for k in c}
+    il = np.tril_indices(6)
+    for t in np.nonzero(fl == 0)[0]:
+        ok, x, J, _ = oracle.propagate(b.seed_state[:, t], int(b.charge[t]), float(np.float32(g.bz)), r)
+        assert ok
+        C = np.zeros((6, 6))
+        C[il] = b.seed_cov[:, t]
+        C = J @ (C + C.T - np.diag(np.diag(C))) @ J.T
+        R, pt = np.hypot(x[0], x[1]), np.hypot(x[3], x[4])
+        ut, uv = np.zeros(6), np.zeros(6)
+        ut[:2] = -x[1] / R, x[0] / R
+        uv[3:5] = -x[4] / pt, x[3] / pt
+        tt, vt, vv = ut @ C @ ut, uv @ C @ ut, uv @ C @ uv
+        for k in c:
+            ctt, cvt, cvv = c[k][[0, 6, 9], t].astype(np.float64)
+            rel[k].append((cvv - cvt ** 2 / ctt - (vv - vt ** 2 / tt)) / (EPS * vv))
+    assert len(rel["FP32"]) > 0.9 * n
+    rms = {k: float(np.sqrt(np.mean(np.square(v)))) for k, v in rel.items()}
+    assert rms["FP32"] <= np.sqrt(2) and rms["float-float"] <= 0.9 * rms["FP32"], rms
