@@ -355,8 +355,8 @@ static __device__ __noinline__ int update_ff(float *slot_p, int stride)
 // The whole update in float-float: update_fp64 to 2^-46 instead of 2^-53, for
 // well-conditioned S (cond_2(R) <= cond_max, the caller's test), where the
 // FP32 results it leaves are the same but for rounding ties.  Some 1,100 FP32
-// instructions, about a tenth of the time of the FP64 pipe's 280.  Returns 2 or
-// 3 (repaired).
+// instructions, about a tenth of the time of the FP64 pipe's 280.  Returns as
+// update_fp64 does.
 __device__ __forceinline__ ff ff_sub(ff x, ff y) { return ff_add(x, ff_neg(y)); }
 __device__ __forceinline__ ff ff_addf(ff x, float y)
 {
@@ -399,10 +399,13 @@ static __device__ __noinline__ int update_wide(float *slot_p, int stride)
         ia = ff_rcp(vnn);
         vt = ff_mul(vnt, ia);
         vz = ff_mul(vnz, ia);
-        it = ff_rcp(ff_sub(ff_addf(vtt, sl.c(0, 0)), ff_mul(vnt, vt)));
+        const ff dt = ff_sub(ff_addf(vtt, sl.c(0, 0)), ff_mul(vnt, vt));
+        it = ff_rcp(dt);
         const ff e = ff_sub(ff_addf(vtz, sl.c(1, 0)), ff_mul(vnt, vz));
         l = ff_mul(e, it);
-        iz = ff_rcp(ff_sub(ff_sub(two_sum(sl.c(1, 1), sl.v(5)), ff_mul(vnz, vz)), ff_mul(l, e)));
+        const ff dz = ff_sub(ff_sub(two_sum(sl.c(1, 1), sl.v(5)), ff_mul(vnz, vz)), ff_mul(l, e));
+        iz = ff_rcp(dz);
+        if (!(vnn.hi > 0.0f && dt.hi > 0.0f && dz.hi > 0.0f && dz.hi < INFINITY)) return 1;
     }
     const float X0 = sl.x(0), X1 = sl.x(1), X2 = sl.x(2);
     ff w1, w2;

@@ -46,3 +46,24 @@ extern "C" void host_enter(int64_t n, const float *state, const float *cov, cons
         for (int i = 0; i < 15; ++i) out[i * n + t] = flags[t] ? NAN : c[i];
     }
 }
+
+// One update on the slot by the routine of `kind` (1 float-float gain, 2 FP64,
+// 3 float-float): n of x [6][n] (position, q1, q2, pz), c [15][n], nx and ny,
+// hits m [3][n] and v [6][n]; x and c in place, chi2 and the routine's result.
+extern "C" void host_slot_update(int kind, int64_t n, float *x, float *c, const float *nrm, const float *m, const float *v,
+                                 float *chi2, int32_t *st)
+{
+    for (int64_t t = 0; t < n; ++t) {
+        float s[kSlotSize] = {};
+        for (int i = 0; i < 6; ++i) s[kSlotX + i] = x[i * n + t];
+        for (int i = 0; i < 15; ++i) s[kSlotC + i] = c[i * n + t];
+        for (int i = 0; i < 3; ++i) s[kSlotM + i] = m[i * n + t];
+        for (int i = 0; i < 6; ++i) s[kSlotV + i] = v[i * n + t];
+        s[kSlotFrame + 2] = nrm[t];
+        s[kSlotFrame + 3] = nrm[n + t];
+        st[t] = update_ext(s, 1, kind);
+        for (int i = 0; i < 6; ++i) x[i * n + t] = s[kSlotX + i];
+        for (int i = 0; i < 15; ++i) c[i * n + t] = s[kSlotC + i];
+        chi2[t] = s[kSlotChi2];
+    }
+}

@@ -70,3 +70,51 @@ def test_seed_covariance_on_the_first_layer(host, oracle):
     assert len(rel["FP32"]) > 0.9 * n
     rms = {k: float(np.sqrt(np.mean(np.square(v)))) for k, v in rel.items()}
     assert rms["FP32"] <= np.sqrt(2) and rms["float-float"] <= 0.9 * rms["FP32"], rms
+
+
+def _updates(rng, n):
+    """n local states, covariances and hits: x [6][n], c [15][n], n [2][n], m [3][n], v [6][n]."""
+    A = rng.normal(size=(n, 5, 5)) * np.array([1e-2, 0.1, 1e-2, 1e-2, 0.1])[:, None]
+    C = A @ A.transpose(0, 2, 1)
+    il = np.tril_indices(5)
+    phi = rng.uniform(0, 2 * np.pi, n)
+    nrm = np.stack([np.cos(phi), np.sin(phi)])
+    x = np.concatenate([4 * nrm, rng.normal(size=(1, n)), rng.normal(size=(3, n))])
+    m = x[:3] + 0.01 * rng.normal(size=(3, n))
+    v = np.zeros((6, n))
+    v[0] = v[2] = 1e-4
+    v[5] = 1e-2
+    return [np.ascontiguousarray(a, dtype=np.float32) for a in (x, C[:, il[0], il[1]].T, nrm, m, v)]
+
+
+def _slot_update(host, kind, x, c, nrm, m, v):
+    n = x.shape[1]
+    x, c, chi2, st = x.copy(), c.copy(), np.empty(n, np.float32), np.empty(n, np.int32)
+    host.host_slot_update(kind, ctypes.c_int64(n), _p(x), _p(c), _p(nrm), _p(m), _p(v), _p(chi2), _p(st))
+    return st, x, c, chi2
+
+
+def test_float_float_update_tells_a_bad_s(host):
+    """A hit covariance whose t pivot, C_tt + V_tt - V_nt^2 / V_nn, lies within
+    some FP32 ulps of zero on either side (float-float resolves 2^-46 of its
+    terms, here it is 2^-28 and more): the float-float update refuses what the
+    FP64 one refuses, with the state and covariance left alone, and agrees with
+    it on the rest."""
+    n = 4000
+    rng = np.random.default_rng(3)
+    x, c, nrm, m, v = _updates(rng, n)
+    nrm[0], nrm[1] = 1, 0
+    c[[0, 1, 3, 6, 10]] = 0
+    c[0] = (1e-9 * rng.uniform(1, 2, n)).astype(np.float32)
+    a = rng.uniform(0.5, 1, n).astype(np.float32)
+    v[0], v[1] = 1, a
+    v[2] = (a.astype(np.float64) ** 2 * (1 + 2.0 ** -23 * rng.integers(-3, 4, n))).astype(np.float32)
+    pivot = c[0].astype(np.float64) + v[2] - a.astype(np.float64) ** 2
+    sel = np.abs(pivot) > 2.0 ** -28
+    assert (pivot[sel] < 0).sum() > 500 and (pivot[sel] > 0).sum() > 500
+    st2 = _slot_update(host, 2, x, c, nrm, m, v)[0]
+    st3, x3, c3, _ = _slot_update(host, 3, x, c, nrm, m, v)
+    assert (st2[sel] == np.where(pivot[sel] > 0, 2, 1)).all()
+    assert np.array_equal(st3[sel], st2[sel])
+    bad = st3 == 1
+    assert np.array_equal(x3[:, bad], x[:, bad]) and np.array_equal(c3[:, bad], c[:, bad])
