@@ -100,7 +100,9 @@ typedef struct {
                                 diagonal) with det R < 27 / (4 cond_max) runs in FP64, so
                                 every FP32 update has cond_2(R) <= cond_max */
     float pt_lo, pt_hi;      /* tracks with pT outside [pt_lo, pt_hi] GeV update in float-float
-                                (46 bits and more throughout) where S is well conditioned */
+                                (45 bits of every term), and in FP64 where S is ill-conditioned
+                                or the prediction's variance along t or z more than 2^20 times
+                                the hit's */
     float gain_max;          /* > 0: an update with C_ii > gain_max V_ii (i = x, y, z) forms
                                 its gain (S^-1 and K) in float-float; 0 = off */
     /* launch shape (fit) */

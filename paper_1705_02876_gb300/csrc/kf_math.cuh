@@ -352,11 +352,13 @@ static __device__ __noinline__ int update_ff(float *slot_p, int stride)
     return 2;
 }
 
-// The whole update in float-float: update_fp64 to 2^-46 instead of 2^-53, for
-// well-conditioned S (cond_2(R) <= cond_max, the caller's test), where the
-// FP32 results it leaves are the same but for rounding ties.  Some 1,100 FP32
-// instructions, about a tenth of the time of the FP64 pipe's 280.  Returns as
-// update_fp64 does.
+// The whole update in float-float: update_fp64 to some 2^-45 of its terms
+// instead of 2^-52.  What a hit leaves of a variance C is about V: a result is
+// off by 2^-45 C / V of itself, so that with C below kWideGain V (and S well
+// conditioned, both the caller's tests) the FP32 results are those of the FP64
+// update but for rounding ties.  Some 1,100 FP32 instructions, about a tenth
+// of the time of the FP64 pipe's 280.  Returns as update_fp64 does.
+constexpr float kWideGain = 1048576.0f;  // 2^20: 2^-25, half an FP32 half-ulp
 __device__ __forceinline__ ff ff_sub(ff x, ff y) { return ff_add(x, ff_neg(y)); }
 __device__ __forceinline__ ff ff_addf(ff x, float y)
 {
@@ -771,7 +773,8 @@ __device__ __forceinline__ void scatter_local(const Local &p, float theta2, floa
 //     cond_2(R) by cond_max on the FP32 path; the spread of S's diagonal, V_nn
 //     << C_zz, is harmless);
 //   * else, when pT lies outside [pt_lo, pt_hi], it is redone in float-float
-//     (update_wide);
+//     (update_wide), or in FP64 after all where the hit is more than a million
+//     times as precise as the prediction (kWideGain, against V's t and z pivots);
 //   * with gain_max > 0, the gain is formed in float-float (update_ff) when
 //     C_ii > gain_max V_ii for some i.
 // Returns 0 updated in FP32, 2 updated with extended-precision arithmetic,
@@ -803,8 +806,12 @@ __device__ __forceinline__ int update_local(Local &p, float c[15], const float m
         const float pt2 = fmaf(p.q1, p.q1, p.q2 * p.q2);
         if (ill)
             kind = 2;
-        else if (outside_pt(pt2, rt))
-            kind = 3;
+        else if (outside_pt(pt2, rt)) {
+            // V's t and z pivots: its variances given n, and given n and t
+            const float vdt = fmaf(-vnt, vt, vtt), ve = fmaf(-vnt, vz, vtz);
+            const float vdz = fmaf(-__fdividef(ve, vdt), ve, fmaf(-vnz, vz, v[5]));
+            kind = c[pk(0, 0)] < kWideGain * vdt && c[pk(1, 1)] < kWideGain * vdz ? 3 : 2;
+        }
         else if (rt.gain_max > 0.0f && (tt * c[pk(0, 0)] > rt.gain_max * v[0] || nn * c[pk(0, 0)] > rt.gain_max * v[2] ||
                                         c[pk(1, 1)] > rt.gain_max * v[5]))
             kind = 1;

@@ -67,3 +67,21 @@ extern "C" void host_slot_update(int kind, int64_t n, float *x, float *c, const 
         chi2[t] = s[kSlotChi2];
     }
 }
+
+// update_local of the same arrays, q1, q2 as given; st as it returns.
+extern "C" void host_update(int64_t n, float *x, float *c, const float *nrm, const float *m, const float *v,
+                            const float *opt, float *chi2, int32_t *st)
+{
+    const Routing rt = routing(opt);
+    for (int64_t t = 0; t < n; ++t) {
+        float cl[15], ml[3], vl[6], slot[kSlotSize];
+        Local p{x[t], x[n + t], x[2 * n + t], x[3 * n + t], x[4 * n + t], x[5 * n + t], 1.0f, 0.0f, nrm[t], nrm[n + t]};
+        for (int i = 0; i < 15; ++i) cl[i] = c[i * n + t];
+        for (int i = 0; i < 3; ++i) ml[i] = m[i * n + t];
+        for (int i = 0; i < 6; ++i) vl[i] = v[i * n + t];
+        st[t] = update_local(p, cl, ml, vl, rt, &chi2[t], slot, 1);
+        const float out[6] = {p.x, p.y, p.z, p.q1, p.q2, p.pz};
+        for (int i = 0; i < 6; ++i) x[i * n + t] = out[i];
+        for (int i = 0; i < 15; ++i) c[i * n + t] = cl[i];
+    }
+}

@@ -118,3 +118,28 @@ def test_float_float_update_tells_a_bad_s(host):
     assert np.array_equal(st3[sel], st2[sel])
     bad = st3 == 1
     assert np.array_equal(x3[:, bad], x[:, bad]) and np.array_equal(c3[:, bad], c[:, bad])
+
+
+def test_update_outside_pt_bounds_keeps_a_precise_hit(host):
+    """Predictions 2^6 to 2^26 times as wide as the hit, in t and z: the variances
+    the update leaves, C V / (C + V) of an uncorrelated pair, against 64 bits.
+    Half an ulp is EPS; the arithmetic adds 2^-45 C / V <= EPS / 2 of float-float
+    below 2^20, and 2^-53 C / V of FP64 beyond."""
+    n = 4000
+    rng = np.random.default_rng(8)
+    x, c, nrm, m, v = _updates(rng, n)
+    nrm[0], nrm[1] = 1, 0
+    c[[1, 3, 4, 6, 7, 10, 11]] = 0  # t and z uncorrelated with the rest
+    c[0], c[2] = (2.0 ** rng.uniform(-10, 8, (2, n))).astype(np.float32)
+    v[0] = v[2] = (c[0] * 2.0 ** rng.uniform(-26, -6, n)).astype(np.float32)
+    v[5] = (c[2] * 2.0 ** rng.uniform(-26, -6, n)).astype(np.float32)
+    m[:2] = x[:2]
+    chi2, st = np.empty(n, np.float32), np.empty(n, np.int32)
+    got = c.copy()
+    host.host_update(ctypes.c_int64(n), _p(x.copy()), _p(got), _p(nrm), _p(m), _p(v),
+                     _p(_opt(cond_max=1e30, pt_lo=1e3, pt_hi=2e3)), _p(chi2), _p(st))
+    assert (st == 2).all()
+    for i, j in ((0, 2), (2, 5)):
+        want = c[i].astype(np.float64) * v[j] / (c[i].astype(np.float64) + v[j])
+        rel = np.abs(got[i] / want - 1) / EPS
+        assert rel.max() <= 1.5, (i, rel.max())
