@@ -75,7 +75,8 @@ typedef struct CUstream_st *kf_stream; /* a cudaStream_t; NULL is the legacy def
 #define KF_PRECISION_ROUTED 1 /* FP32, with ill-conditioned updates redone in FP64 */
 
 /* launch_mode */
-#define KF_LAUNCH_AUTO 0      /* all events in one launch, and one for those in extended precision */
+#define KF_LAUNCH_AUTO 0      /* all events in one launch, and one for those in extended precision
+                                 (with gain_max > 0 and for few tracks in the one) */
 #define KF_LAUNCH_PER_EVENT 1 /* one plain launch per event (needs event_offsets) */
 #define KF_LAUNCH_FLAT 2      /* one plain launch over all tracks */
 
@@ -109,7 +110,8 @@ typedef struct {
     int launch_mode;         /* KF_LAUNCH_* */
     int tracks_per_block;    /* 0 = autotuned, else 32, 64, 128 or 256 */
     int reg_cap;             /* registers per thread of the fit: 0 = autotuned,
-                                -1 = uncapped, 168, 128, 96 or 80 */
+                                -1 = uncapped, 168, 128, 96 or 80 (gain_max > 0: checked, and
+                                always 128; hit_prefetch then 1) */
     int hit_prefetch;        /* how far ahead of its update the fit loads a hit:
                                 0 = autotuned, 1 = at the start of its layer, into registers,
                                 2 or 4 = that many layers, through a ring in shared memory

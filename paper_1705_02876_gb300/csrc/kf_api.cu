@@ -22,7 +22,7 @@ struct kf_context {
     int sm_count = 0;
     unsigned *d_work = nullptr;  // the fit's counters (kFitWorkBytes), 0 between fits
     std::string err;
-    // (L, log2 size, precision, fixed block, fixed cap, fixed depth) -> shape
+    // (L, log2 size, tuning mode, fixed block, fixed cap, fixed depth) -> shape
     std::map<std::tuple<int, int, int, int, int, int>, kf::FitShape> tuned;
     kf::BuildState *build = nullptr;
     kf::MlpState *mlp = nullptr;
@@ -216,6 +216,10 @@ int size_class(int64_t n)
 // as the tuner's size classes.
 constexpr int64_t kOneLaunchTracks = 32768;
 
+// Fits that are tuned apart: 0 FP32, 1 routed, 2 routed with gain_max, whose
+// updates in extended precision run in line at every size (launch_fit_tuned).
+int tuning_mode(const Routing &rt) { return rt.mode == 1 && rt.gain_max > 0.0f ? 2 : rt.mode; }
+
 cudaError_t enqueue_fit(kf_context *ctx, const FitGeom &g, const Routing &rt, const FitIO &io, const FitShape &sh,
                         cudaStream_t stream)
 {
@@ -233,7 +237,7 @@ cudaError_t enqueue_fit(kf_context *ctx, const FitGeom &g, const Routing &rt, co
 FitShape tune_shape(kf_context *ctx, const FitGeom &g, const Routing &rt, const FitIO &io, cudaStream_t stream,
                     const FitShape &fixed)
 {
-    const auto key = std::make_tuple(g.L, size_class(io.T), rt.mode, fixed.block, fixed.cap, fixed.depth);
+    const auto key = std::make_tuple(g.L, size_class(io.T), tuning_mode(rt), fixed.block, fixed.cap, fixed.depth);
     auto it = ctx->tuned.find(key);
     if (it != ctx->tuned.end()) return it->second;
     FitShape cand[64];
@@ -330,9 +334,10 @@ int kf_fit_tracks(kf_context *ctx, const kf_geometry *geom, int64_t n_tracks, co
             e = launch_fit_plain(g, rt, io, event_offsets[ev], event_offsets[ev + 1], block ? block : 128, stream);
         break;
     default: {
-        if (rt.mode == 1 && n_tracks < kOneLaunchTracks && !block && !o.reg_cap && !o.hit_prefetch) {
+        const int mode = tuning_mode(rt);
+        if (((mode == 1 && n_tracks < kOneLaunchTracks) || mode == 2) && !block && !o.reg_cap && !o.hit_prefetch) {
             e = launch_fit_plain(g, rt, io, 0, n_tracks, 64, stream);
-            ctx->tuned[std::make_tuple(g.L, size_class(n_tracks), rt.mode, 0, 0, 0)] = FitShape{64, 0, 1};
+            ctx->tuned[std::make_tuple(g.L, size_class(n_tracks), mode, 0, 0, 0)] = FitShape{64, 128, 1};
             break;
         }
         FitShape shape{block, o.reg_cap < 0 ? 0 : o.reg_cap, o.hit_prefetch};
@@ -349,7 +354,7 @@ int kf_fit_tuned_shape(kf_context *ctx, int n_layers, int64_t n_tracks, int *tra
                        int *hit_prefetch)
 {
     if (!ctx || !tracks_per_block || !reg_cap || !hit_prefetch) return KF_ERR_ARG;
-    for (int mode = 1; mode >= 0; --mode) {
+    for (int mode : {1, 0, 2}) {
         auto it = ctx->tuned.find(std::make_tuple(n_layers, size_class(n_tracks), mode, 0, 0, 0));
         if (it != ctx->tuned.end()) {
             *tracks_per_block = it->second.block;

@@ -47,7 +47,8 @@ cudaError_t launch_fit_plain(const FitGeom &g, const Routing &rt, const FitIO &i
 // registers capped at `cap` per thread (0 = no cap), hits loaded `depth` layers
 // ahead (1: registers; 2, 4: a cp.async ring in shared memory), which counts
 // the tracks that need extended precision in work[0], and with routing a
-// second one for those.  `work` (kFitWorkBytes) must read 0 at launch, and does
+// second one for those; or, with routing and gain_max > 0, the plain kernel in
+// blocks of `block` threads.  `work` (kFitWorkBytes) must read 0 at launch, and does
 // again when the fit has run.
 cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &io, int block, int cap, int depth,
                              int sm_count, unsigned *work, cudaStream_t stream);

@@ -812,9 +812,9 @@ __device__ __forceinline__ int update_local(Local &p, float c[15], const float m
             const float vdz = fmaf(-__fdividef(ve, vdt), ve, fmaf(-vnz, vz, v[5]));
             kind = c[pk(0, 0)] < kWideGain * vdt && c[pk(1, 1)] < kWideGain * vdz ? 3 : 2;
         }
-        else if (rt.gain_max > 0.0f && (tt * c[pk(0, 0)] > rt.gain_max * v[0] || nn * c[pk(0, 0)] > rt.gain_max * v[2] ||
-                                        c[pk(1, 1)] > rt.gain_max * v[5]))
-            kind = 1;
+        else if (rt.gain_max > 0.0f)  // one test (|): the lanes it holds for reach the call together
+            kind = (tt * c[pk(0, 0)] > rt.gain_max * v[0]) | (nn * c[pk(0, 0)] > rt.gain_max * v[2]) |
+                   (c[pk(1, 1)] > rt.gain_max * v[5]);
     } else if (!pd) {
         return 1;
     }

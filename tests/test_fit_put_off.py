@@ -37,3 +37,21 @@ def test_put_off_equals_in_line(kf, n):
                 for k in want:
                     assert np.array_equal(got[k].cpu().numpy(), want[k].cpu().numpy(), equal_nan=True), (lo, k)
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [300, 40_001])
+@pytest.mark.parametrize("gain_max", [1.0, 100.0])
+def test_float_float_gains_run_in_line(kf, n, gain_max):
+    """With gain_max the plain kernel runs whatever the size and the shape: equal
+    to KF_LAUNCH_FLAT bit for bit, and the shape reported is that kernel's."""
+    ctx = kf.Context(0)
+    b = synth.make_fit_batch(62, [n], pt_lo=0.24, pt_hi=500.0, pt_dist="loguniform", hit_eff=0.9)
+    dev, geom = kf.to_device(b), kf.GeometryArgs.of(b.geom)
+    want = kf.fit_tracks(ctx, geom, **dev, opt=kf.options(launch_mode=kf.LAUNCH_FLAT, gain_max=gain_max))
+    assert float(((want["flags"] & 16) != 0).float().mean()) > 0.5
+    for shape in ({}, dict(tracks_per_block=32, reg_cap=96, hit_prefetch=4)):
+        got = kf.fit_tracks(ctx, geom, **dev, opt=kf.options(gain_max=gain_max, **shape))
+        for k in want:
+            assert np.array_equal(got[k].cpu().numpy(), want[k].cpu().numpy(), equal_nan=True), (shape, k)
+        assert ctx.tuned_shape(b.geom.n_layers, n) == (64, 128, 1)
+    ctx.close()
