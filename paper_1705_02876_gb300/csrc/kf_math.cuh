@@ -355,9 +355,10 @@ static __device__ __noinline__ int update_ff(float *slot_p, int stride)
 // The whole update in float-float: update_fp64 to some 2^-45 of its terms
 // instead of 2^-52.  What a hit leaves of a variance C is about V: a result is
 // off by 2^-45 C / V of itself, so that with C below kWideGain V (and S well
-// conditioned, both the caller's tests) the FP32 results are those of the FP64
-// update but for rounding ties.  Some 1,100 FP32 instructions, about a tenth
-// of the time of the FP64 pipe's 280.  Returns as update_fp64 does.
+// conditioned, the caller's test) the FP32 results are those of the FP64 update
+// but for rounding ties.  Some 1,100 FP32 instructions, about a tenth of the
+// time of the FP64 pipe's 280.  Returns as update_fp64 does, or 0 with nothing
+// written where C is larger.
 constexpr float kWideGain = 1048576.0f;  // 2^20: 2^-25, half an FP32 half-ulp
 __device__ __forceinline__ ff ff_sub(ff x, ff y) { return ff_add(x, ff_neg(y)); }
 __device__ __forceinline__ ff ff_addf(ff x, float y)
@@ -401,13 +402,18 @@ static __device__ __noinline__ int update_wide(float *slot_p, int stride)
         ia = ff_rcp(vnn);
         vt = ff_mul(vnt, ia);
         vz = ff_mul(vnz, ia);
-        const ff dt = ff_sub(ff_addf(vtt, sl.c(0, 0)), ff_mul(vnt, vt));
+        // V given n, and what C adds
+        const ff ut = ff_sub(vtt, ff_mul(vnt, vt)), uz = ff_sub(vtz, ff_mul(vnt, vz));
+        const ff dt = ff_addf(ut, sl.c(0, 0));
         it = ff_rcp(dt);
-        const ff e = ff_sub(ff_addf(vtz, sl.c(1, 0)), ff_mul(vnt, vz));
+        const ff e = ff_addf(uz, sl.c(1, 0));
         l = ff_mul(e, it);
         const ff dz = ff_sub(ff_sub(two_sum(sl.c(1, 1), sl.v(5)), ff_mul(vnz, vz)), ff_mul(l, e));
         iz = ff_rcp(dz);
         if (!(vnn.hi > 0.0f && dt.hi > 0.0f && dz.hi > 0.0f && dz.hi < INFINITY)) return 1;
+        // V's z pivot, given n and t
+        const float uzz = fmaf(-__fdividef(uz.hi, ut.hi), uz.hi, fmaf(-vnz.hi, vz.hi, sl.v(5)));
+        if (!(sl.c(0, 0) < kWideGain * ut.hi && sl.c(1, 1) < kWideGain * uzz)) return 0;
     }
     const float X0 = sl.x(0), X1 = sl.x(1), X2 = sl.x(2);
     ff w1, w2;
@@ -463,7 +469,12 @@ static __device__ __noinline__ int update_wide(float *slot_p, int stride)
 
 static __device__ __noinline__ int update_ext(float *slot, int stride, int kind)
 {
-    return kind == 2 ? update_fp64(slot, stride) : kind == 3 ? update_wide(slot, stride) : update_ff(slot, stride);
+    if (kind == 3) {
+        const int st = update_wide(slot, stride);
+        if (st) return st;
+        kind = 2;
+    }
+    return kind == 2 ? update_fp64(slot, stride) : update_ff(slot, stride);
 }
 
 // ---------------------------------------------------------------------------
@@ -806,12 +817,8 @@ __device__ __forceinline__ int update_local(Local &p, float c[15], const float m
         const float pt2 = fmaf(p.q1, p.q1, p.q2 * p.q2);
         if (ill)
             kind = 2;
-        else if (outside_pt(pt2, rt)) {
-            // V's t and z pivots: its variances given n, and given n and t
-            const float vdt = fmaf(-vnt, vt, vtt), ve = fmaf(-vnt, vz, vtz);
-            const float vdz = fmaf(-__fdividef(ve, vdt), ve, fmaf(-vnz, vz, v[5]));
-            kind = c[pk(0, 0)] < kWideGain * vdt && c[pk(1, 1)] < kWideGain * vdz ? 3 : 2;
-        }
+        else if (outside_pt(pt2, rt))
+            kind = 3;
         else if (rt.gain_max > 0.0f)  // one test (|): the lanes it holds for reach the call together
             kind = (tt * c[pk(0, 0)] > rt.gain_max * v[0]) | (nn * c[pk(0, 0)] > rt.gain_max * v[2]) |
                    (c[pk(1, 1)] > rt.gain_max * v[5]);
