@@ -47,11 +47,13 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
     const float *hc = io.hit_cov + base;
     const uint32_t mask = __ldcs(io.hit_mask + base + off);
     float m[3] = {0, 0, 0}, v[6] = {0, 0, 0, 0, 0, 0};
-    auto load_hit = [&](float mm[3], float vv[6]) {
+    auto load_hit = [&](bool has) {
+        if (has) {
 #pragma unroll
-        for (int i = 0; i < 3; ++i) mm[i] = __ldcs(hp + i * T + off);
+            for (int i = 0; i < 3; ++i) m[i] = __ldcs(hp + i * T + off);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) vv[i] = __ldcs(hc + i * T + off);
+            for (int i = 0; i < 6; ++i) v[i] = __ldcs(hc + i * T + off);
+        }
         hp += 3 * T;
         hc += 6 * T;
     };
@@ -79,7 +81,7 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
     for (int i = 0; i < 21; ++i) sc[i] = __ldcs(seed_cov + i * T + off);
     const float qkb = (float)(io.charge + base)[off] * g.qk;
     if constexpr (DEPTH == 1) {
-        load_hit(m, v);  // whether or not it is there, without waiting for the mask
+        load_hit(mask & 1u);  // the seed's loads are in flight
     } else {
 #pragma unroll
         for (int k = 0; k < DEPTH; ++k) issue();
@@ -100,7 +102,7 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
         for (int l = 0; l < g.L; ++l) {
             const bool has = (mask >> l) & 1u;
             if constexpr (DEPTH == 1) {
-                if (l > 0) load_hit(m, v);
+                if (l > 0) load_hit(has);
             } else {
                 issue();                 // layer l + DEPTH
                 cp_async_wait<DEPTH>();  // layer l's group has landed
@@ -170,6 +172,11 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
     (io.out_flags + base)[off] = flags;
     return false;
 }
+
+}  // namespace
+
+#ifdef __CUDACC__  // tests compile the above for the host
+namespace {
 
 // One thread per track over [t_begin, t_end), the updates in extended precision
 // in line.  Two blocks of 256 threads per SM: at 128 registers (162 uncapped)
@@ -365,4 +372,6 @@ cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &i
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, fit_extended_kernel, g, rt, io, work);
 }
+#endif  // __CUDACC__
+
 }  // namespace kf

@@ -1,20 +1,6 @@
 // The per-track arithmetic of csrc/kf_math.cuh compiled for the host, for tests
-// of single steps without a GPU: CUDA's qualifiers are empty and its device
-// functions are the C library's (the approximate ones within their error).
-#include <math.h>
-#include <stdint.h>
-
-#define __device__
-#define __host__
-#define __forceinline__ inline
-#define __noinline__
-static inline float __fdividef(float a, float b) { return a / b; }
-static inline float rsqrtf(float a) { return (float)(1.0 / sqrt((double)a)); }
-#define __logf logf
-static inline float __fadd_rn(float a, float b) { return a + b; }
-static inline float __fsub_rn(float a, float b) { return a - b; }
-static inline float __fmul_rn(float a, float b) { return a * b; }
-static inline float __fmaf_rn(float a, float b, float c) { return fmaf(a, b, c); }
+// of single steps without a GPU.
+#include "cuda_shim.h"
 
 #include "kf_math.cuh"
 

@@ -1,5 +1,5 @@
-"""Single steps of the library's per-track arithmetic (csrc/kf_math.cuh),
-compiled for the host, against the FP64 oracle."""
+"""The library's per-track arithmetic (csrc/kf_math.cuh, fit_track of
+csrc/kf_fit.cu) compiled for the host, against 64 bits."""
 import ctypes
 import os
 import shutil
@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 
 from paper_1705_02876_gb300 import synth
+from paper_1705_02876_gb300.build import nvcc
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -16,13 +17,18 @@ EPS = 2.0 ** -24  # half an ulp of FP32, relative
 pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="no g++")
 
 
-@pytest.fixture(scope="module")
-def host(tmp_path_factory):
-    so = str(tmp_path_factory.mktemp("host") / "track_math.so")
+def _compile(name, tmp):
+    so = str(tmp.mktemp("host") / (name + ".so"))
     subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-ffp-contract=off", "-w",
                     "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_1705_02876_gb300", "csrc"),
-                    "-o", so, os.path.join(HERE, "host", "track_math.cpp")], check=True)
+                    "-I", os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include"),
+                    "-o", so, os.path.join(HERE, "host", name + ".cpp")], check=True)
     return ctypes.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    return _compile("track_math", tmp_path_factory)
 
 
 def _p(a):
@@ -143,3 +149,30 @@ def test_update_outside_pt_bounds_keeps_a_precise_hit(host):
         want = c[i].astype(np.float64) * v[j] / (c[i].astype(np.float64) + v[j])
         rel = np.abs(got[i] / want - 1) / EPS
         assert rel.max() <= 1.5, (i, rel.max())
+
+
+def test_fit_reads_no_absent_hit(tmp_path_factory, oracle):
+    """The hits a fit reads are those of the mask, up to the layer where it stops;
+    what the fit gives is the oracle's."""
+    lib = _compile("fit_track", tmp_path_factory)
+    n = 500
+    b = synth.make_fit_batch(9, [n], geom=synth.toy_geometry(17), hit_eff=0.6, eta_max=2.0)
+    g, L = b.geom, 17
+    pad = np.zeros(3 * n * (32 - L), np.float32)  # hit_cov begins 32 layers after hit_pos
+    block = np.concatenate([np.ravel(b.hit_pos).astype(np.float32), pad, np.ravel(b.hit_cov).astype(np.float32),
+                            np.zeros(6 * n * (32 - L), np.float32)])
+    f32 = lambda a: np.ascontiguousarray(a, dtype=np.float32)
+    r, xx0 = f32(g.radii), f32(g.x_over_x0)
+    mask = np.ascontiguousarray(b.hit_mask, dtype=np.uint32)
+    out = [np.empty((6, n), np.float32), np.empty((21, n), np.float32), np.empty(n, np.float32), np.empty(n, np.int16),
+           np.empty(n, np.uint32)]
+    read = np.empty(n, np.uint32)
+    lib.host_fit(L, _p(r), _p(xx0), ctypes.c_float(g.z_half), ctypes.c_float(0.00299792458 * g.bz), ctypes.c_int64(n),
+                 _p(f32(b.seed_state)), _p(f32(b.seed_cov)), _p(b.charge), _p(block),
+                 ctypes.c_void_p(block.ctypes.data + 4 * 3 * n * 32), _p(mask), *[_p(a) for a in out], _p(read))
+    ref = oracle.fit_batch(b)
+    stopped = (out[4] & 3) != 0
+    assert np.array_equal(out[3], ref["ndof"]) and stopped.any()
+    assert ((read & ~mask) == 0).all()
+    assert (read[~stopped] == mask[~stopped]).all() and (mask != (1 << L) - 1).any()
+    assert np.linalg.norm(out[0] - ref["state"]) < 1e-4 * np.linalg.norm(ref["state"])
