@@ -83,6 +83,17 @@ int check_geometry(kf_context *ctx, const kf_geometry *geom, FitGeom *g)
     return KF_OK;
 }
 
+cudaError_t zero_now(void *p, size_t bytes)
+{
+    cudaStream_t s;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p, 0, bytes, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+    return e == cudaSuccess ? e2 : e;
+}
+
 int check_ptr(kf_context *ctx, const void *p, size_t align, const char *name)
 {
     if (!p) return set_error(ctx, KF_ERR_ARG, "%s is NULL", name);
@@ -170,7 +181,7 @@ int kf_context_create(kf_context **out, int device)
         delete ctx;
         return KF_ERR_NOMEM;
     }
-    if (cudaMemset(ctx->d_work, 0, kFitWorkBytes) != cudaSuccess) {
+    if (zero_now(ctx->d_work, kFitWorkBytes) != cudaSuccess) {
         cudaFree(ctx->d_work);
         delete ctx;
         return KF_ERR_CUDA;

@@ -27,6 +27,10 @@ int set_error(kf_context *ctx, int code, const char *fmt, ...);
 int cuda_error(kf_context *ctx, cudaError_t e, const char *what);
 int check_geometry(kf_context *ctx, const kf_geometry *geom, FitGeom *g);
 int check_ptr(kf_context *ctx, const void *p, size_t align, const char *name);
+// Clear new device memory that work on any stream may read at once: done when it
+// returns.  (cudaMemset returns before it is done, on the legacy stream, which
+// streams made with cudaStreamNonBlocking do not wait for.)
+cudaError_t zero_now(void *p, size_t bytes);
 int check_options(kf_context *ctx, const kf_options &o);
 Routing make_routing(const kf_options &o);
 int context_device(const kf_context *ctx);

@@ -114,7 +114,7 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
     if (!hp) {
         hp = new HostPipe;
         bool ok = cudaMalloc(&hp->work, kHostStreams * kFitWorkBytes) == cudaSuccess &&
-                  cudaMemset(hp->work, 0, kHostStreams * kFitWorkBytes) == cudaSuccess;
+                  zero_now(hp->work, kHostStreams * kFitWorkBytes) == cudaSuccess;
         for (int i = 0; ok && i < kHostStreams; ++i)
             ok = cudaStreamCreateWithFlags(&hp->stream[i], cudaStreamNonBlocking) == cudaSuccess;
         if (!ok) {

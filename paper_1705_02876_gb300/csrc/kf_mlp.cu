@@ -733,7 +733,7 @@ int ensure_state(kf_context *ctx, MlpState **out)
                   cudaMalloc(&s->W1, kW1Elems * sizeof(__nv_bfloat16)) == cudaSuccess &&
                   cudaMalloc(&s->W2, kW2Elems * sizeof(__nv_bfloat16)) == cudaSuccess &&
                   cudaMalloc(&s->status, sizeof(unsigned)) == cudaSuccess &&
-                  cudaMemset(s->status, 0, sizeof(unsigned)) == cudaSuccess;
+                  zero_now(s->status, sizeof(unsigned)) == cudaSuccess;
         if (!ok) {
             destroy_mlp_state(s);
             s = nullptr;

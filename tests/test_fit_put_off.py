@@ -55,3 +55,31 @@ def test_float_float_gains_run_in_line(kf, n, gain_max):
             assert np.array_equal(got[k].cpu().numpy(), want[k].cpu().numpy(), equal_nan=True), (shape, k)
         assert ctx.tuned_shape(b.geom.n_layers, n) == (64, 128, 1)
     ctx.close()
+
+
+def test_new_context_behind_a_busy_default_stream(kf):
+    """A context made while the default stream is busy, used at once on a stream
+    that does not wait for it: what the context clears when it is made is cleared
+    by then, so that no track put off is lost."""
+    b = synth.make_fit_batch(63, [40_001], pt_lo=50.0, pt_hi=500.0, pt_dist="loguniform")
+    dev, geom = kf.to_device(b), kf.GeometryArgs.of(b.geom)
+    pinned = {k: v.cpu().pin_memory() for k, v in dev.items()}
+    shape = dict(tracks_per_block=64, reg_cap=96, hit_prefetch=1)
+    first = kf.Context(0)
+    want = kf.fit_tracks(first, geom, **dev, opt=kf.options(launch_mode=kf.LAUNCH_FLAT))
+    outs = [kf.fit_outputs(40_001, "cuda") for _ in range(100)]
+    a = torch.randn(8192, 8192, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(20):
+        a = (a @ a).clamp_(-1, 1)  # tens of ms on the default stream
+    ctx = kf.Context(0)
+    for out in outs:
+        kf.fit_tracks(ctx, geom, **dev, out=out, opt=kf.options(**shape), stream=side)
+    host = kf.fit_tracks_host(ctx, geom, **pinned)
+    torch.cuda.synchronize()
+    for out in outs + [host]:
+        for k in want:
+            assert np.array_equal(out[k].cpu().numpy(), want[k].cpu().numpy(), equal_nan=True), k
+    ctx.close()
+    first.close()
