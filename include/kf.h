@@ -532,19 +532,18 @@ int kf_fit_tuned_shape(kf_context *ctx, int n_layers, int64_t n_tracks, int *tra
  * allocation while their own work is in flight can call this instead.  It
  * runs the same fit kernels (same steps, inputs, outputs and flags
  * as kf_fit_tracks, all events in one launch and those in extended precision in
- * another) and allocates nothing: the kernels' only scratch, two 4-byte
- * counters, is a fixed array in the library's device memory that every GPU
- * loading the library holds until the process exits.
+ * another) and allocates nothing: the kernels' only scratch, 4 bytes, is in the
+ * library's device memory, which every GPU loading the library holds until the
+ * process exits.
  *
  *   - Runs on the current CUDA device.  The first call on a device looks up
- *     that array's device address once (cudaGetSymbolAddress); make that
+ *     the scratch's device address once (cudaGetSymbolAddress); make that
  *     first call before any stream capture.
- *   - The counters read 0 between calls: the second launch clears them.  All
- *     calls on a device share them, so calls whose work overlaps on the GPU
- *     (different streams, not ordered) race and give wrong results: order
- *     them on one stream or synchronise.
+ *   - All calls on a device share the scratch, so calls whose work overlaps on
+ *     the GPU (different streams, not ordered) race and give wrong results:
+ *     order them on one stream or synchronise.  A later call is not affected.
  *   - n_tracks must be at most KF_NOALLOC_MAX_TRACKS (2^36, the limit of
- *kf_fit_tracks too); larger batches return KF_ERR_TOO_LARGE.
+ *     kf_fit_tracks too); larger batches return KF_ERR_TOO_LARGE.
  *   - No tuning runs.  The shape is opt->tracks_per_block, opt->reg_cap and
  *     opt->hit_prefetch where set, else 64 tracks per block, no register cap
  *     and the register prefetch (depth 1).  Only the (block, cap, depth)

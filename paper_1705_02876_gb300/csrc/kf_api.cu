@@ -20,7 +20,8 @@ using namespace kf;
 struct kf_context {
     int device = 0;
     int sm_count = 0;
-    unsigned *d_work = nullptr;  // the fit's counters (kFitWorkBytes), 0 between fits
+    unsigned *d_work = nullptr;  // the tag of the last fit that put a track off
+    unsigned fit_tag = 0;        // the last fit's
     std::string err;
     // (L, log2 size, tuning mode, fixed block, fixed cap, fixed depth) -> shape
     std::map<std::tuple<int, int, int, int, int, int>, kf::FitShape> tuned;
@@ -177,11 +178,11 @@ int kf_context_create(kf_context **out, int device)
     kf_context *ctx = new kf_context;
     ctx->device = device;
     ctx->sm_count = prop.multiProcessorCount;
-    if (cudaMalloc(&ctx->d_work, kFitWorkBytes) != cudaSuccess) {
+    if (cudaMalloc(&ctx->d_work, sizeof(unsigned)) != cudaSuccess) {
         delete ctx;
         return KF_ERR_NOMEM;
     }
-    if (zero_now(ctx->d_work, kFitWorkBytes) != cudaSuccess) {
+    if (zero_now(ctx->d_work, sizeof(unsigned)) != cudaSuccess) {
         cudaFree(ctx->d_work);
         delete ctx;
         return KF_ERR_CUDA;
@@ -236,7 +237,8 @@ cudaError_t enqueue_fit(kf_context *ctx, const FitGeom &g, const Routing &rt, co
 {
     const int ok = fit_shape_usable(sh.block, sh.cap, sh.depth);
     if (ok <= 0) return cudaErrorInvalidConfiguration;
-    return launch_fit_tuned(g, rt, io, sh.block, sh.cap, sh.depth, ctx->sm_count, ctx->d_work, stream);
+    return launch_fit_tuned(g, rt, io, sh.block, sh.cap, sh.depth, ctx->sm_count, ctx->d_work, ++ctx->fit_tag,
+                            stream);
 }
 
 // Time every compiled (tracks per block, register cap, hit prefetch depth)

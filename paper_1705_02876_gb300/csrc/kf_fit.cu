@@ -197,16 +197,17 @@ __global__ void __launch_bounds__(256, 2) fit_plain_kernel(const FitGeom g, cons
 // An update in extended precision (float-float: some 1,100 instructions; FP64:
 // a pipe 64 times narrower than the FP32 one) takes as long for one lane of a
 // warp as for 32, so a track that needs one is put off: its flags are set to
-// kPutOff and it is counted in work[0], and fit_extended_kernel, launched
-// behind, fits these tracks from their seeds in full warps (none: it returns
-// at once).  With one track in eight above pt_hi (1,000,000 tracks, pT
+// kPutOff and *work to the fit's tag, and fit_extended_kernel, launched behind,
+// fits these tracks from their seeds in full warps (no tag: it returns at
+// once; the tag of a fit replayed from a graph may stand from an earlier
+// replay, and the kernel then finds no marked track).  With one track in eight above pt_hi (1,000,000 tracks, pT
 // log-uniform 0.24 to 500 GeV) nearly every warp held one and stopped for it
 // at every layer: 7.09 ms in line in FP64, 1.03 ms put off in FP64, 0.31 ms
 // in float-float.  Without that code this kernel also needs fewer registers
 // (96 with the ring, no spills).
 template <int BLOCK, int MINB, int DEPTH>
 __global__ void __launch_bounds__(BLOCK, MINB) fit_kernel(const FitGeom g, const Routing rt, const FitIO io,
-                                                           unsigned *work)
+                                                           unsigned *work, unsigned tag)
 {
     extern __shared__ float ring[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -215,8 +216,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) fit_kernel(const FitGeom g, const
     bool put_off = false;
     if (base + off < io.T) put_off = fit_track<DEPTH, true>(g, rt, io, base, off, nullptr, BLOCK, ring + off);
     if (put_off) (io.out_flags + base)[off] = kPutOff;
-    const unsigned n = __popc(__ballot_sync(0xffffffffu, put_off));
-    if (n && (off & 31u) == 0) atomicAdd(work, n);
+    if (__any_sync(0xffffffffu, put_off) && (off & 31u) == 0) *work = tag;
 }
 
 // The tracks put off by the launch before: a block gathers them from the flags
@@ -226,13 +226,13 @@ __global__ void __launch_bounds__(BLOCK, MINB) fit_kernel(const FitGeom g, const
 // 330 and 342 with 64 and 32 threads).
 constexpr int kExtBlock = 256;
 __global__ void __launch_bounds__(kExtBlock, 2) fit_extended_kernel(const FitGeom g, const Routing rt, const FitIO io,
-                                                                     unsigned *work)
+                                                                     const unsigned *work, unsigned tag)
 {
     __shared__ float slots[kSlotSize * kExtBlock];
     __shared__ int64_t queue[2 * kExtBlock];
     __shared__ int queued;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (__ldcg(work) == 0) return;
+    if (__ldcg(work) != tag) return;
     if (threadIdx.x == 0) queued = 0;
     __syncthreads();
     const int64_t chunks = (io.T + kExtBlock - 1) / kExtBlock;
@@ -252,11 +252,9 @@ __global__ void __launch_bounds__(kExtBlock, 2) fit_extended_kernel(const FitGeo
         if (threadIdx.x == 0) queued = n;
         __syncthreads();
     }
-    // the last block to end clears the count: every block has read it
-    if (threadIdx.x == 0 && atomicInc(work + 1, gridDim.x - 1) == gridDim.x - 1) work[0] = 0u;
 }
 
-using FitFn = void (*)(FitGeom, Routing, FitIO, unsigned *);
+using FitFn = void (*)(FitGeom, Routing, FitIO, unsigned *, unsigned);
 
 // Dynamic shared memory of a shape: DEPTH + 1 stages of 9 floats per thread.
 constexpr size_t ring_bytes(int block, int depth) { return depth > 1 ? (size_t)(depth + 1) * 9 * block * 4 : 0; }
@@ -346,7 +344,7 @@ int fit_shapes(int *blocks, int *caps, int *depths, int max_n)
 }
 
 cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &io, int block, int cap, int depth,
-                                  int sm_count, unsigned *work, cudaStream_t stream)
+                                  int sm_count, unsigned *work, unsigned tag, cudaStream_t stream)
 {
     const Shape *sh = find_shape(block, cap, depth);
     if (!sh) return cudaErrorInvalidValue;
@@ -359,7 +357,7 @@ cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &i
     if (rt.mode == 1 && rt.gain_max > 0.0f) return launch_fit_plain(g, rt, io, 0, io.T, block, stream);
     const int64_t grid = (io.T + block - 1) / block;
     if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
-    sh->fn<<<(unsigned)grid, block, ring_bytes(block, depth), stream>>>(g, rt, io, work);
+    sh->fn<<<(unsigned)grid, block, ring_bytes(block, depth), stream>>>(g, rt, io, work, tag);
     if ((e = cudaGetLastError()) != cudaSuccess || rt.mode == 0) return e;  // without routing no track is put off
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)std::min<int64_t>((io.T + kExtBlock - 1) / kExtBlock, (int64_t)sm_count * 2));
@@ -370,7 +368,7 @@ cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &i
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fit_extended_kernel, g, rt, io, work);
+    return cudaLaunchKernelEx(&cfg, fit_extended_kernel, g, rt, io, (const unsigned *)work, tag);
 }
 #endif  // __CUDACC__
 

@@ -45,14 +45,14 @@ cudaError_t launch_fit_plain(const FitGeom &g, const Routing &rt, const FitIO &i
                              int64_t t_end, int block, cudaStream_t stream);
 // The fit of the whole batch: a kernel of blocks of `block` threads with
 // registers capped at `cap` per thread (0 = no cap), hits loaded `depth` layers
-// ahead (1: registers; 2, 4: a cp.async ring in shared memory), which counts
-// the tracks that need extended precision in work[0], and with routing a
-// second one for those; or, with routing and gain_max > 0, the plain kernel in
-// blocks of `block` threads.  `work` (kFitWorkBytes) must read 0 at launch, and does
-// again when the fit has run.
+// ahead (1: registers; 2, 4: a cp.async ring in shared memory), which writes
+// `tag` to *work when a track needs extended precision, and with routing a
+// second one for those tracks; or, with routing and gain_max > 0, the plain
+// kernel in blocks of `block` threads.  *work is the launch's own until it has
+// run; what it holds before does not matter, as long as each launch on it has
+// another tag than the one before.
 cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &io, int block, int cap, int depth,
-                             int sm_count, unsigned *work, cudaStream_t stream);
-constexpr size_t kFitWorkBytes = 2 * sizeof(unsigned);
+                             int sm_count, unsigned *work, unsigned tag, cudaStream_t stream);
 // 1 if this shape can be launched on the current device, 0 if it is not
 // compiled in, -1 if its shared-memory opt-in failed.
 int fit_shape_usable(int block, int cap, int depth);

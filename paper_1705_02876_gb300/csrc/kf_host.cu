@@ -19,7 +19,8 @@ constexpr int kHostStreams = 3;
 
 struct HostPipe {
     cudaStream_t stream[kHostStreams] = {};
-    char *work = nullptr;  // the work counters of one launch per stream
+    unsigned *work = nullptr;  // per stream, the tag of the last launch that put a track off
+    unsigned tag = 0;          // the last launch's
     char *buf[kHostStreams] = {};  // staging for one chunk per stream
     size_t buf_bytes = 0;
 };
@@ -113,8 +114,8 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
     HostPipe *&hp = context_host_state(ctx);
     if (!hp) {
         hp = new HostPipe;
-        bool ok = cudaMalloc(&hp->work, kHostStreams * kFitWorkBytes) == cudaSuccess &&
-                  zero_now(hp->work, kHostStreams * kFitWorkBytes) == cudaSuccess;
+        bool ok = cudaMalloc(&hp->work, kHostStreams * sizeof(unsigned)) == cudaSuccess &&
+                  zero_now(hp->work, kHostStreams * sizeof(unsigned)) == cudaSuccess;
         for (int i = 0; ok && i < kHostStreams; ++i)
             ok = cudaStreamCreateWithFlags(&hp->stream[i], cudaStreamNonBlocking) == cudaSuccess;
         if (!ok) {
@@ -165,8 +166,8 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
                 block = n_tracks < 20000 ? 64 : 256;
                 depth = 4;
             }
-            const cudaError_t e = launch_fit_tuned(g, rt, io, block, cap, depth, context_sm_count(ctx),
-                                                   reinterpret_cast<unsigned *>(hp->work), s);
+            const cudaError_t e =
+                launch_fit_tuned(g, rt, io, block, cap, depth, context_sm_count(ctx), hp->work, ++hp->tag, s);
             const cudaError_t e2 = cudaStreamSynchronize(s);
             if (e != cudaSuccess) return cuda_error(ctx, e, "host-buffer fit");
             if (e2 != cudaSuccess) return cuda_error(ctx, e2, "host-buffer fit");
@@ -225,8 +226,7 @@ extern "C" int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int6
                      reinterpret_cast<float *>(b + lay.out_chi2),
                      reinterpret_cast<int16_t *>(b + lay.out_ndof),
                      reinterpret_cast<uint32_t *>(b + lay.out_flags)};
-            e = launch_fit_tuned(g, rt, io, block, cap, depth, context_sm_count(ctx),
-                                 reinterpret_cast<unsigned *>(hp->work + k * kFitWorkBytes), s);
+            e = launch_fit_tuned(g, rt, io, block, cap, depth, context_sm_count(ctx), hp->work + k, ++hp->tag, s);
         }
         out(out_state, lay.out_state, 4, 6);
         out(out_cov, lay.out_cov, 4, 21);

@@ -7,27 +7,29 @@
 // real-time or embedded loops that must not touch the allocator after
 // start-up, and hosts that forbid allocation while their own work is in
 // flight.  This entry point runs the same fit kernels, but the only scratch
-// that they need -- two 32-bit counters of the tracks put off for FP64 -- lives
-// in a fixed array of this file's device memory.
+// that they need -- a word that says whether a track was put off for extended
+// precision -- lives in this file's device memory.
 // Nothing here calls cudaMalloc, cudaFree or any routine that allocates.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "kf.h"
 #include "kf_api_internal.h"
 
-// The scratch: two 32-bit counters, 8 bytes.  Every GPU that loads the library
-// holds this array until the process exits.  All calls on a device share it;
-// it reads 0 between calls (the second launch of a fit clears it).
-static __device__ __align__(256) unsigned g_noalloc_scratch[kf::kFitWorkBytes / sizeof(unsigned)];
+// The scratch: the tag of the last call that put a track off, 4 bytes.  Every
+// GPU that loads the library holds it until the process exits.  All calls on a
+// device share it.
+static __device__ __align__(256) unsigned g_noalloc_scratch[1];
 
 namespace {
 
 constexpr int kMaxDevices = 64;
 unsigned *g_scratch_address[kMaxDevices];  // device address of g_noalloc_scratch, per device
 std::mutex g_setup_mutex;
+std::atomic<unsigned> g_tag{0};  // the last call's
 
 // Once per device, with that device current: look up the array's device
 // address.  In host code the symbol is only a host-side stand-in; a kernel
@@ -88,7 +90,7 @@ extern "C" int kf_fit_tracks_noalloc(const kf_geometry *geom, int64_t n_tracks, 
     const FitIO io{n_tracks, seed_state, seed_cov, charge, hit_pos, hit_cov, hit_mask,
                    out_state, out_cov, out_chi2, out_ndof, out_flags};
     cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
-    if (launch_fit_tuned(g, make_routing(o), io, block, cap, depth, sms, work, stream) != cudaSuccess)
+    if (launch_fit_tuned(g, make_routing(o), io, block, cap, depth, sms, work, ++g_tag, stream) != cudaSuccess)
         return KF_ERR_CUDA;
     return KF_OK;
 }

@@ -2,8 +2,7 @@
 the same tracks with the FP64 update in line (KF_LAUNCH_FLAT): the same
 arithmetic in another launch, so every output is equal bit for bit.  Sizes on
 both sides of the one-launch limit (32,768 tracks), of the gathering blocks (256
-tracks) and with every, some, and no track put off; each batch runs twice, and
-the batch after it finds the counters cleared."""
+tracks) and with every, some, and no track put off; each batch runs twice."""
 import numpy as np
 import pytest
 
@@ -83,3 +82,32 @@ def test_new_context_behind_a_busy_default_stream(kf):
             assert np.array_equal(out[k].cpu().numpy(), want[k].cpu().numpy(), equal_nan=True), k
     ctx.close()
     first.close()
+
+
+def test_replayed_fit_finds_its_own_tracks(kf):
+    """A fit captured in a graph and replayed on batches with and without tracks to
+    put off, other fits of the context in between: each replay's outputs are
+    those of its own batch."""
+    n, ctx, side = 40_001, kf.Context(0), torch.cuda.Stream()
+    opt, flat = kf.options(tracks_per_block=64, reg_cap=96, hit_prefetch=1), kf.options(launch_mode=kf.LAUNCH_FLAT)
+    batches = [synth.make_fit_batch(64, [n], pt_lo=50.0, pt_hi=500.0, pt_dist="loguniform"),
+               synth.make_fit_batch(65, [n], pt_lo=1.0, pt_hi=5.0)]
+    geom, dev = kf.GeometryArgs.of(batches[0].geom), [kf.to_device(b) for b in batches]
+    want = [kf.fit_tracks(ctx, geom, **d, opt=flat) for d in dev]
+    shares = [float(((w["flags"] & 16) != 0).float().mean()) for w in want]
+    assert shares[0] > 0.05 and shares[1] == 0.0, shares
+    buf, out, other = {k: v.clone() for k, v in dev[0].items()}, kf.fit_outputs(n, "cuda"), kf.fit_outputs(n, "cuda")
+    kf.fit_tracks(ctx, geom, **buf, out=out, opt=opt)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        kf.fit_tracks(ctx, geom, **buf, out=out, opt=opt, stream=side)
+    for i in (0, 1, 0, 0, 1, 1, 0):
+        for k in buf:
+            buf[k].copy_(dev[i][k])
+        graph.replay()
+        for k in out:
+            assert np.array_equal(out[k].cpu().numpy(), want[i][k].cpu().numpy(), equal_nan=True), (i, k)
+        kf.fit_tracks(ctx, geom, **dev[i ^ 1], out=other, opt=opt)
+        assert all(np.array_equal(other[k].cpu().numpy(), want[i ^ 1][k].cpu().numpy(), equal_nan=True) for k in other)
+    ctx.close()

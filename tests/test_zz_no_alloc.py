@@ -3,10 +3,9 @@ memory, against the FP64 oracle and against kf_fit_tracks on the same inputs.
 
 Such callers (code inside a device-memory pool it does not own, loops that must
 not allocate after start-up) cannot create a kf_context, whose creation calls
-cudaMalloc.  The entry point keeps its only scratch, the persistent kernel's
-work counter, in a fixed array of the library's device memory and clears it
-on every call; two calls in a row check that the second call starts from a
-cleared counter.  Two launch shapes: the default (64 tracks per block, no
+cudaMalloc.  The entry point keeps its only scratch, the word by which the
+batch kernel tells the one for the tracks put off that there are some, in the
+library's device memory; each case is called twice in a row.  Two launch shapes: the default (64 tracks per block, no
 register cap, hits prefetched into registers) and a shared-memory ring shape
 (128 tracks per block, 128 registers, hits four layers ahead through
 cp.async).  This file is collected last so that a run stopping at the first
