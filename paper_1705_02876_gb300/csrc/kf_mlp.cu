@@ -17,6 +17,8 @@
 
 namespace kf {
 
+constexpr uint32_t kTcWaitLimit = 1u << 24;  // mbarrier polls before a tcgen05 scoring wait gives up
+
 struct MlpState {
     float *m = nullptr, *v = nullptr;                   // [kMlpParams] each: Adam's moments
     float *partial = nullptr;                           // [2 per SM][kPartLd]: the training blocks' gradients
@@ -24,6 +26,7 @@ struct MlpState {
     float *w32 = nullptr;                               // loaded weights, FP32
     __nv_bfloat16 *W1 = nullptr, *W2 = nullptr;         // loaded weights, BF16, transposed and padded
     unsigned *status = nullptr;                         // set by a tcgen05 scoring wait that expired
+    uint32_t wait_limit = kTcWaitLimit;                 // polls of such a wait
     bool loaded = false;
 };
 
@@ -419,7 +422,7 @@ __global__ void __launch_bounds__(32 * kScoreWarps) mlp_score_kernel(const __nv_
 // product, read: the issue slots are half idle), so tiles in flight count: with
 // one set of columns and of operands per tile, and the weights shared by three
 // tiles, an SM holds six (before: four, each with its own weights and two
-// sets).  4,194,301 rows: 143 us, 158 with four (52 B a row would take 32 us at
+// sets).  4,194,301 rows: 137 us, 158 with four (52 B a row would take 32 us at
 // the copy bandwidth).  Shared memory is busy for some 60% of that, 66 KB of
 // operand reads and 40 KB of writes a tile.
 //
@@ -434,7 +437,6 @@ constexpr int kTcRows = 128, kTcGroups = 3;        // rows per tile; tiles of a 
 constexpr int kTcThreads = kTcRows * kTcGroups;
 constexpr int kTcCols = 256;                       // TMEM columns of a CTA (a power of two): 64 per tile
 constexpr int kTcCtasPerSm = 2;                    // 2 x 256 = the SM's 512 TMEM columns
-constexpr uint32_t kTcWaitLimit = 1u << 24;        // mbarrier polls before a wait gives up
 
 struct __align__(128) TcSmem {
     // per tile, the A operand's hi and lo parts: the first hidden layer (K =
@@ -494,12 +496,12 @@ __device__ __forceinline__ void tc_commit(unsigned long long *mbar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(a) : "memory");
 }
 
-// Wait for the mbarrier's phase `parity` to complete, polling at most
-// kTcWaitLimit times; false if it did not.
-__device__ __forceinline__ bool mbar_wait(unsigned long long *mbar, uint32_t parity)
+// Wait for the mbarrier's phase `parity` to complete, polling at most `limit`
+// times; false if it did not.
+__device__ __forceinline__ bool mbar_wait(unsigned long long *mbar, uint32_t parity, uint32_t limit)
 {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(mbar);
-    for (uint32_t i = 0; i < kTcWaitLimit; ++i) {
+    for (uint32_t i = 0; i < limit; ++i) {
         uint32_t done;
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -540,10 +542,15 @@ __device__ __forceinline__ void st_shared_v4(uint8_t *p, uint32_t a, uint32_t b,
 }
 
 // VEC: the rows start on 16-byte boundaries and are read as three float4.
+// A warp one of whose waits for a product expires (`limit` polls) touches
+// neither the operands, which the product may still read, nor the accumulator:
+// it votes at the group's next barrier (if there is one) to end the group, and
+// before the CTA gives its TMEM back it waits on that same phase, with
+// kTcWaitLimit polls, for what is in flight.
 template <bool VEC>
 __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) mlp_score_tc_kernel(const float *w32, const float *X,
                                                                                  int64_t n, float *logits,
-                                                                                 unsigned *status)
+                                                                                 unsigned *status, uint32_t limit)
 {
     extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
     TcSmem &s = *reinterpret_cast<TcSmem *>(tc_smem_raw);
@@ -641,7 +648,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) mlp_score_tc_kernel(
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         // the group's rows are written, and its reads of the last tile's columns done
-        if ((failed = group_or(group + 1, failed))) break;
+        if ((failed = group_or(group + 1, false))) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             tc_mma(d, smem_desc(Ah, 128, 256), smem_desc(s.B1, 128, 256), 0u);
@@ -649,8 +656,12 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) mlp_score_tc_kernel(
             tc_commit(mbar);
         }
         load_row(tile + step, fin);
-        failed = !mbar_wait(mbar, parity);
+        failed = __any_sync(0xffffffffu, !mbar_wait(mbar, parity, limit));
         parity ^= 1u;
+        if (failed) {
+            group_or(group + 1, true);
+            break;
+        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // layer 1 epilogue (the bias is in the accumulator): ReLU, split ->
         // layer-2 A operand (row tid), over the inputs, which are consumed
@@ -674,7 +685,7 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) mlp_score_tc_kernel(
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        if ((failed = group_or(group + 1, failed))) break;
+        if ((failed = group_or(group + 1, false))) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
@@ -686,8 +697,12 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) mlp_score_tc_kernel(
             tc_mma(d, smem_desc(s.ones, 128, 256), smem_desc(s.B2b, 128, 256), 1u);  // + b2
             tc_commit(mbar);
         }
-        failed = !mbar_wait(mbar, parity);
+        failed = __any_sync(0xffffffffu, !mbar_wait(mbar, parity, limit));
         parity ^= 1u;
+        if (failed) {
+            if (tile + step < tiles) group_or(group + 1, true);
+            break;
+        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // layer 2 epilogue (the bias is in the accumulator): ReLU, the 64 -> 1
         // dot product
@@ -710,10 +725,10 @@ __global__ void __launch_bounds__(kTcThreads, kTcCtasPerSm) mlp_score_tc_kernel(
         if (row < n) logits[row] = z;
     }
     if (failed) {
-        // a product did not complete in time: report it, and give whatever is
-        // still in flight a bounded while to land before TMEM is released
-        if (tid == 0) atomicOr(status, 1u);
-        mbar_wait(mbar, parity);
+        // a product did not complete in time: report it, and give it a bounded
+        // while to land before TMEM is released
+        if ((tid & 31) == 0) atomicOr(status, 1u);
+        mbar_wait(mbar, parity ^ 1u, kTcWaitLimit);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -919,7 +934,7 @@ int kf_proposal_score_with(kf_context *ctx, const float *features, int64_t n, fl
         const int64_t tiles = (n + kTcRows - 1) / kTcRows;
         const unsigned grid = (unsigned)std::min<int64_t>((tiles + kTcGroups - 1) / kTcGroups,
                                                           (int64_t)context_sm_count(ctx) * kTcCtasPerSm);
-        kern<<<grid, kTcThreads, sizeof(TcSmem), stream>>>(s->w32, features, n, logits, s->status);
+        kern<<<grid, kTcThreads, sizeof(TcSmem), stream>>>(s->w32, features, n, logits, s->status, s->wait_limit);
     } else {
         if ((e = cudaFuncSetAttribute(mlp_score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(ScoreSmem))) != cudaSuccess)
@@ -937,6 +952,15 @@ int kf_proposal_score_with(kf_context *ctx, const float *features, int64_t n, fl
 int kf_proposal_score(kf_context *ctx, const float *features, int64_t n, float *logits, kf_stream stream)
 {
     return kf_proposal_score_with(ctx, features, n, logits, KF_SCORE_AUTO, stream);
+}
+
+// For tests, not in kf.h: the polls after which a tcgen05 scoring wait of this
+// context gives up (0: at once).  Weights must have been loaded.
+int kf_test_score_wait_limit(kf_context *ctx, uint32_t polls)
+{
+    if (!ctx || !proposal_loaded(ctx)) return KF_ERR_ARG;
+    context_mlp_state(ctx)->wait_limit = polls;
+    return KF_OK;
 }
 
 int kf_proposal_status(kf_context *ctx, int *expired)

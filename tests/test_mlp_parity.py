@@ -10,6 +10,8 @@ its value, and accumulates in FP32, so a logit is within a few 2^-18 of the
 network's absolute-value magnitude |W3|^T (|W2|^T (|W1|^T |x| + |b1|) +
 |b2|) + |b3|; the bar is 2^-14 of it.
 """
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -158,3 +160,32 @@ def test_automatic_engine_line(kf, ctx, n, engine):
     kf.proposal_load(ctx, cu(w))
     x = cu(X)
     assert torch.equal(kf.proposal_score(ctx, x), kf.proposal_score(ctx, x, engine=engine))
+
+
+@pytest.mark.parametrize("n", [1, 128 * 3 + 5, 152 * 2 * 3 * 128 * 2 + 77])
+def test_expired_score_wait_is_reported(kf, n):
+    """A tcgen05 scoring wait that runs out at once (a limit of no polls: the
+    products themselves complete, and the CTA waits for them before it ends)
+    leaves every logit unwritten and sets the status; with one poll, which may or
+    may not see the product, a logit is right or unwritten, and an unwritten one
+    is reported; with the limit as it was, scoring works again."""
+    X, _, w = data(8, n)
+    c = kf.Context(0)
+    kf.proposal_load(c, cu(w))
+    x = cu(X)
+    want = kf.proposal_score(c, x, engine=2)
+    assert not kf.proposal_status(c)
+    limit = kf.load().kf_test_score_wait_limit
+    limit.argtypes, limit.restype = [ctypes.c_void_p, ctypes.c_uint32], ctypes.c_int
+    z = torch.full((n,), 7e30, device="cuda")
+    assert limit(c.handle, 1) == 0
+    kf.load().kf_proposal_score_with(c.handle, x.data_ptr(), n, z.data_ptr(), 2, torch.cuda.current_stream().cuda_stream)
+    left = z == 7e30
+    assert bool((left | (z == want)).all()) and (kf.proposal_status(c) or not bool(left.any()))
+    z.fill_(7e30)
+    assert limit(c.handle, 0) == 0
+    kf.load().kf_proposal_score_with(c.handle, x.data_ptr(), n, z.data_ptr(), 2, torch.cuda.current_stream().cuda_stream)
+    assert bool((z == 7e30).all()) and kf.proposal_status(c)
+    assert limit(c.handle, 1 << 24) == 0
+    assert torch.equal(kf.proposal_score(c, x, engine=2), want)
+    c.close()
