@@ -32,14 +32,15 @@ sys.path.insert(0, ROOT)
 
 METRIC = "fitted tracks/s and built seeds/s on 1 GB300 (chosen vs plain form), % of FP32 roofline"
 WORKLOAD = ("fit: 10-layer toy barrel r=4..40 cm, |z|<100 cm, Bz=3.8 T, x/X0=0.01; 100 events x 20,000 "
-            "tracks, pT U(0.5,10) GeV, |eta|<1, seeds smeared 10%; FP32 with FP64 routing, one launch "
-            "over all events")
+            "tracks, pT U(0.5,10) GeV, |eta|<1, seeds smeared 10%; FP32 with updates routed to extended "
+            "precision, one launch over all events")
 N_LAYERS = 10
-# FP32 flops of one track-layer with a hit, counted on the kernel's formulation
-# (add, multiply, reciprocal, square root, log = 1, FMA = 2): propagation 75,
-# Jacobian 88, J C J^T 308, scattering 42, local-frame update 255.  The routed
-# form also spends about 30 flops per update on its routing tests (not counted).
-FLOPS_PER_TRACK_LAYER = 768
+# FP32 flops the fit executes, counted by tests/test_track_math_host.py on the
+# kernels' own source (add, multiply, reciprocal, square root, log = 1, FMA = 2;
+# the routing tests included): a layer with a hit, and what a track's first
+# layer, from the seed, and its result take.
+FLOPS_PER_TRACK_LAYER = 465
+FLOPS_PER_TRACK_ENDS = 625
 # the proposal network per scored row: 2 (12 x 64 + 64 x 64 + 64) multiply-adds
 # (the split activations issue each layer-1 and layer-2 product twice; that
 # doubling is not counted)
@@ -389,7 +390,7 @@ def bench_build(args, kf, ctx, dev, stream, rank, world):
         "bound": "latency", "call_ms": ms_call, "fp32_tflops": flops / (ms_call * 1e-3) / 1e12,
         "fp32_frac": flops / (ms_call * 1e-3) / 1e12 / FP32_PEAK_TFLOPS,
         "fp32_flops_per_call": flops,
-        "fp32_flops_note": "seeds x build layers x N x 768: every candidate slot live at every layer (upper bound)",
+        "fp32_flops_note": f"seeds x build layers x N x {FLOPS_PER_TRACK_LAYER}: every candidate slot live at every layer (upper bound)",
         "dram_gbs": dram / (ms_call * 1e-3) / 1e9 if dram else None,
         "dram_frac": (dram / (ms_call * 1e-3) / 1e9 / hbm) if (dram and hbm) else None,
         "dram_bytes_per_call": dram,
@@ -858,7 +859,7 @@ def main():
     e2e_ms = max_over_ranks((time.perf_counter() - t_e) * 1e3 / n_e2e, world, dev)
 
     routed_share = float(((out["flags"] & 16) != 0).float().mean().item())
-    flops = FLOPS_PER_TRACK_LAYER * N_LAYERS * T
+    flops = (FLOPS_PER_TRACK_LAYER * (N_LAYERS - 1) + FLOPS_PER_TRACK_ENDS) * T
     achieved_tflops = flops / (kern_ms * 1e-3) / 1e12
     src_hash = kernel_source_hash()
     traffic = recorded_traffic(src_hash)
@@ -889,8 +890,11 @@ def main():
                 "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms,
                 "form": "kf_fit_tracks_host on pinned host buffers: the fit reads the inputs and "
                         "writes the outputs in host memory over the host link"},
-        "fp64_routed_share": routed_share,
-        "gpu_launches": 2 * args.steps,  # the batch's kernel and that of the tracks put off
+        "fp64_routed_share": routed_share,  # with an update in extended precision, float-float or FP64
+        # the batch's kernel and, in routed precision on more tracks than one launch
+        # serves, that of the tracks put off
+        "gpu_launches": args.steps * (2 if chosen.precision_mode == kf.PRECISION_ROUTED
+                                      and (T >= 32768 or args.shape) else 1),
         "clocks": clocks,
         "kernel_source_hash": src_hash,
         "wall_s_timed": t_wall,

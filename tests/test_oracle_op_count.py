@@ -1,7 +1,7 @@
 """The FP64 oracle's operation count per track-layer, measured by compiling
 its own source with a counting scalar type: the reference figure beside the
-fit's structured numerator (768 flops per track-layer, counted on the
-Cartesian formulation with the Jacobian's structural zeros)."""
+fit's own count (465 flops per track-layer in local coordinates) and that of a
+Cartesian formulation with the Jacobian's structural zeros (768)."""
 import shutil
 
 import pytest

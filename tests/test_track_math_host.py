@@ -176,3 +176,21 @@ def test_fit_reads_no_absent_hit(tmp_path_factory, oracle):
     assert ((read & ~mask) == 0).all()
     assert (read[~stopped] == mask[~stopped]).all() and (mask != (1 << L) - 1).any()
     assert np.linalg.norm(out[0] - ref["state"]) < 1e-4 * np.linalg.norm(ref["state"])
+
+
+def test_flop_count(tmp_path_factory):
+    """The flops per track-layer and per track by which bench.py rates the fit and
+    the build: counted on the kernels' source, the same for every track of the
+    fit workload."""
+    import bench
+    lib = _compile("track_flops", tmp_path_factory)
+    n, L = 100, 10
+    b = synth.make_fit_batch(1, [n])
+    g = b.geom
+    f32 = lambda a: np.ascontiguousarray(a, dtype=np.float32)
+    arrays = [f32(b.seed_state), f32(b.seed_cov), b.charge, f32(b.hit_pos), f32(b.hit_cov)]
+    count = np.zeros(3, np.uint64)
+    lib.host_count(L, _p(f32(g.radii)), _p(f32(g.x_over_x0)), ctypes.c_float(g.z_half),
+                   ctypes.c_float(0.00299792458 * g.bz), ctypes.c_int64(n), *[_p(a) for a in arrays], _p(count))
+    assert count[1] == n * (L - 1)
+    assert count[0] == bench.FLOPS_PER_TRACK_LAYER * count[1] and count[2] == bench.FLOPS_PER_TRACK_ENDS * n
