@@ -1,8 +1,10 @@
-"""Tracks put off to the second launch of a fit (those that need FP64) against
-the same tracks with the FP64 update in line (KF_LAUNCH_FLAT): the same
+"""Tracks put off to the second launch of a fit (those that need extended
+precision: pT outside the bounds, ill-conditioned updates, hits that fail the
+update) against the same tracks with it in line (KF_LAUNCH_FLAT): the same
 arithmetic in another launch, so every output is equal bit for bit.  Sizes on
 both sides of the one-launch limit (32,768 tracks), of the gathering blocks (256
-tracks) and with every, some, and no track put off; each batch runs twice."""
+tracks) and of what they gather in one pass (2 per SM), with every, some, and no
+track put off."""
 import numpy as np
 import pytest
 
@@ -35,6 +37,40 @@ def test_put_off_equals_in_line(kf, n):
                 got = kf.fit_tracks(ctx, geom, **dev, opt=opt)
                 for k in want:
                     assert np.array_equal(got[k].cpu().numpy(), want[k].cpu().numpy(), equal_nan=True), (lo, k)
+    ctx.close()
+
+
+@pytest.mark.parametrize("cond_max,share", [(1e4, (0.05, 0.3)), (10.0, (0.1, 0.5))])
+def test_put_off_with_holes_stops_and_bad_hits(kf, cond_max, share):
+    """More tracks than the gathering blocks take in one pass, sparsely put off, with
+    hits missing, tracks that leave the barrel, hits and seeds that are not
+    finite, and (cond_max 10) updates put off for their condition; every hit
+    prefetch depth.  No mark of a track put off is left in the flags."""
+    ctx, n = kf.Context(0), 160_001
+    b = synth.make_fit_batch(66, [n], pt_lo=0.24, pt_hi=500.0, pt_dist="loguniform", eta_max=2.5, hit_eff=0.85,
+                             sigma_rphi=0.001)
+    rng = np.random.default_rng(1)
+    bad = rng.choice(n, 300, replace=False)
+    for k, t in enumerate(bad):  # the first used hit of some, a seed's value of others
+        first = (int(b.hit_mask[t]) & -int(b.hit_mask[t])).bit_length() - 1
+        if k % 3 == 0 and first >= 0:
+            b.hit_pos[first, k % 2, t] = (np.nan, np.inf)[k % 2]
+        elif k % 3 == 1 and first >= 0:
+            b.hit_cov[first, (0, 2, 5)[k // 3 % 3], t] = (np.nan, np.inf, -1.0)[k // 9 % 3]
+        else:
+            b.seed_state[k % 6, t] = np.inf
+    dev, geom = kf.to_device(b), kf.GeometryArgs.of(b.geom)
+    want = kf.fit_tracks(ctx, geom, **dev, opt=kf.options(launch_mode=kf.LAUNCH_FLAT, cond_max=cond_max))
+    flags = want["flags"].cpu().numpy()
+    assert share[0] <= ((flags & 16) != 0).mean() <= share[1], ((flags & 16) != 0).mean()
+    assert ((flags & 8) != 0).sum() >= 100 and ((flags & 2) != 0).sum() > 1000
+    for shape in ({}, dict(tracks_per_block=32, reg_cap=96, hit_prefetch=2),
+                  dict(tracks_per_block=256, reg_cap=128, hit_prefetch=4),
+                  dict(tracks_per_block=64, reg_cap=80, hit_prefetch=1)):
+        got = kf.fit_tracks(ctx, geom, **dev, opt=kf.options(cond_max=cond_max, **shape))
+        assert (got["flags"] >= 0).all()  # bit 31 marks a track put off
+        for k in want:
+            assert np.array_equal(got[k].cpu().numpy(), want[k].cpu().numpy(), equal_nan=True), (shape, k)
     ctx.close()
 
 
