@@ -656,7 +656,7 @@ def bench_ragged(args, kf, ctx, dev, stream, rank):
     out = kf.fit_outputs(T, dev)
     res = {"workload": "17-layer toy barrel r=4..68 cm, 256 events, lognormal sizes (median 5,000, "
                        "500..50,000), hit efficiency 0.95", "tracks": T}
-    for name, mode in (("persistent", kf.LAUNCH_AUTO), ("flat", kf.LAUNCH_FLAT), ("per_event", kf.LAUNCH_PER_EVENT)):
+    for name, mode in (("tuned", kf.LAUNCH_AUTO), ("flat", kf.LAUNCH_FLAT), ("per_event", kf.LAUNCH_PER_EVENT)):
         opt = kf.options(launch_mode=mode)
 
         def step():
@@ -674,7 +674,7 @@ def bench_ragged(args, kf, ctx, dev, stream, rank):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / n
         res[name] = {"value": T / (ms * 1e-3), "unit": "tracks/s", "ms_per_step": ms,
-                     "launches_per_step": 1 if mode != kf.LAUNCH_PER_EVENT else len(b.event_offsets) - 1}
+                     "launches_per_step": {"tuned": 2, "flat": 1}.get(name, len(b.event_offsets) - 1)}
     shape = ctx.tuned_shape(b.geom.n_layers, T)
     res["tuned_shape"] = ({"tracks_per_block": shape[0], "reg_cap": shape[1], "hit_prefetch": shape[2]}
                           if shape else None)

@@ -256,7 +256,9 @@ int kf_fit_tracks_host(kf_context *ctx, const kf_geometry *geom, int64_t n_track
  * Scratch: 16 bytes per hit plus 4 (n_phi_bins n_z_bins + 1) bytes per
  * (event, layer) (16,384 bins when tuned), kept by the context and grown on
  * demand (KF_ERR_NOMEM).
- * The call copies hit_offsets to the device and waits for that copy.
+ * The call copies hit_offsets before it returns (through page-locked staging of
+ * the context, four calls deep) and does not wait for the GPU, but for tuning;
+ * it cannot be captured in a graph (KF_ERR_CUDA).
  */
 int kf_build_tracks(kf_context *ctx, const kf_geometry *geom, int n_events, const int64_t *hit_offsets,
                     const float *hit_pos, const float *hit_cov, int64_t n_hits, int64_t n_seeds,

@@ -200,11 +200,12 @@ __global__ void __launch_bounds__(256, 2) fit_plain_kernel(const FitGeom g, cons
 // kPutOff and *work to the fit's tag, and fit_extended_kernel, launched behind,
 // fits these tracks from their seeds in full warps (no tag: it returns at
 // once; the tag of a fit replayed from a graph may stand from an earlier
-// replay, and the kernel then finds no marked track).  With one track in eight above pt_hi (1,000,000 tracks, pT
-// log-uniform 0.24 to 500 GeV) nearly every warp held one and stopped for it
-// at every layer: 7.09 ms in line in FP64, 1.03 ms put off in FP64, 0.31 ms
-// in float-float.  Without that code this kernel also needs fewer registers
-// (96 with the ring, no spills).
+// replay, and the kernel then finds no marked track).  With one track in eight
+// outside the pT bounds (1,000,000 tracks, pT log-uniform 0.24 to 500 GeV)
+// nearly every warp holds one and stops for it at every layer: 7.09 ms in line
+// in FP64, 1.03 ms put off in FP64, 0.31 ms put off in float-float (0.70 in
+// line).  Without that code this kernel also needs fewer registers (80 to 96,
+// no spills).
 template <int BLOCK, int MINB, int DEPTH>
 __global__ void __launch_bounds__(BLOCK, MINB) fit_kernel(const FitGeom g, const Routing rt, const FitIO io,
                                                            unsigned *work, unsigned tag)

@@ -13,12 +13,12 @@
 // multiplies the scattering noise, so the FP32 rounding that Cp's correlations
 // amplify enters A scaled by |Q| / |Cp|.  K has the three momentum rows only,
 // and G^-1 has the form of G itself (a step back along the helix), so that
-// the covariance goes through the transport of the forward pass.  The forward pass writes the filtered coordinates, their covariance
-// and frames (25 floats) of every layer to the output arrays; the backward
-// pass reads them, repeats the step to layer l+1 (xp, G and Q come out the
-// same, bit for bit) and overwrites them with the smoothed estimate.  Nothing
-// else is stored: they are read back while still in L2, and each output line
-// reaches DRAM once, smoothed.
+// the covariance goes through the transport of the forward pass.  The forward
+// pass writes the filtered coordinates, their covariance and frames (25 floats)
+// of every layer to the output arrays; the backward pass reads them, repeats the
+// step to layer l+1 (xp, G and Q come out the same, bit for bit) and overwrites
+// them with the smoothed estimate.  Nothing else is stored: they are read back
+// while still in L2, and each output line reaches DRAM once, smoothed.
 #include "kf.h"
 #include "kf_api_internal.h"
 #include "kf_fit.cuh"
@@ -44,7 +44,7 @@ struct SmoothIO {
 
 // Registers capped at 128 (four blocks, 16 warps per SM).  Bound by FP32 issue:
 // 1,530 warp instructions per 32 track-layers, 65% of the issue slots (500,000
-// tracks of 10 layers: 0.355 ms on the 6x6 covariance, 0.29 ms now; 1.56 KB
+// tracks of 10 layers: 0.355 ms on the 6x6 covariance, 0.297 ms now; 1.56 KB
 // per track at the copy bandwidth would take 0.115 ms).
 __global__ void __launch_bounds__(128, 4) smooth_kernel(const FitGeom g, const Routing rt, const SmoothIO io)
 {

@@ -93,7 +93,7 @@ def test_float_float_gain_routing(kf, ctx, oracle):
 @pytest.mark.parametrize("block", [32, 64, 128, 256])
 def test_ragged_events_missing_hits(kf, ctx, oracle, block):
     """17 layers, 95% hit efficiency, uneven events with a ragged tail
-    (several persistent units and a partial one)."""
+    (several blocks of each size and a partial one)."""
     b = synth.make_fit_batch(31, [517, 1, 2049, 33, 700], geom=synth.toy_geometry(17), hit_eff=0.95)
     ref = oracle.fit_batch(b)
     for launch in (0, 1):

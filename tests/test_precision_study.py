@@ -4,7 +4,8 @@
 fitted sigma (median, 99th percentile, maximum; the position taken along
 the layer's tangent, since the radial one is fixed by the cylinder and has
 no sigma) for the FP32-only form and
-the routed form (ill-conditioned updates redone in FP64), the share of
+the routed form (ill-conditioned updates redone in FP64, those of extreme pT
+in float-float), the share of
 tracks routed, and the pull widths against the simulated truth for the
 oracle and both forms.  With KF_REPORT_DIR set the numbers are written there
 as precision_study.json.

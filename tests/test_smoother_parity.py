@@ -88,7 +88,8 @@ def test_smoother_fp32_only(kf, ctx, oracle):
 
 def test_smoother_stops(kf, ctx, oracle):
     """Loopers and tracks leaving the barrel stop early (routed precision: the
-    loopers below 0.25 GeV update in FP64, as the fit's parity bar needs)."""
+    loopers below 0.25 GeV update in extended precision, as the fit's parity bar
+    needs)."""
     b = synth.make_fit_batch(40, [1500], pt_lo=0.2, pt_hi=2.0, eta_max=2.0)
     g, ref, _ = _compare(kf, ctx, oracle, b)
     assert (ref["reached"] < b.geom.n_layers).any()
