@@ -221,11 +221,11 @@ int size_class(int64_t n)
 // Routed fits of fewer tracks than this run in one launch, blocks of 64 tracks
 // with the updates in extended precision in line, and are not tuned: the launch
 // for the tracks put off costs the host 2 to 3 us a call, and few warps share
-// an SM, so that one waiting for its own such update holds up little.  At
-// 10 layers the kernels take 8.9 and 8.8 us for 10,000 tracks (in line, put
-// off), 10.6 and 11.0 for 20,000, 13.0 and 13.2 for 40,000; with one track in
-// eight in extended precision 26 and 33, 30 and 37, 40 and 39.  A power of two,
-// as the tuner's size classes.
+// an SM, so that one waiting for its own such update holds up little.  At 10
+// layers the kernels take 13.8 us in line and 15.4 put off for 20,000 tracks,
+// 15.3 and 17.0 for 40,000, 26.8 and 22.9 for 80,000 (with caches cold); with one
+// track in eight in extended precision 37 and 43, 46 and 49, 83 and 58.  A power
+// of two, as the tuner's size classes.
 constexpr int64_t kOneLaunchTracks = 32768;
 
 // Fits that are tuned apart: 0 FP32, 1 routed, 2 routed with gain_max, whose

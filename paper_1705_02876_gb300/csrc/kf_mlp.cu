@@ -372,9 +372,9 @@ __global__ void to_bf16_kernel(float *w32, __nv_bfloat16 *W1t, __nv_bfloat16 *W2
 
 constexpr int kScoreWarps = 4, kScoreLd = 12;
 // kf_proposal_score's engine (KF_SCORE_AUTO), chosen by measurement on one
-// GB300: mma.sync below this many rows (65,536 rows 9.3 against 11.2 us), tcgen05
-// from it on (131,072 rows 12.9 against 13.3 us, 163,840 12.9 and 16.6, 262,144
-// 17.4 and 24.0, 2^24 537 and 1,146)
+// GB300: mma.sync below this many rows (65,536 rows 9.3 against 10.6 us; the two
+// meet near 80,000), tcgen05 from it on (131,072 rows 12.1 against 13.3 us,
+// 163,840 12.3 and 16.4, 262,144 16.5 and 24.2, 2^24 512 and 1,145)
 constexpr int64_t kScoreTcMinRows = 131072;
 
 struct ScoreSmem {
@@ -423,8 +423,8 @@ __global__ void __launch_bounds__(32 * kScoreWarps) mlp_score_kernel(const __nv_
 // one set of columns and of operands per tile, and the weights shared by three
 // tiles, an SM holds six (before: four, each with its own weights and two
 // sets).  4,194,301 rows: 137 us, 158 with four (52 B a row would take 32 us at
-// the copy bandwidth).  Shared memory is busy for some 60% of that, 66 KB of
-// operand reads and 40 KB of writes a tile.
+// the copy bandwidth).  Of that time the tensor pipe works 29%, the load-store
+// data pipe 55%, the ALU pipe (the splits) 54%, and 59% of the issue slots are used.
 //
 // Operands are K-major without swizzle, in core matrices of 8 rows x 16 bytes
 // (8 BF16 values): element (r, k) of a tile with K columns is at byte
