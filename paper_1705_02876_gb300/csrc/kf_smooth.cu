@@ -43,7 +43,7 @@ struct SmoothIO {
 };
 
 // Registers capped at 128 (four blocks, 16 warps per SM).  Bound by FP32 issue:
-// 1,530 warp instructions per 32 track-layers, 65% of the issue slots (500,000
+// 1,474 warp instructions per 32 track-layers, 62% of the issue slots (500,000
 // tracks of 10 layers: 0.355 ms on the 6x6 covariance, 0.297 ms now; 1.56 KB
 // per track at the copy bandwidth would take 0.115 ms).
 __global__ void __launch_bounds__(128, 4) smooth_kernel(const FitGeom g, const Routing rt, const SmoothIO io)
