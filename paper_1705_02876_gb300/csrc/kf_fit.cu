@@ -19,6 +19,9 @@ __device__ __forceinline__ void cp_async4(float *dst, const float *src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+#ifdef __CUDACC__
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+#endif
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
@@ -34,6 +37,10 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // so that the loads in flight hold no registers.  A non-finite value in a
 // used hit makes the chi2 increment non-finite, or makes S fail its positive
 // definiteness test, so the hit is tested only then.
+// Without DEFER (the plain kernel's small batches and single events, and the
+// tracks put off, which lie apart: few warps wait for DRAM with nothing to do)
+// the next layer's hit goes to L2 a layer ahead.  Events of 5,000 tracks, one
+// launch each, not in L2: 12.7 us, 14.8 without; of 20,000 14.8 and 15.9.
 // DEFER: a track outside the pT bounds on the first layer, and any other at the
 // first update that needs extended precision, is given up and true returned
 // (nothing is written).
@@ -103,6 +110,12 @@ __device__ __forceinline__ bool fit_track(const FitGeom &g, const Routing &rt, c
             const bool has = (mask >> l) & 1u;
             if constexpr (DEPTH == 1) {
                 if (l > 0) load_hit(has);
+                if (!DEFER && l + 1 < g.L && ((mask >> (l + 1)) & 1u)) {
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) prefetch_l2(hp + i * T + off);
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) prefetch_l2(hc + i * T + off);
+                }
             } else {
                 issue();                 // layer l + DEPTH
                 cp_async_wait<DEPTH>();  // layer l's group has landed
@@ -180,7 +193,7 @@ namespace {
 
 // One thread per track over [t_begin, t_end), the updates in extended precision
 // in line.  Two blocks of 256 threads per SM: at 128 registers (162 uncapped)
-// 1,000,000 tracks take 212 us, 255 uncapped.
+// 1,000,000 tracks take 205 us (212 without the prefetch, 255 uncapped).
 __global__ void __launch_bounds__(256, 2) fit_plain_kernel(const FitGeom g, const Routing rt, const FitIO io,
                                                          int64_t t_begin, int64_t t_end)
 {
@@ -354,7 +367,7 @@ cudaError_t launch_fit_tuned(const FitGeom &g, const Routing &rt, const FitIO &i
     // A float-float gain takes three times an FP32 update and may be asked of
     // any share of the tracks, which a fit from the seed anew pays for only if
     // they are few.  1,000,000 tracks with gain_max 1, 100 and 10,000 (all, 76%
-    // and none of them): 655, 258 and 213 us in line, 712, 401 and 178 put off.
+    // and none of them): 657, 250 and 205 us in line, 712, 401 and 178 put off.
     if (rt.mode == 1 && rt.gain_max > 0.0f) return launch_fit_plain(g, rt, io, 0, io.T, block, stream);
     const int64_t grid = (io.T + block - 1) / block;
     if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;

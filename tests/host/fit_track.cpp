@@ -1,5 +1,6 @@
 // The fit of one track (fit_track of csrc/kf_fit.cu, hits loaded at their layer)
-// compiled for the host, recording which hits it reads.
+// compiled for the host, recording which hits it reads
+// or fetches ahead.
 #include "cuda_shim.h"
 
 #define __CUDA_RUNTIME_H__  // the CUDA runtime's header is not needed
@@ -24,6 +25,7 @@ static T __ldcs(const T *p)
     record(p);
     return *p;
 }
+static void prefetch_l2(const float *p) { record(p); }
 template <class T>
 static void __stcs(T *p, T v)
 {
